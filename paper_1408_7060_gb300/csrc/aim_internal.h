@@ -235,13 +235,22 @@ struct aim_ctx {
   int* d_order = nullptr;      // [ns] RWGs in Morton order of their anchors (interpolation visit order)
   double* d_lam = nullptr;     // [ns][4][64]  FP64 anterpolation rows
   float* d_lamf = nullptr;     // [ns][4][64]  FP32 copy (C64 path)
-  int* d_nptr = nullptr;       // [N^3 + 1]    node-major CSR of the transpose
+  // node-major CSR of the transpose over the nodes some stencil touches, in (z, y, x) order
+  int* d_arow = nullptr;       // [NZ * box rows + 1] first node of each box row (z, y)
+  int* d_anode = nullptr;      // [n_active] y N + x
+  int* d_aptr = nullptr;       // [n_active + 1] first entry of each node
   int* d_nidx = nullptr;       // [64 ns]
   double4_32a* d_ncoef = nullptr;  // [64 ns]  (x, y, z, div) coefficients
   float4* d_ncoeff = nullptr;  // [64 ns]  FP32 copy
 
   double2* d_kspec = nullptr;  // [(N_g+1)][2][LZ/2+1][N+1][N+1] kernel spectra octant (FP64)
   float2* d_kspecf = nullptr;  // FP32 copy
+  // plane kernel: kernel spectra in its order, [m][plane_spec_elems] (plane.cuh); the FP64
+  // table of a complex64 context holds m = 0 only (the refinement residual)
+  float2* d_planef = nullptr;
+  double2* d_plane = nullptr;
+  bool plane = false;          // complex64 grids are kx-major and run the plane kernel
+  bool plane64 = false;        // complex128 grids do
   double2* d_tw = nullptr;     // [L] twiddles W_L^t (FP64)
   float2* d_twf = nullptr;     // [L] FP32
   double2* d_twz = nullptr;    // [LZ] twiddles W_LZ^t of the z transform (FP64)
@@ -277,15 +286,15 @@ struct aim_ctx {
   double2* d_nearT = nullptr;  // [(N_g+1)][nnz] values of the transposed near matrices (lazy)
 
   // ---- work buffers (sized for batch_max) ----
-  void* d_A = nullptr;         // [B][4][NZ][N][L]  after the x pass
-  void* d_Bf = nullptr;        // [B][4][NZ][L][L]  after the y pass (the slab)
+  void* d_A = nullptr;         // [B][4][NZ][N][L]  after the x pass; kx-major contexts: [B][4][L][NZ][N]
+  void* d_Bf = nullptr;        // [B][4][NZ][L][L]  after the y pass (the slab); unused when kx-major
   void* d_P = nullptr;         // [B][4][NZ][N][N]  potentials on the grid
   void* d_ring = nullptr;      // [N_g][B][4][Z][L][L] history slabs: z-spectra (Z = LZ, power-of-two
-                               // LZ) or x/y-transformed grids (Z = NZ)
+                               // LZ, and plane-kernel contexts, in its order) or x/y-transformed grids (Z = NZ)
   CUtensorMap ring_map;        // TMA view of the ring [slot][B*4*LZ][L][L] (complex64, power-of-two LZ)
   bool ring_tma = false;
   int* d_err = nullptr;        // device error flag (a bounded wait gave up)
-  void* d_xs = nullptr;        // [B][ns] prepared operator input, grid precision
+  void* d_xs = nullptr;        // [ns][nb] prepared operator input, grid precision (nb of the call)
   double2* d_xd = nullptr;     // [B][ns] prepared operator input, FP64 (near zone)
   DotFuse dotfuse;             // set by the Arnoldi step around its operator application
   float2* d_vf = nullptr;      // [B][ns] complex64 copy of the Krylov vector the next SAI application

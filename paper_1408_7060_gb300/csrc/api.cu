@@ -249,7 +249,7 @@ void setup_impl(aim_ctx* c, const aim_mesh* mesh, const aim_grid* grid, double n
     sl.m[0] = 1;
     sl.n = 1;
     NearList nl{};
-    op_apply_rhs(c, 1, sl, nl, nullptr, 1.0, c->d_y);
+    op_apply_rhs(c, 1, sl, c->d_ring, nl, nullptr, 1.0, c->d_y);
   }
   AIM_CUDA(cudaStreamSynchronize(c->stream));
   c->prof = ProfState();
@@ -259,10 +259,18 @@ void setup_impl(aim_ctx* c, const aim_mesh* mesh, const aim_grid* grid, double n
 // buffer; it is allocated on the first call that needs it
 void ensure_ring(aim_ctx* c) {
   if (c->d_ring) return;
-  const size_t slab = op_slab_bytes(c, c->batch_max);
   // blocked sums: 2^P >= N_g source slots and 2^(P+1) pending slots
   const int nslots = c->rhs_blocked ? 1 << c->blk_P : c->n_delays;
-  c->d_ring = aim_alloc(c, (size_t)nslots * slab);
+  size_t slab = op_slab_bytes(c, c->batch_max);
+  try {
+    c->d_ring = aim_alloc(c, (size_t)nslots * slab);
+  } catch (const AimError&) {
+    // a factor-3 z length: the ring of x/y-transformed slabs is the smaller one
+    if (!op_plane(c) || (c->LZ & (c->LZ - 1)) == 0) throw;
+    (c->precision == AIM_C64 ? c->plane : c->plane64) = false;
+    slab = op_slab_bytes(c, c->batch_max);
+    c->d_ring = aim_alloc(c, (size_t)nslots * slab);
+  }
   if (c->rhs_blocked) {
     c->d_pend = aim_alloc(c, ((size_t)2 << c->blk_P) * slab);
     AIM_CUDA(cudaMemsetAsync(c->d_pend, 0, ((size_t)2 << c->blk_P) * slab, c->stream));
@@ -270,7 +278,7 @@ void ensure_ring(aim_ctx* c) {
   // TMA view for the complex64 delayed sum over the z-spectra: [slot][B*4*LZ][L][L],
   // boxes of 16 x 1 x LZ x 1
   const int L = c->L, LZ = c->LZ;
-  if (c->precision == AIM_C64 && (LZ & (LZ - 1)) == 0 && LZ <= 256 && L <= 256) {
+  if (c->precision == AIM_C64 && !c->plane && (LZ & (LZ - 1)) == 0 && LZ <= 256 && L <= 256) {
     const cuuint64_t dims[4] = {(cuuint64_t)L, (cuuint64_t)L, (cuuint64_t)c->batch_max * 4 * LZ,
                                 (cuuint64_t)c->n_delays};
     const cuuint64_t strides[3] = {(cuuint64_t)L * 8, (cuuint64_t)L * L * 8, (cuuint64_t)slab};
@@ -550,7 +558,7 @@ int aim_rhs(aim_ctx* c, int32_t l, int32_t nb, const aim_c128* hist, aim_c128* r
     }
     const bool ydev = is_device_ptr(rhs);
     double2* ys = ydev ? reinterpret_cast<double2*>(rhs) : c->d_y;
-    op_apply_rhs(c, nb, sl, nl, nullptr, 1.0, ys);
+    op_apply_rhs(c, nb, sl, (char*)c->d_ring + (size_t)(ng - 1) * slab, nl, nullptr, 1.0, ys);
     if (!ydev) AIM_CUDA(cudaMemcpyAsync(rhs, ys, n * sizeof(double2), cudaMemcpyDeviceToHost, c->stream));
     int h_err = 0;
     AIM_CUDA(cudaMemcpyAsync(&h_err, c->d_err, sizeof(int), cudaMemcpyDeviceToHost, c->stream));
@@ -1078,7 +1086,8 @@ static int march_steps(aim_ctx* c, const StepIO& io, int n_steps, double tol, ai
     if (c->rhs_blocked && l > 1)  // the grid part was gathered by the squares of earlier steps
       op_apply_rhs_pending(c, nb, (char*)c->d_pend + (size_t)(l % (2 * nsrc)) * slab, nl, c->d_b, -1.0, c->d_b);
     else
-      op_apply_rhs(c, nb, sl, nl, c->d_b, -1.0, c->d_b);  // b = V_l - sum_m Z_m I_{l-m}
+      // b = V_l - sum_m Z_m I_{l-m}; the slot that I_l's slab will take is free for the sum
+      op_apply_rhs(c, nb, sl, (char*)c->d_ring + (size_t)(l % nsrc) * slab, nl, c->d_b, -1.0, c->d_b);
     AIM_CUDA(cudaEventRecord(ev[1], st));
     if (c->zero_start) AIM_CUDA(cudaMemsetAsync(c->d_x, 0, n * sizeof(double2), st));
     const bool refining = c->refine > 0 && l % c->refine_every == 0;

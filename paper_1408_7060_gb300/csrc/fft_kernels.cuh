@@ -16,6 +16,20 @@ __device__ __forceinline__ void load_twiddles(C* tw, const C* __restrict__ twg, 
   for (int i = threadIdx.x; i < L; i += blockDim.x) tw[i] = twg[i];
 }
 
+__device__ __forceinline__ int fold(int k, int N) { return k <= N ? k : 2 * N - k; }
+
+// Grid order of the z-pass blocks: (right-hand side, component) fastest, then the x
+// tile, then the row y taken in mirror pairs (0, N, 1, L-1, 2, L-2, ...).  Every block
+// reads the kernel-spectrum octant at (fold(kz), fold(y), fold(x)); the octant of a large
+// grid does not fit in L2, and this order keeps the blocks that read the same entries
+// (all right-hand sides and components of one kernel kind, the rows y and L-y) close in
+// time, so the octant comes from DRAM about once per launch.
+__device__ __forceinline__ int zpass_row(int j, int N) {
+  if (j < 2) return j * N;
+  const int k = ((j - 2) >> 1) + 1;
+  return (j & 1) ? 2 * N - k : k;
+}
+
 // Transform the lines of a tile (after a __syncthreads that publishes a); returns
 // the buffer holding the natural-order result.  Lengths with a two-step plan use the
 // two-step transform, any other the Stockham passes.

@@ -17,7 +17,7 @@ void body_apply(aim_ctx*, int, int, const double2*, const double2*, const double
 template <class C>
 void body_forward_slab(aim_ctx*, int, const double2*, void*);
 template <class C>
-void body_apply_rhs(aim_ctx*, int, const SlabList&, const NearList&, const double2*, double, double2*);
+void body_apply_rhs(aim_ctx*, int, const SlabList&, void*, const NearList&, const double2*, double, double2*);
 template <class C>
 void body_apply_rhs_pending(aim_ctx*, int, void*, const NearList&, const double2*, double, double2*);
 template <class C>
@@ -26,6 +26,8 @@ template <class C>
 void body_tune(aim_ctx*);
 template <class C>
 void body_plan_fill(aim_ctx*);
+template <class C>
+bool plane_tables(aim_ctx*, int, const C*, C**);
 
 void op_apply(aim_ctx* c, int m, int nb, const double2* v, const double2* dinv, const double2* base, double sign,
               const int* active, double2* y, VecSel vin, VecSel yout) {
@@ -73,12 +75,12 @@ void op_forward_slab(aim_ctx* c, int nb, const double2* v, void* dst) {
     body_forward_slab<double2>(c, nb, v, dst);
 }
 
-void op_apply_rhs(aim_ctx* c, int nb, const SlabList& sl, const NearList& nl, const double2* base, double sign,
-                  double2* y) {
+void op_apply_rhs(aim_ctx* c, int nb, const SlabList& sl, void* scratch, const NearList& nl, const double2* base,
+                  double sign, double2* y) {
   if (c->precision == AIM_C64)
-    body_apply_rhs<float2>(c, nb, sl, nl, base, sign, y);
+    body_apply_rhs<float2>(c, nb, sl, scratch, nl, base, sign, y);
   else
-    body_apply_rhs<double2>(c, nb, sl, nl, base, sign, y);
+    body_apply_rhs<double2>(c, nb, sl, scratch, nl, base, sign, y);
 }
 
 void op_apply_rhs_pending(aim_ctx* c, int nb, void* P, const NearList& nl, const double2* base, double sign,
@@ -179,16 +181,40 @@ void op_autotune(aim_ctx* c, int mode) {
 }
 
 // kernels one operator application launches: prep, anterp + x, y, z, y^-1, x^-1, interp
-int op_kernel_count(const aim_ctx*) { return 7; }
+// (y, z and y^-1 are one kernel on a kx-major grid)
+int op_kernel_count(const aim_ctx* c) { return op_plane(c) ? 5 : 7; }
+
+bool op_plane(const aim_ctx* c) { return c->precision == AIM_C64 ? c->plane : c->plane64; }
+
+// A plane kept in shared memory saves the padded slab's four trips through memory, so every
+// size that fits uses it.  Its history ring holds z-spectra; for a z length with a factor 3
+// that is LZ / NZ times the bytes of the x/y-transformed ring, so there it also has to leave
+// three quarters of the free memory to everything else.
+void plane_setup(aim_ctx* c) {
+  const int nm = c->n_delays + 1;
+  const bool c64 = c->precision == AIM_C64;
+  if ((c->LZ & (c->LZ - 1)) != 0) {
+    size_t free = 0, total = 0;
+    AIM_CUDA(cudaMemGetInfo(&free, &total));
+    const size_t ring = (size_t)c->n_delays * c->batch_max * 4 * c->L * c->L * c->LZ * (c64 ? 8 : 16);
+    if (ring > free / 4) return;
+  }
+  if (c64) {
+    c->plane = plane_tables<float2>(c, nm, c->d_kspecf, &c->d_planef);
+    if (c->refine > 0) c->plane64 = plane_tables<double2>(c, 1, c->d_kspec, &c->d_plane);
+  } else {
+    c->plane64 = plane_tables<double2>(c, nm, c->d_kspec, &c->d_plane);
+  }
+}
 
 size_t grid_a_elems(const aim_ctx* c, int nb) { return (size_t)nb * 4 * c->NZ * c->N * c->L; }
 size_t grid_bf_elems(const aim_ctx* c, int nb) { return (size_t)nb * 4 * c->NZ * c->L * c->L; }
 size_t grid_p_elems(const aim_ctx* c, int nb) { return (size_t)nb * 4 * c->NZ * c->N * c->N; }
 
-// bytes of one history slab: [nb][4][Z][L][L] with Z = LZ (z-transformed, power-of-two
-// LZ) or NZ (x/y-transformed only)
+// bytes of one history slab: nb * 4 * L * L * Z elements with Z = LZ (z-transformed:
+// power-of-two LZ and plane-kernel contexts) or NZ (x/y-transformed only)
 size_t op_slab_bytes(const aim_ctx* c, int nb) {
-  const int L = c->L, Z = (c->LZ & (c->LZ - 1)) == 0 ? c->LZ : c->NZ;
+  const int L = c->L, Z = (c->LZ & (c->LZ - 1)) == 0 || op_plane(c) ? c->LZ : c->NZ;
   return (size_t)nb * 4 * Z * (size_t)L * L * (c->precision == AIM_C64 ? sizeof(float2) : sizeof(double2));
 }
 

@@ -57,9 +57,11 @@ void op_apply(aim_ctx* c, int m, int nb, const double2* v, const double2* dinv, 
 void op_apply_f64(aim_ctx* c, int m, int nb, const double2* v, const double2* base, double sign, double2* y);
 // slab of one current vector (anterpolation + forward x and y passes) written to dst
 void op_forward_slab(aim_ctx* c, int nb, const double2* v, void* dst);
-// y = base + sign * [ sum_s Z~FFT_{m_s} (slab_s) + near terms ]
-void op_apply_rhs(aim_ctx* c, int nb, const SlabList& sl, const NearList& nl, const double2* base, double sign,
-                  double2* y);
+// y = base + sign * [ sum_s Z~FFT_{m_s} (slab_s) + near terms ]; scratch: a ring slot whose
+// contents are not needed afterwards (it may be one of the slabs), for the delay sum of
+// plane-kernel contexts
+void op_apply_rhs(aim_ctx* c, int nb, const SlabList& sl, void* scratch, const NearList& nl, const double2* base,
+                  double sign, double2* y);
 // blocked right-hand side: y = base + sign * [ grid part from the pending z-spectra P
 // (which are read and cleared) + near terms ]
 void op_apply_rhs_pending(aim_ctx* c, int nb, void* P, const NearList& nl, const double2* base, double sign,
@@ -68,6 +70,16 @@ void op_block_square(aim_ctx* c, int nb, const BlockSquare& sq);
 // V_l for the plane waves in exc (device parameter block [nb][6]: khat, phat)
 void op_excitation(aim_ctx* c, int nb, const double* d_kp, double sigma, double t_d, int step_l, double2* out);
 int op_kernel_count(const aim_ctx* c);
+// the context's own operator runs the plane kernel on kx-major grids
+bool op_plane(const aim_ctx* c);
+// decide that, and tabulate the plane kernel's spectra (after the octants)
+void plane_setup(aim_ctx* c);
+// one launch of the plane kernel (mode: PLANE_* of plane.cuh) on d_A
+template <class C>
+void plane_launch(aim_ctx* c, int nb, int mode, int m, const int* active, C* S);
+// d_A = inverse of the delay sum over the z-spectra sl (S: scratch for one spectrum)
+template <class C>
+void plane_rhs(aim_ctx* c, int nb, const SlabList& sl, C* S);
 // choose the launch shapes of the grid passes (aim_opts.autotune: 1 tune or reuse the
 // cached plan, 2 tune and refresh the cache); leaves the defaults on mode 0
 void op_autotune(aim_ctx* c, int mode);

@@ -33,12 +33,12 @@ void body_apply(aim_ctx* c, int m, int nb, const double2* v, const double2* dinv
   });
 }
 
-// a history slab: x/y-transformed (factor-3 z lengths) or, for power-of-two z lengths,
-// also z-transformed (through Bf, which must not be dst)
+// a history slab: z-transformed (power-of-two z lengths and every plane-kernel context;
+// through A or Bf, which must not be dst) or x/y-transformed (other factor-3 z lengths)
 template <class C>
 void body_forward_slab(aim_ctx* c, int nb, const double2* v, void* dst) {
   AIM_DISPATCH_L(c->L, {
-    if (pow2_len(c->LZ)) {
+    if (pow2_len(c->LZ) || GridOps<LL, C>::kxm(c)) {
       GridOps<LL, C>::forward_slab(c, nb, v, nullptr, nullptr, reinterpret_cast<C*>(c->d_Bf));
       GridOps<LL, C>::zfwd(c, nb, reinterpret_cast<C*>(dst));
     } else {
@@ -48,11 +48,11 @@ void body_forward_slab(aim_ctx* c, int nb, const double2* v, void* dst) {
 }
 
 template <class C>
-void body_apply_rhs(aim_ctx* c, int nb, const SlabList& sl, const NearList& nl, const double2* base, double sign,
-                    double2* y) {
+void body_apply_rhs(aim_ctx* c, int nb, const SlabList& sl, void* scratch, const NearList& nl, const double2* base,
+                    double sign, double2* y) {
   AIM_DISPATCH_L(c->L, {
     if (sl.n > 0) {
-      GridOps<LL, C>::zrhs(c, nb, sl);
+      GridOps<LL, C>::zrhs(c, nb, sl, reinterpret_cast<C*>(scratch));
       GridOps<LL, C>::backward(c, nb, nl, base, sign, nullptr, y);
     } else {
       GridOps<LL, C>::interp(c, nb, nullptr, nl, base, sign, nullptr, y);
@@ -96,8 +96,8 @@ void body_plan_fill(aim_ctx* c) {
   template void body_apply<C>(aim_ctx*, int, int, const double2*, const double2*, const double2*, double,       \
                               const int*, double2*, VecSel, VecSel);                                             \
   template void body_forward_slab<C>(aim_ctx*, int, const double2*, void*);                                     \
-  template void body_apply_rhs<C>(aim_ctx*, int, const SlabList&, const NearList&, const double2*, double,      \
-                                  double2*);                                                                   \
+  template void body_apply_rhs<C>(aim_ctx*, int, const SlabList&, void*, const NearList&, const double2*,       \
+                                  double, double2*);                                                           \
   template void body_apply_rhs_pending<C>(aim_ctx*, int, void*, const NearList&, const double2*, double,        \
                                           double2*);                                                           \
   template void body_block_square<C>(aim_ctx*, int, const BlockSquare&);

@@ -19,6 +19,7 @@
 #include "aim_internal.h"
 #include "fft_kernels.cuh"
 #include "operator.h"
+#include "plane.cuh"
 #include "tma.cuh"
 
 template <class C> struct Real;
@@ -30,67 +31,76 @@ template <> __device__ __forceinline__ float2 cvt<float2>(double2 a) { return ma
 template <> __device__ __forceinline__ double2 cvt<double2>(double2 a) { return a; }
 
 // ---------------------------------------------------------------- stage i + x pass
-// S_c[n] = sum_k L_c[n,k] x_k gathered node by node (the transpose of the
-// interpolation rows), then the forward x-FFT of each grid row.  One block holds
-// the 4 components of ypb consecutive rows (z, y); grid (nb, rows / ypb, nz) with the
-// right-hand side fastest, so the CSR rows a block gathers serve the other right-hand
-// sides from L2.
-template <int L, class C>
-__global__ void __launch_bounds__(256) k_anterp_rows(const int* __restrict__ nptr, const int* __restrict__ nidx,
-                                                     const typename Real<C>::F4* __restrict__ ncoef,
-                                                     const C* __restrict__ xs, const int* __restrict__ active,
-                                                     int ns, int N, int ypb, C* __restrict__ A,
-                                                     const C* __restrict__ twg, int ylo, int yhi, int zlo, int nz) {
-  pdl_wait();
+// radix split of the x passes
+__host__ __device__ constexpr int x_r1(int L) { return L == 768 ? 32 : pl_r1(L); }
+__host__ __device__ constexpr int x_r2(int L) { return L / x_r1(L); }
+// elements between the rows of an x tile: R1 blocks of R2 + 1; kx-major stores take YB rows
+// in consecutive lanes, so the pitch is 16 / YB mod 16 (no bank conflict between them)
+__host__ __device__ constexpr int x_pitch(int L, int yb) {
+  int p = x_r1(L) * (x_r2(L) + 1);
+  while (p % 16 != (yb >= 16 ? 1 : yb == 1 ? 0 : 16 / yb)) ++p;
+  return p;
+}
+template <int R, int L, bool INV, class C>
+__device__ __forceinline__ void half_in(C* v, const C* tw) {
+  if constexpr (R <= 16 && (R & (R - 1)) == 0) HalfDFT<R, INV, C>::in(v);
+  else dft_half_in<R, L, INV, C>(v, tw);
+}
+template <int R, int L, bool INV, class C>
+__device__ __forceinline__ void half_out(C* v, const C* tw) {
+  if constexpr (R <= 16 && (R & (R - 1)) == 0) HalfDFT<R, INV, C>::out(v);
+  else dft_half_out<R, L, INV, C>(v, tw);
+}
+
+// S_c[n] = sum_k L_c[n,k] x_k gathered node by node (the transpose of the interpolation
+// rows), then the forward x-FFT of each grid row.  One block holds the 4 components of YB
+// consecutive rows y of one plane z for BB right-hand sides.  Only the nodes some stencil
+// touches are visited (arow: their range per box row, anode: y N + x, aptr: their CSR
+// entries); the operator input is interleaved, xs[k][b], so the BB lanes of a node share
+// its coefficients and gather adjacent values.  KXM stores the kx-major grid of the plane
+// kernel, A[b][c][kx][z][y - ylo] (rows beyond the box written as zeros up to N), runs of
+// YB values; otherwise A[b][c][z][y][kx].
+template <int L, int YB, int BB, bool KXM, class C>
+__global__ void __launch_bounds__(256) k_anterp(const int* __restrict__ arow, const int* __restrict__ anode,
+                                                const int* __restrict__ aptr, const int* __restrict__ nidx,
+                                                const typename Real<C>::F4* __restrict__ ncoef,
+                                                const C* __restrict__ xs, const int* __restrict__ active, int nb,
+                                                C* __restrict__ A, const C* __restrict__ twg, int ylo, int nyb, int nz) {
   using R = typename Real<C>::T;
-  const int b = blockIdx.x;
-  if (active && !active[b]) return;
+  constexpr int N = L / 2, R1 = x_r1(L), R2 = x_r2(L), PX = x_pitch(L, KXM ? YB : 1), ROWS = 4 * YB * BB;
   C* tw = reinterpret_cast<C*>(aim_smem);
-  C* b0 = tw + L;
-  C* b1 = b0 + 4 * ypb * L;
+  C* in = tw + L;             // [bs][c][yy][N]
+  C* tmp = in + ROWS * N;     // [bs][c][yy][PX]
   load_twiddles(tw, twg, L);
-  const int z = zlo + blockIdx.z, y0 = ylo + blockIdx.y * ypb;  // rows of the active box
-  const C* vb = xs + (size_t)b * ns;
-  // gather the N nodes of each row (all threads busy), zero the padding half
-  for (int t = threadIdx.x; t < ypb * N; t += blockDim.x) {
-    const int yy = t / N, x = t % N, y = y0 + yy;
-    C a0{}, a1{}, a2{}, a3{};
-    if (y <= yhi) {
-      const size_t n = ((size_t)z * N + y) * N + x;
-      int e = nptr[n];
-      const int e1 = nptr[n + 1];
-      // eight entries at a time: their index and coefficient loads, then their gathers of
+  for (int i = threadIdx.x; i < ROWS * N; i += 256) in[i] = C{};
+  pdl_wait();
+  const int b0 = blockIdx.x * BB, y0 = blockIdx.y * YB, z = blockIdx.z;  // y relative to the box
+  if (BB == 1 && active && !active[b0]) return;
+  __syncthreads();
+  const int ye = min(y0 + YB, nyb);
+  if (y0 < nyb) {
+    const int k0 = arow[z * nyb + y0], items = (arow[z * nyb + ye] - k0) * BB;
+    for (int i = threadIdx.x; i < items; i += 256) {
+      const int bs = i % BB, k = k0 + i / BB, b = b0 + bs;
+      if (BB > 1 && (b >= nb || (active && !active[b]))) continue;
+      const int nd = anode[k], yy = nd / N - ylo - y0, x = nd % N;
+      const C* vb = xs + b;
+      C a0{}, a1{}, a2{}, a3{};
+      int e = aptr[k];
+      const int e1 = aptr[k + 1];
+      // four entries at a time: their index and coefficient loads, then their gathers of
       // x, are independent and in flight together (the sums keep the entry order)
-      for (; e + 8 <= e1; e += 8) {
-        int k[8];
-        typename Real<C>::F4 w[8];
-        C xv[8];
-#pragma unroll
-        for (int u = 0; u < 8; ++u) {
-          k[u] = nidx[e + u];
-          w[u] = ncoef[e + u];
-        }
-#pragma unroll
-        for (int u = 0; u < 8; ++u) xv[u] = vb[k[u]];
-#pragma unroll
-        for (int u = 0; u < 8; ++u) {
-          a0 += (R)w[u].x * xv[u];
-          a1 += (R)w[u].y * xv[u];
-          a2 += (R)w[u].z * xv[u];
-          a3 += (R)w[u].w * xv[u];
-        }
-      }
-      if (e + 4 <= e1) {  // then four
-        int k[4];
+      for (; e + 4 <= e1; e += 4) {
+        int j[4];
         typename Real<C>::F4 w[4];
         C xv[4];
 #pragma unroll
         for (int u = 0; u < 4; ++u) {
-          k[u] = nidx[e + u];
+          j[u] = nidx[e + u];
           w[u] = ncoef[e + u];
         }
 #pragma unroll
-        for (int u = 0; u < 4; ++u) xv[u] = vb[k[u]];
+        for (int u = 0; u < 4; ++u) xv[u] = vb[(size_t)j[u] * nb];
 #pragma unroll
         for (int u = 0; u < 4; ++u) {
           a0 += (R)w[u].x * xv[u];
@@ -98,46 +108,102 @@ __global__ void __launch_bounds__(256) k_anterp_rows(const int* __restrict__ npt
           a2 += (R)w[u].z * xv[u];
           a3 += (R)w[u].w * xv[u];
         }
-        e += 4;
       }
       for (; e < e1; ++e) {
-        const int k = nidx[e];
         const typename Real<C>::F4 w = ncoef[e];
-        const C xv = vb[k];
+        const C xv = vb[(size_t)nidx[e] * nb];
         a0 += (R)w.x * xv;
         a1 += (R)w.y * xv;
         a2 += (R)w.z * xv;
         a3 += (R)w.w * xv;
       }
+      C* t = in + (bs * 4 * YB + yy) * N + x;
+      t[0] = a0;
+      t[YB * N] = a1;
+      t[2 * YB * N] = a2;
+      t[3 * YB * N] = a3;
     }
-    b0[(0 * ypb + yy) * L + x] = a0;
-    b0[(1 * ypb + yy) * L + x] = a1;
-    b0[(2 * ypb + yy) * L + x] = a2;
-    b0[(3 * ypb + yy) * L + x] = a3;
   }
-  C* res;
-  if constexpr (two_step_len(L)) {  // the padding half is never read
-    __syncthreads();
-    row_fft2<L, false, C, true>(b0, b1, 4 * ypb, tw);
-    res = b0;
-  } else {
-    for (int t = threadIdx.x; t < 4 * ypb * (L - N); t += blockDim.x) {
-      const int row = t / (L - N), x = N + t % (L - N);
-      b0[row * L + x] = C{};
+  __syncthreads();
+  for (int u = threadIdx.x; u < ROWS * R2; u += 256) {
+    const int n2 = u % R2, row = u / R2;
+    C v[R1];
+#pragma unroll
+    for (int n1 = 0; n1 < R1 / 2; ++n1) v[n1] = in[row * N + R2 * n1 + n2];
+    half_in<R1, L, false, C>(v, tw);
+#pragma unroll
+    for (int k1 = 0; k1 < R1; ++k1) tmp[row * PX + k1 * (R2 + 1) + n2] = k1 ? v[k1] * tw[n2 * k1] : v[k1];
+  }
+  __syncthreads();
+  for (int u = threadIdx.x; u < ROWS * R1; u += 256) {
+    int k1, row;
+    if (KXM) {
+      const int yy = u % YB, r = u / YB;
+      k1 = r % R1;
+      row = (r / R1) * YB + yy;
+    } else {
+      k1 = u % R1;
+      row = u / R1;
     }
-    __syncthreads();
-    res = line_fft_rows<L, false, C>(b0, b1, 4 * ypb, tw);
+    const int yy = row % YB, c = (row / YB) & 3, b = b0 + row / (4 * YB);
+    if (BB > 1 && (b >= nb || (active && !active[b]))) continue;
+    C v[R2];
+#pragma unroll
+    for (int n2 = 0; n2 < R2; ++n2) v[n2] = tmp[row * PX + k1 * (R2 + 1) + n2];
+    DFTL<R2, L, false, C>::run(v, tw);
+    if (KXM) {
+      C* dst = A + ((size_t)(b * 4 + c) * L * nz + z) * N + y0 + yy;
+#pragma unroll
+      for (int k2 = 0; k2 < R2; ++k2) dst[(size_t)(k1 + R1 * k2) * nz * N] = v[k2];
+    } else if (y0 + yy < nyb) {
+      C* dst = A + (((size_t)(b * 4 + c) * nz + z) * N + ylo + y0 + yy) * L + k1;
+#pragma unroll
+      for (int k2 = 0; k2 < R2; ++k2) dst[R1 * k2] = v[k2];
+    }
   }
-  for (int t = threadIdx.x; t < 4 * ypb * L; t += blockDim.x) {
-    const int row = t / L, x = t % L, c = row / ypb, y = y0 + row % ypb;
-    if (y <= yhi) A[((((size_t)b * 4 + c) * nz + blockIdx.z) * N + y) * L + x] = res[t];
+}
+
+// Inverse x-FFT of the kx-major grid: A[bc][kx][z][y] -> P[bc][z][ylo + y][x < N].  One
+// block takes YB rows y of one plane z; lanes walk the rows first, so every load is a run
+// of YB values, and only the outputs x < N are formed.
+template <int L, int YB, class C>
+__global__ void __launch_bounds__(256) k_xinv(const C* __restrict__ A, C* __restrict__ P,
+                                              const C* __restrict__ twg, int ylo, int nyb, int nz) {
+  constexpr int N = L / 2, R1 = x_r1(L), R2 = x_r2(L), PX = x_pitch(L, YB);
+  C* tw = reinterpret_cast<C*>(aim_smem);
+  C* tmp = tw + L;
+  load_twiddles(tw, twg, L);
+  pdl_wait();
+  __syncthreads();
+  const int y0 = blockIdx.x * YB, z = blockIdx.y, bc = blockIdx.z;
+  const C* src = A + ((size_t)bc * L * nz + z) * N + y0;
+  for (int u = threadIdx.x; u < YB * R2; u += 256) {
+    const int yy = u % YB, n2 = u / YB;
+    C v[R1];
+#pragma unroll
+    for (int n1 = 0; n1 < R1; ++n1) v[n1] = src[(size_t)(R2 * n1 + n2) * nz * N + yy];
+    DFTL<R1, L, true, C>::run(v, tw);
+#pragma unroll
+    for (int k1 = 0; k1 < R1; ++k1)
+      tmp[yy * PX + k1 * (R2 + 1) + n2] = k1 ? v[k1] * conjc(tw[n2 * k1]) : v[k1];
   }
-  pdl_trigger();
+  __syncthreads();
+  C* dst = P + ((size_t)bc * nz + z) * N * N + (size_t)(ylo + y0) * N;
+  for (int u = threadIdx.x; u < YB * R1; u += 256) {
+    const int k1 = u % R1, yy = u / R1;
+    C v[R2];
+#pragma unroll
+    for (int n2 = 0; n2 < R2; ++n2) v[n2] = tmp[yy * PX + k1 * (R2 + 1) + n2];
+    half_out<R2, L, true, C>(v, tw);
+    if (y0 + yy < nyb)
+#pragma unroll
+      for (int k2 = 0; k2 < R2 / 2; ++k2) dst[(size_t)yy * N + k1 + R1 * k2] = v[k2];
+  }
 }
 
 // Operator input: x_b = scale_b(j) * dinv .* v_b (selection, Krylov scale and
 // preconditioner applied once), in the grid precision for the anterpolation gather
-// and in FP64 for the near-zone product.
+// (interleaved, xs[k][b]) and in FP64 for the near-zone product (xd[b][k]).
 template <class C>
 __global__ void __launch_bounds__(256) k_prep(const double2* __restrict__ v, const double2* __restrict__ dinv,
                                               VecSel vs, const int* __restrict__ active, int ns, int nb,
@@ -159,9 +225,8 @@ __global__ void __launch_bounds__(256) k_prep(const double2* __restrict__ v, con
     const double2 d = dinv[k];
     x = make_double2(x.x * d.x - x.y * d.y, x.x * d.y + x.y * d.x);
   }
-  xs[idx] = cvt<C>(x);
+  xs[(size_t)k * nb + b] = cvt<C>(x);
   if (xd) xd[idx] = x;
-  pdl_trigger();
 }
 
 // The same with the SAI as the preconditioner: x_b[k] = scale_b(j) *
@@ -234,14 +299,12 @@ __global__ void __launch_bounds__(256) k_prep_sai(const double2* __restrict__ v,
   if (on && lane == 0) {
     const double2 x = make_double2(sc * (double)xr, sc * (double)xi);
     const size_t idx = (size_t)b * ns + k;
-    xs[idx] = cvt<C>(x);
+    xs[(size_t)k * nb + b] = cvt<C>(x);
     if (xd) xd[idx] = x;
   }
-  pdl_trigger();
 }
 
 // ---------------------------------------------------------------- z pass with the kernel
-__device__ __forceinline__ int fold(int k, int N) { return k <= N ? k : 2 * N - k; }
 
 // Geometry of a z pass.  The slab holds the nz z-planes of the active box (plane p is grid
 // z = box_lo + p), each an L x L plane of x/y spectra.  The z transform length LZ (a
@@ -339,18 +402,6 @@ __device__ __forceinline__ void zcol_step_c(const C* t, const C* tw, C* __restri
       if (p < nz) col[(long long)p * es + l] = v[n1];
     }
   }
-}
-
-// Grid order of the z-pass blocks: (right-hand side, component) fastest, then the x
-// tile, then the row y taken in mirror pairs (0, N, 1, L-1, 2, L-2, ...).  Every block
-// reads the kernel-spectrum octant at (fold(kz), fold(y), fold(x)); the octant of a large
-// grid does not fit in L2, and this order keeps the blocks that read the same entries
-// (all right-hand sides and components of one kernel kind, the rows y and L-y) close in
-// time, so the octant comes from DRAM about once per launch.
-__device__ __forceinline__ int zpass_row(int j, int N) {
-  if (j < 2) return j * N;
-  const int k = ((j - 2) >> 1) + 1;
-  return (j & 1) ? 2 * N - k : k;
 }
 
 // the kernel-spectrum column of kind `kind` at (x, y): entry kz at [fold(kz, LZ/2) * n1^2]
@@ -646,6 +697,36 @@ __global__ void __launch_bounds__(256) k_block_square(BlockSquare sq, const C* _
   }
 }
 
+// The same on spectra in the plane kernel's order, [bc][kx][group][pair][unit][2], with the
+// taps from its tabulated kernel spectra.
+template <int B, class C>
+__global__ void __launch_bounds__(256) k_block_square_plane(BlockSquare sq, const C* __restrict__ G, PlaneOrder o,
+                                                            int ng, long long n) {
+  const long long per_bc = (long long)o.L * o.L * o.LZ;
+  const size_t kind_off = (size_t)(o.L / 2 + 1) * plane_g_elems(o), gm = plane_spec_elems(o);
+  const int m0 = sq.toff - B + 1;  // tap[t] = G^_{m0 + t}
+  for (long long q = blockIdx.x * 256LL + threadIdx.x; q < n; q += (long long)gridDim.x * 256) {
+    const size_t go = ((q / per_bc) & 3) == 3 ? kind_off + plane_g_index(o, q % per_bc) : plane_g_index(o, q % per_bc);
+    C tap[2 * B - 1];
+#pragma unroll
+    for (int t = 0; t < 2 * B - 1; ++t) {
+      const int m = m0 + t;
+      tap[t] = (m >= 1 && m <= ng) ? __ldg(G + (size_t)m * gm + go) : C{};
+    }
+    C s[B];
+#pragma unroll
+    for (int j = 0; j < B; ++j) s[j] = reinterpret_cast<const C*>(sq.src[j])[q];
+#pragma unroll
+    for (int i = 0; i < B; ++i) {
+      C acc{};
+#pragma unroll
+      for (int j = 0; j < B; ++j) acc += tap[B - 1 + i - j] * s[j];
+      C* d = reinterpret_cast<C*>(sq.dst[i]) + q;
+      *d = *d + acc;
+    }
+  }
+}
+
 // z lengths with a factor 3 keep x/y-transformed history slabs: the delay sum recomputes
 // each slab's forward z-transform (steps A and B of the z pass), multiplies it by its
 // delay's kernel spectrum and accumulates in the registers of the step-B threads; then one
@@ -866,6 +947,8 @@ inline const float2* sel_twz(aim_ctx* c, float2*) { return c->d_twzf; }
 inline const double2* sel_twz(aim_ctx* c, double2*) { return c->d_twz; }
 inline const float2* sel_kspec(aim_ctx* c, float2*) { return c->d_kspecf; }
 inline const double2* sel_kspec(aim_ctx* c, double2*) { return c->d_kspec; }
+inline const float2* sel_plane(aim_ctx* c, float2*) { return c->d_planef; }
+inline const double2* sel_plane(aim_ctx* c, double2*) { return c->d_plane; }
 inline const float4* sel_ncoef(aim_ctx* c, float2*) { return c->d_ncoeff; }
 inline const double4_32a* sel_ncoef(aim_ctx* c, double2*) { return c->d_ncoef; }
 inline const float* sel_lam(aim_ctx* c, float2*) { return c->d_lamf; }
@@ -900,6 +983,13 @@ inline void with_zlen(int lz, F&& f) {
 }
 constexpr size_t kPlanSmemMax = 220 * 1024;  // dynamic shared memory a plan may ask for
 
+// sizes whose z passes always run in the plane kernel (a factor-3 z length may fall back to
+// the separate passes, see plane_setup)
+template <int L, int LZ, class C>
+constexpr bool plane_always() {
+  return plane_fits<L, LZ, C>() && pow2_len(LZ);
+}
+
 template <int L, class C>
 struct GridOps {
   // ------------------------------------------------------------ launch shapes
@@ -909,19 +999,35 @@ struct GridOps {
     return w;
   }
   static int def_cw() { return col_width_p2<L, C>(); }
-  static int def_rp() { return pow2_len(L) ? std::max(1, 4096 / L) : std::max(1, 256 / split_r1(L)); }
-  static int def_ypb() { return std::max(1, 256 / (L / 2)); }
+  // kx-major grids (the plane kernel runs the y and z passes)
+  static bool kxm(const aim_ctx* c) { return sizeof(C) == sizeof(float2) ? c->plane : c->plane64; }
+  static int def_rp(const aim_ctx* c) {
+    if (!kxm(c)) return pow2_len(L) ? std::max(1, 4096 / L) : std::max(1, 256 / split_r1(L));
+    return fill_rows(c, 16, (long long)c->batch_max * 4 * c->NZ);
+  }
+  static int def_ypb(const aim_ctx* c) {
+    return kxm(c) ? fill_rows(c, 8, (long long)c->NZ * ((c->batch_max + 1) / 2)) : 1;
+  }
+  // the most rows per block (a power of two up to `most`) that still give every SM two blocks
+  static int fill_rows(const aim_ctx* c, int most, long long others) {
+    int r = std::min(most, L / 2);
+    while (r > 1 && (c->N / r) * others < 304) r /= 2;
+    return r;
+  }
   static size_t smem_z(int lz, int w) { return (size_t)(lz + lz * w) * sizeof(C); }
   static size_t smem_y(int w) { return (size_t)(L + L * w) * sizeof(C); }
   static size_t smem_x(int rp) { return (size_t)(L + rp * row_tmp_pitch<L>()) * sizeof(C); }
-  static size_t smem_anterp(int yp) { return (size_t)(L + 4 * yp * L + row_scratch<L>(4 * yp)) * sizeof(C); }
+  static size_t smem_anterp(int yb, int bb, bool k) {
+    return (L + (size_t)4 * yb * bb * (L / 2 + x_pitch(L, k ? yb : 1))) * sizeof(C);
+  }
+  static size_t smem_xinv(int yb) { return (L + (size_t)yb * x_pitch(L, yb)) * sizeof(C); }
   // the plan holds the shapes of the context's own precision (the FP64 residual of the
   // refinement on the complex64 path runs with the defaults)
   static bool own(const aim_ctx* c) { return (c->precision == AIM_C64) == (sizeof(C) == sizeof(float2)); }
   static int zw(const aim_ctx* c) { return own(c) && c->plan.zw ? c->plan.zw : def_zw(c); }
   static int cw(const aim_ctx* c) { return own(c) && c->plan.cw ? c->plan.cw : def_cw(); }
-  static int rp(const aim_ctx* c) { return own(c) && c->plan.rp ? c->plan.rp : def_rp(); }
-  static int ypb(const aim_ctx* c) { return own(c) && c->plan.ypb ? c->plan.ypb : def_ypb(); }
+  static int rp(const aim_ctx* c) { return own(c) && c->plan.rp ? c->plan.rp : def_rp(c); }
+  static int ypb(const aim_ctx* c) { return own(c) && c->plan.ypb ? c->plan.ypb : def_ypb(c); }
   // candidates the autotuner times: z tiles of x-adjacent columns (w divides L), y tiles
   static std::vector<int> zwidths(const aim_ctx* c) {
     std::vector<int> v;
@@ -935,17 +1041,32 @@ struct GridOps {
       if (w <= L && L % w == 0 && smem_y(w) <= kPlanSmemMax) v.push_back(w);
     return v;
   }
-  static std::vector<int> rps() {
+  static std::vector<int> rps(const aim_ctx* c) {
     std::vector<int> v;
-    for (int r : {2, 4, 8, 16, 32, 64})
-      if (smem_x(r) <= 100 * 1024) v.push_back(r);
+    if (kxm(c)) {
+      for (int r : {1, 2, 4, 8, 16})
+        if (r <= c->N) v.push_back(r);
+    } else {
+      for (int r : {2, 4, 8, 16, 32, 64})
+        if (smem_x(r) <= 100 * 1024) v.push_back(r);
+    }
     return v;
   }
-  static std::vector<int> ypbs(int N) {
+  static std::vector<int> ypbs(const aim_ctx* c) {
     std::vector<int> v;
     for (int y : {1, 2, 4, 8})
-      if (y <= N && smem_anterp(y) <= 100 * 1024) v.push_back(y);
+      if (y <= c->N && smem_anterp(y, 1, kxm(c)) <= 100 * 1024) v.push_back(y);
     return v;
+  }
+  // rows per block of the x passes: the largest instantiated count not above the plan's
+  template <class F>
+  static void with_rows(int r, int most, F&& f) {
+    r = std::min(r, most);
+    if (r >= 16) f(std::integral_constant<int, 16>{});
+    else if (r >= 8) f(std::integral_constant<int, 8>{});
+    else if (r >= 4) f(std::integral_constant<int, 4>{});
+    else if (r >= 2) f(std::integral_constant<int, 2>{});
+    else f(std::integral_constant<int, 1>{});
   }
 
   // stage i + forward x and y passes: v[nb][ns] (optionally times dinv) -> slab [nb][4][nz][L][L]
@@ -971,15 +1092,38 @@ struct GridOps {
   static ZGeom zgeom(const aim_ctx* c) { return ZGeom{L, c->N, c->NZ}; }
 
   // anterpolation gather + forward x pass: d_xs -> A (rows of the active box)
+  template <bool KXM>
+  static void anterp_as(aim_ctx* c, int nb, const int* active) {
+    const int most = std::min(8, L / 2), nyb = nbox(c, 1);
+    // a batch in pairs: two right-hand sides per block share the coefficient loads
+    const int bb = nb > 1 ? 2 : 1;
+    int yp = ypb(c);
+    while (yp > 1 && smem_anterp(yp, bb, KXM) > (size_t)kPlaneSmemMax) yp /= 2;
+    with_rows(yp, most, [&](auto yt) {
+      constexpr int YB = decltype(yt)::value;
+      if constexpr (YB <= 8 && YB <= L / 2) {
+        auto go = [&](auto bt) {
+          constexpr int BB = decltype(bt)::value;
+          auto kern = k_anterp<L, YB, BB, KXM, C>;
+          const size_t sm = smem_anterp(YB, BB, KXM);
+          if (sm > (size_t)kPlaneSmemMax) throw AimError{AIM_ERR_ARG, "launch plan: anterpolation tile"};
+          smem_opt_in(kern, sm);
+          launch_pdl(c->stream, dim3((nb + BB - 1) / BB, ((KXM ? c->N : nyb) + YB - 1) / YB, c->NZ), dim3(256), sm,
+                     kern, (const int*)c->d_arow, (const int*)c->d_anode, (const int*)c->d_aptr,
+                     (const int*)c->d_nidx, ncoef(c), reinterpret_cast<const C*>(c->d_xs), active, nb,
+                     reinterpret_cast<C*>(c->d_A), twiddles(c), c->box_lo[1], nyb, c->NZ);
+        };
+        if (bb == 2) go(std::integral_constant<int, 2>{});
+        else go(std::integral_constant<int, 1>{});
+      }
+    });
+  }
   static void anterp_x(aim_ctx* c, int nb, const int* active) {
-    const int N = c->N, yp = ypb(c);
-    const size_t sm = smem_anterp(yp);
-    smem_opt_in(k_anterp_rows<L, C>, sm);
     KScope ks(c, AIM_K_ANTERP_XFFT);
-    launch_pdl(c->stream, dim3(nb, (nbox(c, 1) + yp - 1) / yp, c->NZ), dim3(256), sm, k_anterp_rows<L, C>,
-               (const int*)c->d_nptr, (const int*)c->d_nidx, ncoef(c), reinterpret_cast<const C*>(c->d_xs), active,
-               c->ns, N, yp, reinterpret_cast<C*>(c->d_A), twiddles(c), c->box_lo[1], c->box_hi[1], c->box_lo[2],
-               c->NZ);
+    if constexpr (L <= 256) {
+      if (kxm(c)) return anterp_as<true>(c, nb, active);
+    }
+    anterp_as<false>(c, nb, active);
   }
 
   // forward y pass (pruned input): A -> slab
@@ -1025,6 +1169,21 @@ struct GridOps {
 
   // inverse x pass (pruned output): A -> P, the rows of the active box, outputs x in the box
   static void x_inv(aim_ctx* c, int nb) {
+    if constexpr (L <= 256) {
+      if (kxm(c)) {
+        KScope ks(c, AIM_K_XFFT_INV);
+        with_rows(rp(c), std::min(16, L / 2), [&](auto yt) {
+          constexpr int YB = decltype(yt)::value;
+          if constexpr (YB <= L / 2) {
+            const size_t sm = smem_xinv(YB);
+            smem_opt_in(k_xinv<L, YB, C>, sm);
+            launch_pdl(c->stream, dim3((nbox(c, 1) + YB - 1) / YB, c->NZ, nb * 4), dim3(256), sm, k_xinv<L, YB, C>,
+                       (const C*)c->d_A, reinterpret_cast<C*>(c->d_P), twiddles(c), c->box_lo[1], nbox(c, 1), c->NZ);
+          }
+        });
+        return;
+      }
+    }
     const int N = c->N, r = rp(c), nz = c->NZ, ny = nbox(c, 1), nrows = nb * 4 * nz * ny;
     const size_t sm = smem_x(r);
     smem_opt_in(k_rows_p2<L, true, C>, sm);
@@ -1038,13 +1197,13 @@ struct GridOps {
                            VecSel vs = VecSel(), bool want_fp64 = false) {
     prep(c, nb, v, dinv, vs, active, want_fp64);
     anterp_x(c, nb, active);
-    y_fwd(c, nb, slab);
+    if (!kxm(c)) y_fwd(c, nb, slab);
   }
 
   // inverse y and x passes: Bf slab -> P, then interpolation + near terms
   static void backward(aim_ctx* c, int nb, const NearList& nl, const double2* base, double sign, const int* active,
                        double2* y, VecSel ys = VecSel()) {
-    y_inv(c, nb);
+    if (!kxm(c)) y_inv(c, nb);
     x_inv(c, nb);
     interp(c, nb, reinterpret_cast<const C*>(c->d_P), nl, base, sign, active, y, ys);
   }
@@ -1064,12 +1223,13 @@ struct GridOps {
   static size_t octant(const aim_ctx* c) { return (size_t)(c->N + 1) * (c->N + 1) * (c->LZ / 2 + 1); }
 
   static void zconv(aim_ctx* c, int nb, int m, const int* active) {
+    KScope ks(c, AIM_K_ZCONV);
+    if (kxm(c)) return plane_launch<C>(c, nb, PLANE_CONV, m, active, nullptr);
     C* Bf = reinterpret_cast<C*>(c->d_Bf);
     const C* G = kspec(c) + (size_t)m * 2 * octant(c);
-    KScope ks(c, AIM_K_ZCONV);
     with_zlen(c->LZ, [&](auto lz) {
       constexpr int LZ = decltype(lz)::value;
-      if constexpr (LZ <= L) {
+      if constexpr (LZ <= L && !plane_always<L, LZ, C>()) {
         with_width(zw(c), [&](auto wt) {
           constexpr int ZW = decltype(wt)::value;
           if constexpr (ZW <= L) {
@@ -1124,13 +1284,18 @@ struct GridOps {
       }
       field = arg;
     };
-    pick(p.zw, zwidths(c), [&] { zconv(c, nb, 0, nullptr); });
-    pick(p.cw, ywidths(), [&] {
-      y_fwd(c, nb, reinterpret_cast<C*>(c->d_Bf));
-      y_inv(c, nb);
-    });
-    pick(p.rp, rps(), [&] { x_inv(c, nb); });
-    pick(p.ypb, ypbs(c->N), [&] { anterp_x(c, nb, nullptr); });
+    if (kxm(c)) {  // the plane kernel has one shape; its fields keep the defaults
+      p.zw = def_zw(c);
+      p.cw = def_cw();
+    } else {
+      pick(p.zw, zwidths(c), [&] { zconv(c, nb, 0, nullptr); });
+      pick(p.cw, ywidths(), [&] {
+        y_fwd(c, nb, reinterpret_cast<C*>(c->d_Bf));
+        y_inv(c, nb);
+      });
+    }
+    pick(p.rp, rps(c), [&] { x_inv(c, nb); });
+    pick(p.ypb, ypbs(c), [&] { anterp_x(c, nb, nullptr); });
     cudaEventDestroy(e0);
     cudaEventDestroy(e1);
   }
@@ -1138,9 +1303,13 @@ struct GridOps {
   // forward z-FFT of the slab in Bf into the z-spectral history layout at dst
   // (power-of-two z lengths only)
   static void zfwd(aim_ctx* c, int nb, C* dst) {
+    if (kxm(c)) {
+      KScope ks(c, AIM_K_ZFWD);
+      return plane_launch<C>(c, nb, PLANE_FWD, 0, nullptr, dst);
+    }
     with_zlen(c->LZ, [&](auto lz) {
       constexpr int LZ = decltype(lz)::value;
-      if constexpr (pow2_len(LZ) && LZ <= L) {
+      if constexpr (pow2_len(LZ) && LZ <= L && !plane_always<L, LZ, C>()) {
         constexpr int ZW = zcol_width<LZ, C>();
         const size_t sm = smem_z(LZ, ZW);
         KScope ks(c, AIM_K_ZFWD);
@@ -1154,12 +1323,13 @@ struct GridOps {
     });
   }
 
-  static void zrhs(aim_ctx* c, int nb, const SlabList& sl) {
+  static void zrhs(aim_ctx* c, int nb, const SlabList& sl, C* scratch) {
     C* Bf = reinterpret_cast<C*>(c->d_Bf);
     KScope ks(c, AIM_K_ZRHS);
+    if (kxm(c)) return plane_rhs<C>(c, nb, sl, scratch);
     with_zlen(c->LZ, [&](auto lz) {
       constexpr int LZ = decltype(lz)::value;
-      if constexpr (LZ <= L) {
+      if constexpr (LZ <= L && !plane_always<L, LZ, C>()) {
         if constexpr (pow2_len(LZ) && LZ <= 256 && L <= 256 && std::is_same<C, float2>::value) {
           // the spectra's ring slots (the march and aim_rhs keep every history slab in the ring)
           const size_t slab = op_slab_bytes(c, c->batch_max);
@@ -1207,9 +1377,13 @@ struct GridOps {
 
   // blocked right-hand side: pending z-spectra -> slab of potentials in Bf (cleared)
   static void zinv_pending(aim_ctx* c, int nb, C* S) {
+    if (kxm(c)) {
+      KScope ks(c, AIM_K_ZINV_PENDING);
+      return plane_launch<C>(c, nb, PLANE_PENDING, 0, nullptr, S);
+    }
     with_zlen(c->LZ, [&](auto lz) {
       constexpr int LZ = decltype(lz)::value;
-      if constexpr (pow2_len(LZ) && LZ <= L) {
+      if constexpr (pow2_len(LZ) && LZ <= L && !plane_always<L, LZ, C>()) {
         constexpr int ZW = L < 16 ? L : 16;
         const size_t sm = smem_z(LZ, ZW);
         KScope ks(c, AIM_K_ZINV_PENDING);
@@ -1229,7 +1403,14 @@ struct GridOps {
     KScope ks(c, AIM_K_BLOCK_SQUARE);
     auto go = [&](auto bt) {
       constexpr int B = decltype(bt)::value;
-      k_block_square<B, C><<<grid, 256, 0, c->stream>>>(sq, kspec(c), zgeom(c), c->LZ, c->n_delays, n);
+      if (kxm(c))
+        with_zlen(c->LZ, [&](auto lz) {
+          if constexpr (plane_fits<L, decltype(lz)::value, C>())
+            k_block_square_plane<B, C><<<grid, 256, 0, c->stream>>>(
+                sq, plane_spec(c), plane_order<L, decltype(lz)::value, C>(), c->n_delays, n);
+        });
+      else
+        k_block_square<B, C><<<grid, 256, 0, c->stream>>>(sq, kspec(c), zgeom(c), c->LZ, c->n_delays, n);
     };
     switch (sq.b) {
       case 1: go(std::integral_constant<int, 1>{}); break;
@@ -1245,6 +1426,7 @@ struct GridOps {
   static const C* twiddles(aim_ctx* c) { return sel_tw(c, (C*)nullptr); }
   static const C* ztwiddles(aim_ctx* c) { return sel_twz(c, (C*)nullptr); }
   static const C* kspec(aim_ctx* c) { return sel_kspec(c, (C*)nullptr); }
+  static const C* plane_spec(aim_ctx* c) { return sel_plane(c, (C*)nullptr); }
   static const typename Real<C>::F4* ncoef(aim_ctx* c) { return sel_ncoef(c, (C*)nullptr); }
   static const typename Real<C>::T* lam(aim_ctx* c) { return sel_lam(c, (C*)nullptr); }
 };

@@ -18,6 +18,7 @@
 #include "aim_internal.h"
 #include "fft_kernels.cuh"
 #include "setup_host.h"
+#include "operator.h"
 #include "setup_gpu.h"
 #include "tbasis.cuh"
 
@@ -611,11 +612,31 @@ void setup_device_tables(aim_ctx* c, HostMesh& hm, const std::vector<int>& ancho
       cf[e] = make_double4_32a(l[0], l[64], l[128], l[192]);
       cff[e] = make_float4((float)l[0], (float)l[64], (float)l[128], (float)l[192]);
     }
-    c->d_nptr = (int*)aim_alloc(c, nptr.size() * sizeof(int));
+    // the nodes with entries, by box row (the entries of consecutive nodes are contiguous)
+    std::vector<int> arow, anode, aptr;
+    for (int z = c->box_lo[2]; z <= c->box_hi[2]; ++z)
+      for (int y = c->box_lo[1]; y <= c->box_hi[1]; ++y) {
+        arow.push_back((int)anode.size());
+        const size_t n0 = ((size_t)z * N + y) * N;
+        for (int x = 0; x < N; ++x)
+          if (nptr[n0 + x + 1] > nptr[n0 + x]) {
+            anode.push_back(y * N + x);
+            aptr.push_back(nptr[n0 + x]);
+          }
+      }
+    arow.push_back((int)anode.size());
+    aptr.push_back((int)nidx.size());
+    auto put = [&](const std::vector<int>& v) {
+      int* d = (int*)aim_alloc(c, v.size() * sizeof(int));
+      AIM_CUDA(cudaMemcpyAsync(d, v.data(), v.size() * sizeof(int), cudaMemcpyHostToDevice, st));
+      return d;
+    };
+    c->d_arow = put(arow);
+    c->d_anode = put(anode);
+    c->d_aptr = put(aptr);
     c->d_nidx = (int*)aim_alloc(c, nidx.size() * sizeof(int));
     c->d_ncoef = (double4_32a*)aim_alloc(c, cf.size() * sizeof(double4_32a));
     c->d_ncoeff = (float4*)aim_alloc(c, cff.size() * sizeof(float4));
-    AIM_CUDA(cudaMemcpyAsync(c->d_nptr, nptr.data(), nptr.size() * sizeof(int), cudaMemcpyHostToDevice, st));
     AIM_CUDA(cudaMemcpyAsync(c->d_nidx, nidx.data(), nidx.size() * sizeof(int), cudaMemcpyHostToDevice, st));
     AIM_CUDA(cudaMemcpyAsync(c->d_ncoef, cf.data(), cf.size() * sizeof(double4_32a), cudaMemcpyHostToDevice, st));
     AIM_CUDA(cudaMemcpyAsync(c->d_ncoeff, cff.data(), cff.size() * sizeof(float4), cudaMemcpyHostToDevice, st));
@@ -698,6 +719,7 @@ void setup_device_tables(aim_ctx* c, HostMesh& hm, const std::vector<int>& ancho
     cudaFree(GA);
     cudaFree(GP);
   }
+  plane_setup(c);
   // ---- near zone
   {
     std::vector<int> rowptr, col;
