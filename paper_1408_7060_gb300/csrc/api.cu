@@ -884,7 +884,9 @@ int aim_rcs(aim_ctx* c, int32_t n_freq, const double* freqs, int32_t nb, const a
     const double2* ds = dev_in(c, spec, n, scratch(c, n, 1));
     const bool dev = is_device_ptr(sigma);
     double* out = dev ? sigma : reinterpret_cast<double*>(scratch(c, no / 2 + 1, 2));
-    rcs_farfield(c, n_freq, nb, ds, nd, dd, dd + 6 * nd, out);
+    int nfc, splits;
+    double2* work = scratch(c, rcs_workspace(c, n_freq, nd, nfc, splits), 3);
+    rcs_farfield(c, n_freq, nb, ds, nd, dd, dd + 6 * nd, work, out);
     if (!dev) AIM_CUDA(cudaMemcpyAsync(sigma, out, no * sizeof(double), cudaMemcpyDeviceToHost, c->stream));
     AIM_CUDA(cudaStreamSynchronize(c->stream));
     return AIM_OK;

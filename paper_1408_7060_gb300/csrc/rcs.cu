@@ -14,6 +14,7 @@
 //    EFIE times j w), whose far field is E = -j w mu/(4 pi) e^{-j k r}/r F with
 //    F = (I - r r) . sum_k I_k int S_k(r') e^{+j k r.r'} dS' (7-point cubature), and
 //    sigma = 4 pi |pol . E r|^2.
+#include <algorithm>
 #include <cmath>
 #include <complex>
 #include <vector>
@@ -49,64 +50,168 @@ __global__ void __launch_bounds__(kT) k_scale_freq(RcsPhases s, long long n, dou
     }
 }
 
-__device__ __forceinline__ double warp_sum_d(double v) {
-  for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
-  return v;
-}
+// The far field in three steps.  On a face the current is affine,
+//   J(r) = sum_e c_e I_e (r - v_e) = a (r - C) - b,  c_e = sign l_e / (2 A), C the centroid,
+// so a face carries one complex scalar and one complex vector per right-hand side
+// (k_rcs_faces), whatever the direction.  For a direction the projected current at a
+// cubature point is u . J = a u . (r - C) - u . b, u = pol - r (r . pol), and the sums over the
+// 7 points  X = sum_q w_q u . (r_q - C) e^{jkr.r_q},  Y = sum_q w_q e^{jkr.r_q}  do not depend on
+// the right-hand side (k_rcs_dirs); the points are the centroid and, for two fractions s,
+// centroid + s (vertex - centroid), so their phases differ from the centroid's by small
+// angles, which need the Taylor series of sine and cosine instead of a range reduction.
+// The kernels are bound by FP64 arithmetic: about 270 operations per face, direction and
+// frequency plus 20 per right-hand side (each
+// point evaluated by itself for every right-hand side took about 120 per point: 12.5 ms for
+// 5120 faces, 288 directions, 3 frequencies and 2 waves, 2.3 ms now).
+constexpr int kRcsB = 4;  // right-hand sides per pass
 
-// One block per (direction d, right-hand side b, frequency f): the radiation vector of
-// spec[f][b] summed over every cubature point of every face, then projected.
-// dirs: [nd][6] (rhat, pol); fk: [n_freq][2] (k, 4 pi (w mu0 / 4 pi)^2).
-__global__ void __launch_bounds__(kT) k_rcs(int nt, const int* __restrict__ tbk, const double* __restrict__ tbs,
-                                             const int* __restrict__ tbf, const double* __restrict__ len,
-                                             const double* __restrict__ area, const double* __restrict__ V,
-                                             const double* __restrict__ qp, const double* __restrict__ qw, int ns,
-                                             int nb, const double2* __restrict__ spec, const double* __restrict__ fk,
-                                             const double* __restrict__ dirs, int nd, double* __restrict__ sig) {
-  const int d = blockIdx.x, b = blockIdx.y, f = blockIdx.z;
-  const double* rd = dirs + 6 * d;
-  const double rx = rd[0], ry = rd[1], rz = rd[2];
-  const double k = fk[2 * f];
-  const double2* I = spec + ((size_t)f * nb + b) * ns;
-  double a[6] = {0, 0, 0, 0, 0, 0};  // (re, im) of x, y, z
-  for (int idx = threadIdx.x; idx < nt * 7; idx += kT) {
-    const int t = idx / 7, q = idx % 7;
-    const double* r = qp + 21 * t + 3 * q;
-    double sn, cs;
-    sincos(k * (rx * r[0] + ry * r[1] + rz * r[2]), &sn, &cs);
-    const double wq = qw[7 * t + q];
+// fc[fb][4][nt]: a, b_x, b_y, b_z of every face for right-hand sides b0 .. b0 + nb' - 1 of
+// frequencies f0 .. (fb = (f - f0) kRcsB + (b - b0))
+__global__ void __launch_bounds__(kT) k_rcs_faces(int nt, const int* __restrict__ F, const int* __restrict__ tbk, const double* __restrict__ tbs,
+                                                  const int* __restrict__ tbf, const double* __restrict__ len,
+                                                  const double* __restrict__ area, const double* __restrict__ V, int ns,
+                                                  int nb, int b0, const double2* __restrict__ spec,
+                                                  double2* __restrict__ fc) {
+  const int t = blockIdx.x * kT + threadIdx.x, bs = blockIdx.y, f = blockIdx.z;
+  if (t >= nt) return;
+  double2 m[4] = {};
+  if (b0 + bs < nb) {
+    const double2* I = spec + ((size_t)f * nb + b0 + bs) * ns;
+    double C[3];
+    for (int d = 0; d < 3; ++d) C[d] = (V[3 * F[3 * t] + d] + V[3 * F[3 * t + 1] + d] + V[3 * F[3 * t + 2] + d]) / 3.0;
     for (int e = 0; e < 3; ++e) {
-      const int kk = tbk[3 * t + e];
-      if (kk < 0) continue;
-      const double cS = tbs[3 * t + e] * len[kk] / (2.0 * area[t]) * wq;
-      const double2 Ik = I[kk];
-      const double pr = cS * (Ik.x * cs - Ik.y * sn), pi = cS * (Ik.x * sn + Ik.y * cs);
+      const int k = tbk[3 * t + e];
+      if (k < 0) continue;
+      const double c = tbs[3 * t + e] * len[k] / (2.0 * area[t]);
+      const double2 x = make_double2(c * I[k].x, c * I[k].y);
       const double* vf = V + 3 * tbf[3 * t + e];
-      for (int x = 0; x < 3; ++x) {
-        const double dx = r[x] - vf[x];
-        a[2 * x] += pr * dx;
-        a[2 * x + 1] += pi * dx;
+      m[0].x += x.x;
+      m[0].y += x.y;
+      for (int d = 0; d < 3; ++d) {
+        m[1 + d].x += x.x * (vf[d] - C[d]);
+        m[1 + d].y += x.y * (vf[d] - C[d]);
       }
     }
   }
-  __shared__ double part[kT / 32][6];
+  for (int i = 0; i < 4; ++i) fc[((size_t)(f * kRcsB + bs) * 4 + i) * nt + t] = m[i];
+}
+
+// sin and cos of |x| <= 1/2: Taylor series to x^15 and x^14 (remainders below 1e-18)
+__device__ __forceinline__ void small_sincos(double x, double& s, double& c) {
+  const double y = x * x;
+  double p = -1.0 / 1307674368000.0, q = -1.0 / 87178291200.0;
+  p = p * y + 1.0 / 6227020800.0;
+  p = p * y - 1.0 / 39916800.0;
+  p = p * y + 1.0 / 362880.0;
+  p = p * y - 1.0 / 5040.0;
+  p = p * y + 1.0 / 120.0;
+  p = p * y - 1.0 / 6.0;
+  s = x + x * (y * p);
+  q = q * y + 1.0 / 479001600.0;
+  q = q * y - 1.0 / 3628800.0;
+  q = q * y + 1.0 / 40320.0;
+  q = q * y - 1.0 / 720.0;
+  q = q * y + 1.0 / 24.0;
+  q = q * y - 0.5;
+  c = 1.0 + y * q;
+}
+
+// part[fb][d][split] = sum over the faces of a split of u . int J e^{jkr.r'} dS'; grid
+// (nd, splits, frequencies).  dirs: [nd][6] (rhat, pol); fk: [n_freq][2] (k, prefactor).
+__global__ void __launch_bounds__(kT) k_rcs_dirs(int nt, const int* __restrict__ F, const double* __restrict__ V,
+                                                 const double* __restrict__ area, const double2* __restrict__ fc,
+                                                 const double* __restrict__ fk, const double* __restrict__ dirs,
+                                                 int nbc, double2* __restrict__ part) {
+  const int d = blockIdx.x, f = blockIdx.z, nd = gridDim.x, ns = gridDim.y;
+  const double* rd = dirs + 6 * d;
+  const double k = fk[2 * f];
+  const double rp = rd[0] * rd[3] + rd[1] * rd[4] + rd[2] * rd[5];
+  const double u[3] = {rd[3] - rd[0] * rp, rd[4] - rd[1] * rp, rd[5] - rd[2] * rp};
+  // the orbits (p, p, 1 - 2p) of the rule: fraction 1 - 3p towards the vertex, and weights
+  const double s15 = 3.8729833462074168852;  // sqrt 15
+  const double fr[2] = {1.0 - (6.0 - s15) / 7.0, 1.0 - (6.0 + s15) / 7.0};
+  const double w[2] = {(155.0 - s15) / 1200.0, (155.0 + s15) / 1200.0}, w0 = 9.0 / 40.0;
+  double2 acc[kRcsB] = {};
+  for (int t = blockIdx.y * kT + threadIdx.x; t < nt; t += ns * kT) {
+    double ph[3], g[3];
+    for (int i = 0; i < 3; ++i) {
+      const double* v = V + 3 * F[3 * t + i];
+      ph[i] = rd[0] * v[0] + rd[1] * v[1] + rd[2] * v[2];
+      g[i] = u[0] * v[0] + u[1] * v[1] + u[2] * v[2];
+    }
+    // (divisions: a rounded 1/3 or k r would shift every phase the same way)
+    const double dc = (ph[0] + ph[1] + ph[2]) / 3.0, gc = (g[0] + g[1] + g[2]) / 3.0, pc = k * dc;
+    for (int i = 0; i < 3; ++i) {
+      ph[i] = k * (ph[i] - dc);
+      g[i] -= gc;
+    }
+    const double big = fmax(fabs(ph[0]), fmax(fabs(ph[1]), fabs(ph[2])));
+    double2 X = make_double2(0.0, 0.0), Y = make_double2(w0, 0.0);
+    for (int o = 0; o < 2; ++o) {
+      double2 x = make_double2(0, 0), y = make_double2(0, 0);
+      for (int i = 0; i < 3; ++i) {
+        double sn, cs;
+        if (big * fabs(fr[1]) <= 0.5 && big * fabs(fr[0]) <= 0.5) small_sincos(fr[o] * ph[i], sn, cs);
+        else sincos(fr[o] * ph[i], &sn, &cs);
+        y.x += cs;
+        y.y += sn;
+        x.x += g[i] * cs;
+        x.y += g[i] * sn;
+      }
+      X.x += w[o] * fr[o] * x.x;
+      X.y += w[o] * fr[o] * x.y;
+      Y.x += w[o] * y.x;
+      Y.y += w[o] * y.y;
+    }
+    double sn, cs;
+    sincos(pc, &sn, &cs);
+    const double A = area[t];
+    sn *= A;
+    cs *= A;
+    X = make_double2(X.x * cs - X.y * sn, X.x * sn + X.y * cs);
+    Y = make_double2(Y.x * cs - Y.y * sn, Y.x * sn + Y.y * cs);
+#pragma unroll
+    for (int b = 0; b < kRcsB; ++b)
+      if (b < nbc) {
+        const double2* m = fc + (size_t)(f * kRcsB + b) * 4 * nt + t;
+        const double2 a = m[0], bx = m[nt], by = m[2 * (size_t)nt], bz = m[3 * (size_t)nt];
+        const double qx = u[0] * bx.x + u[1] * by.x + u[2] * bz.x, qy = u[0] * bx.y + u[1] * by.y + u[2] * bz.y;
+        acc[b].x += a.x * X.x - a.y * X.y - (qx * Y.x - qy * Y.y);
+        acc[b].y += a.x * X.y + a.y * X.x - (qx * Y.y + qy * Y.x);
+      }
+  }
+  __shared__ double red[kT / 32][2 * kRcsB];
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  for (int i = 0; i < 6; ++i) {
-    const double s = warp_sum_d(a[i]);
-    if (lane == 0) part[warp][i] = s;
+  for (int b = 0; b < nbc; ++b) {
+    const double2 s = warp_sum_c(acc[b]);
+    if (lane == 0) {
+      red[warp][2 * b] = s.x;
+      red[warp][2 * b + 1] = s.y;
+    }
   }
   __syncthreads();
-  if (threadIdx.x == 0) {
-    double v[6] = {0, 0, 0, 0, 0, 0};
-    for (int w = 0; w < kT / 32; ++w)
-      for (int i = 0; i < 6; ++i) v[i] += part[w][i];
-    const double* pol = rd + 3;
-    // e = pol . (v - r (r . v)), real and imaginary parts
-    const double rvr = rx * v[0] + ry * v[2] + rz * v[4], rvi = rx * v[1] + ry * v[3] + rz * v[5];
-    const double er = pol[0] * (v[0] - rx * rvr) + pol[1] * (v[2] - ry * rvr) + pol[2] * (v[4] - rz * rvr);
-    const double ei = pol[0] * (v[1] - rx * rvi) + pol[1] * (v[3] - ry * rvi) + pol[2] * (v[5] - rz * rvi);
-    sig[((size_t)f * nb + b) * nd + d] = fk[2 * f + 1] * (er * er + ei * ei);
+  if ((int)threadIdx.x < nbc) {
+    double2 s = make_double2(0, 0);
+    for (int q = 0; q < kT / 32; ++q) {
+      s.x += red[q][2 * threadIdx.x];
+      s.y += red[q][2 * threadIdx.x + 1];
+    }
+    part[((size_t)(f * kRcsB + threadIdx.x) * nd + d) * ns + blockIdx.y] = s;
   }
+}
+
+// sig[f][b0 + bs][d] = prefactor |sum of the splits|^2
+__global__ void __launch_bounds__(kT) k_rcs_finish(int nd, int splits, int nb, int b0, const double* __restrict__ fk,
+                                                   const double2* __restrict__ part, double* __restrict__ sig) {
+  const int d = blockIdx.x * kT + threadIdx.x, bs = blockIdx.y, f = blockIdx.z;
+  if (d >= nd) return;
+  double2 s = make_double2(0, 0);
+  for (int q = 0; q < splits; ++q) {
+    const double2 v = part[((size_t)(f * kRcsB + bs) * nd + d) * splits + q];
+    s.x += v.x;
+    s.y += v.y;
+  }
+  sig[((size_t)f * nb + b0 + bs) * nd + d] = fk[2 * f + 1] * (s.x * s.x + s.y * s.y);
 }
 
 int blocks_for(long long n) { return (int)std::min<long long>((n + kT - 1) / kT, 152LL * 16); }
@@ -154,9 +259,32 @@ void rcs_scale(aim_ctx* c, int nb, const RcsPhases& s, double2* acc) {
   AIM_CHECK_LAUNCH();
 }
 
+size_t rcs_workspace(const aim_ctx* c, int n_freq, int nd, int& nfc, int& splits) {
+  // frequencies per pass: at most 64 MB of face currents (at least one frequency)
+  const size_t per_f = (size_t)kRcsB * 4 * c->nt;
+  nfc = (int)std::max<size_t>(1, std::min<size_t>((size_t)n_freq, (size_t(64) << 20) / (per_f * sizeof(double2))));
+  // splits of the faces so that few directions still occupy every SM
+  splits = (int)std::max<long long>(1, std::min<long long>((c->nt + kT - 1) / kT, 608 / ((long long)nd * nfc)));
+  return per_f * nfc + (size_t)nfc * kRcsB * nd * splits;
+}
+
 void rcs_farfield(aim_ctx* c, int n_freq, int nb, const double2* spec, int nd, const double* dirs, const double* fk,
-                  double* sig) {
-  k_rcs<<<dim3(nd, nb, n_freq), kT, 0, c->stream>>>(c->nt, c->d_tbk, c->d_tbs, c->d_tbf, c->d_len, c->d_area,
-                                                      c->d_v, c->d_qp, c->d_qw, c->ns, nb, spec, fk, dirs, nd, sig);
-  AIM_CHECK_LAUNCH();
+                  double2* work, double* sig) {
+  int nfc, splits;
+  rcs_workspace(c, n_freq, nd, nfc, splits);
+  double2* part = work + (size_t)kRcsB * 4 * c->nt * nfc;
+  for (int f0 = 0; f0 < n_freq; f0 += nfc)
+    for (int b0 = 0; b0 < nb; b0 += kRcsB) {
+      const int nf = std::min(nfc, n_freq - f0), nbc = std::min(kRcsB, nb - b0);
+      k_rcs_faces<<<dim3((c->nt + kT - 1) / kT, nbc, nf), kT, 0, c->stream>>>(
+          c->nt, c->d_tri, c->d_tbk, c->d_tbs, c->d_tbf, c->d_len, c->d_area, c->d_v, c->ns, nb, b0,
+          spec + (size_t)f0 * nb * c->ns, work);
+      AIM_CHECK_LAUNCH();
+      k_rcs_dirs<<<dim3(nd, splits, nf), kT, 0, c->stream>>>(c->nt, c->d_tri, c->d_v, c->d_area, work, fk + 2 * f0,
+                                                             dirs, nbc, part);
+      AIM_CHECK_LAUNCH();
+      k_rcs_finish<<<dim3((nd + kT - 1) / kT, nbc, nf), kT, 0, c->stream>>>(nd, splits, nb, b0, fk + 2 * f0, part,
+                                                                            sig + (size_t)f0 * nb * nd);
+      AIM_CHECK_LAUNCH();
+    }
 }
