@@ -231,6 +231,8 @@ struct aim_ctx {
   double rmax = 0;             // largest vertex distance from the origin (bounds the time reach
                                // r.u / (c dt) of every cubature point)
 
+  double rwg_span = 0;         // largest distance between two vertices of one RWG's faces
+
   int* d_anchor = nullptr;     // [ns][3]
   int* d_order = nullptr;      // [ns] RWGs in Morton order of their anchors (interpolation visit order)
   double* d_lam = nullptr;     // [ns][4][64]  FP64 anterpolation rows
@@ -317,6 +319,8 @@ struct aim_ctx {
   GmresState gs;
   double2* adj_buf[5] = {nullptr, nullptr, nullptr, nullptr, nullptr};  // adjoint-helper staging
   size_t adj_cap[5] = {0, 0, 0, 0, 0};
+  double2* far_part = nullptr;  // partial sums of the far field
+  size_t far_cap = 0;
   ProfState prof;
   int l_done = 0, march_nb = 0;   // march state for aim_march_continue
   bool use_graphs = true;

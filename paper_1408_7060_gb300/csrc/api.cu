@@ -135,6 +135,16 @@ void setup_impl(aim_ctx* c, const aim_mesh* mesh, const aim_grid* grid, double n
   for (int i = 0; i < hm.nv; ++i)
     c->rmax = std::max(c->rmax, std::sqrt(hm.V[3 * i] * hm.V[3 * i] + hm.V[3 * i + 1] * hm.V[3 * i + 1] +
                                           hm.V[3 * i + 2] * hm.V[3 * i + 2]));
+  for (int k = 0; k < hm.ns; ++k) {
+    const int* e = &hm.edge[2 * k];
+    const int v[4] = {e[0], e[1], hm.rfree[2 * k], hm.rfree[2 * k + 1]};
+    for (int i = 0; i < 4; ++i)
+      for (int j = 0; j < i; ++j) {
+        const double *p = &hm.V[3 * v[i]], *q = &hm.V[3 * v[j]];
+        const double x = p[0] - q[0], y = p[1] - q[1], z = p[2] - q[2];
+        c->rwg_span = std::max(c->rwg_span, std::sqrt(x * x + y * y + z * z));
+      }
+  }
   c->h_edge = hm.edge;
   c->h_tri = hm.rtri;
   c->h_free = hm.rfree;

@@ -62,6 +62,43 @@ def d_basis(u, Q, dt, wc):
     return D / dt + 1j * wc * T
 
 
+# (subdivision, order, c dt in m, directions, steps, far times): the last two hold several
+# steps per RWG, one within the tap tables and one beyond them
+@pytest.mark.parametrize("sub,order,cdt,nd,steps,n_out", [(1, 2, 0.8, 1, 1, 3), (1, 3, 0.8, 5, 9, 70),
+                                                         (2, 1, 0.5, 17, 66, 20), (2, 4, 1.0, 4, 5, 64),
+                                                         (1, 2, 0.3, 6, 20, 40), (1, 3, 0.1, 3, 30, 50)])
+def test_far_field_and_adjoint(sub, order, cdt, nd, steps, n_out):
+    from paper_1408_7060_gb300 import abi
+
+    f_c, dt, n0 = 150e6, cdt / C0, -4
+    V, F, c = context(sub, order, dt, f_c)
+    with c:
+        r, wS = surface(c, V, F)
+        rh, e1 = random_plane_waves(nd, 2)
+        e2 = np.cross(rh, e1)
+        rng = np.random.default_rng(5)
+        I = rng.standard_normal((steps, c.ns)) + 1j * rng.standard_normal((steps, c.ns))
+        G_in = rng.standard_normal((n_out, nd, 2)) + 1j * rng.standard_normal((n_out, nd, 2))
+        got = abi.aim_farfield(c.handle, rh, e1, e2, I, n0, n_out)
+        adj = abi.aim_farfield_adjoint(c.handle, rh, e1, e2, steps, n0, G_in)
+        ref, radj = np.zeros_like(got), np.zeros_like(adj)
+        wc = 2 * math.pi * f_c
+        for d in range(nd):
+            rr = r @ rh[d]
+            ph = -MU0 / (4 * math.pi) * np.exp(1j * wc / C0 * rr)
+            taps = {}
+            for i in range(n_out):
+                for l in range(steps):
+                    s = n0 + i - (l + 1)
+                    if s not in taps:
+                        t = d_basis(s + rr / cdt, order, dt, wc) * ph
+                        taps[s] = np.stack([(t * (wS @ e1[d])).sum(1), (t * (wS @ e2[d])).sum(1)], 1)
+                    ref[i, d] += I[l] @ taps[s]
+                    radj[l] += taps[s].conj() @ G_in[i, d]
+    assert np.abs(got - ref).max() <= 1e-12 * np.abs(ref).max()
+    assert np.abs(adj - radj).max() <= 1e-12 * np.abs(radj).max()
+
+
 @pytest.mark.parametrize("sub,f_mhz,nb,nf,nd", [(1, 100.0, 1, 1, 1), (2, 300.0, 5, 2, 33), (1, 2000.0, 2, 3, 300)])
 def test_rcs(sub, f_mhz, nb, nf, nd):
     V, F, c = context(sub, 2, 0.8 / C0, 150e6)
