@@ -92,9 +92,13 @@ __device__ __forceinline__ double2 warp_sum_c(double2 v) {
   return make_double2(__shfl_sync(0xffffffffu, keep, 0), __shfl_sync(0xffffffffu, keep, 16));
 }
 
+// Rows per warp of the interpolation kernel (8 warps per block): 4, or 1 where 32 rows per
+// block would leave half of the SMs without one (480 unknowns: 60 blocks instead of 15).
+inline int interp_rows(int ns) { return ns >= 76 * 32 ? 4 : 1; }
+
 // Raw Krylov dots formed by the interpolation kernel of an Arnoldi step's operator:
 // d[b][i] = conj(vt_i) . y_b for i <= *jdev, y the kernel's output (Krylov slot j+1);
-// partials per block of 32 rows, summed by the last block of each RHS.
+// partials per block of 8 interp_rows rows, summed by the last block of each RHS.
 struct DotFuse {
   const double2* V = nullptr;  // Krylov basis; null: no dots
   long long vstride = 0;

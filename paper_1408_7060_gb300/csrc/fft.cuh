@@ -154,7 +154,7 @@ template <bool INV, class C> struct DFT<16, INV, C> {
       case 1: c = c1; s = s1; break;
       case 2: c = h; s = h; break;
       case 3: c = s1; s = c1; break;
-      case 4: c = 0; s = 1; break;
+      case 4: return rot_q<INV>(a);
       case 6: c = -h; s = h; break;
       case 9: c = -c1; s = -s1; break;
       default: c = 0; s = 0; break;
@@ -263,6 +263,10 @@ template <int R, bool INV, class C>
 __device__ __forceinline__ C mul_root(C a, int q) {
   using Rl = decltype(a.x);
   double c, s;  // cos, sin of 2 pi q / R
+  if (q % R == 0) return a;  // multiples of a quarter turn need no arithmetic
+  if (2 * (q % R) == R) return mkc(-a.x, -a.y);
+  if (4 * (q % R) == R) return rot_q<INV>(a);
+  if (4 * (q % R) == 3 * R) return rot_q<!INV>(a);
   if constexpr (R == 6) {
     const double h = 0.866025403784438646764;
     const int m = q % 6;
@@ -323,12 +327,108 @@ struct DFTL {
   }
 };
 
+// ---------------------------------------------------------------- butterflies with a zero / unused half
+template <bool INV, class C>
+__device__ __forceinline__ void dft4_half_in(C a, C b, C& x0, C& x1, C& x2, C& x3) {  // inputs (a, b, 0, 0)
+  const C r = rot_q<INV>(b);
+  x0 = a + b;
+  x1 = a + r;
+  x2 = a - b;
+  x3 = a - r;
+}
+template <int R, bool INV, class C>
+struct HalfDFT {
+  // v[0..R/2) in, v[0..R) out (the other inputs are zero)
+  __device__ __forceinline__ static void in(C* v) {
+    if constexpr (R == 4) {
+      dft4_half_in<INV>(v[0], v[1], v[0], v[1], v[2], v[3]);
+    } else if constexpr (R == 8) {
+      using Rl = decltype(v[0].x);
+      const Rl h = (Rl)0.70710678118654752440;
+      C e0, e1, e2, e3, o0, o1, o2, o3;
+      dft4_half_in<INV>(v[0], v[2], e0, e1, e2, e3);
+      dft4_half_in<INV>(v[1], v[3], o0, o1, o2, o3);
+      const C w1 = INV ? mkc(h * (o1.x - o1.y), h * (o1.x + o1.y)) : mkc(h * (o1.x + o1.y), h * (o1.y - o1.x));
+      const C w2 = rot_q<INV>(o2);
+      const C w3 = INV ? mkc(-h * (o3.x + o3.y), h * (o3.x - o3.y)) : mkc(h * (o3.y - o3.x), -h * (o3.x + o3.y));
+      v[0] = e0 + o0; v[4] = e0 - o0;
+      v[1] = e1 + w1; v[5] = e1 - w1;
+      v[2] = e2 + w2; v[6] = e2 - w2;
+      v[3] = e3 + w3; v[7] = e3 - w3;
+    } else {
+      static_assert(R == 16, "half-input radix");
+      C t[16];
+#pragma unroll
+      for (int n2 = 0; n2 < 4; ++n2) dft4_half_in<INV>(v[n2], v[4 + n2], t[n2], t[4 + n2], t[8 + n2], t[12 + n2]);
+#pragma unroll
+      for (int k1 = 0; k1 < 4; ++k1) {
+        C a0 = t[4 * k1], a1 = t[4 * k1 + 1], a2 = t[4 * k1 + 2], a3 = t[4 * k1 + 3];
+        if (k1) {
+          a1 = DFT<16, INV, C>::w16(a1, k1);
+          a2 = DFT<16, INV, C>::w16(a2, 2 * k1);
+          a3 = DFT<16, INV, C>::w16(a3, 3 * k1);
+        }
+        dft4<INV>(a0, a1, a2, a3);
+        v[k1] = a0;
+        v[k1 + 4] = a1;
+        v[k1 + 8] = a2;
+        v[k1 + 12] = a3;
+      }
+    }
+  }
+  // v[0..R) in, v[0..R/2) out (the other outputs are not needed)
+  __device__ __forceinline__ static void out(C* v) {
+    if constexpr (R == 4) {
+      const C s0 = v[0] + v[2], d0 = v[0] - v[2], s1 = v[1] + v[3], d1 = rot_q<INV>(v[1] - v[3]);
+      v[0] = s0 + s1;
+      v[1] = d0 + d1;
+    } else if constexpr (R == 8) {
+      using Rl = decltype(v[0].x);
+      const Rl h = (Rl)0.70710678118654752440;
+      dft4<INV>(v[0], v[2], v[4], v[6]);
+      dft4<INV>(v[1], v[3], v[5], v[7]);
+      const C o1 = v[3], o2 = v[5], o3 = v[7];
+      const C w1 = INV ? mkc(h * (o1.x - o1.y), h * (o1.x + o1.y)) : mkc(h * (o1.x + o1.y), h * (o1.y - o1.x));
+      const C w2 = rot_q<INV>(o2);
+      const C w3 = INV ? mkc(-h * (o3.x + o3.y), h * (o3.x - o3.y)) : mkc(h * (o3.y - o3.x), -h * (o3.x + o3.y));
+      const C e1 = v[2], e2 = v[4], e3 = v[6];
+      v[0] = v[0] + v[1];
+      v[1] = e1 + w1;
+      v[2] = e2 + w2;
+      v[3] = e3 + w3;
+    } else {
+      static_assert(R == 16, "half-output radix");
+#pragma unroll
+      for (int n2 = 0; n2 < 4; ++n2) dft4<INV>(v[n2], v[4 + n2], v[8 + n2], v[12 + n2]);
+      C t[8];
+#pragma unroll
+      for (int k1 = 0; k1 < 4; ++k1) {
+        C a0 = v[4 * k1], a1 = v[4 * k1 + 1], a2 = v[4 * k1 + 2], a3 = v[4 * k1 + 3];
+        if (k1) {
+          a1 = DFT<16, INV, C>::w16(a1, k1);
+          a2 = DFT<16, INV, C>::w16(a2, 2 * k1);
+          a3 = DFT<16, INV, C>::w16(a3, 3 * k1);
+        }
+        const C s0 = a0 + a2, d0 = a0 - a2, s1 = a1 + a3, d1 = rot_q<INV>(a1 - a3);
+        t[k1] = s0 + s1;
+        t[k1 + 4] = d0 + d1;
+      }
+#pragma unroll
+      for (int q = 0; q < 8; ++q) v[q] = t[q];
+    }
+  }
+};
+
 // Even radix R with only the first R/2 inputs non-zero (the pruned zero padding):
 //   X[2k] = DFT_{R/2}(x)[k],  X[2k+1] = DFT_{R/2}(x[n] W_R^n)[k],
 // two half-length butterflies instead of a full one fed with zeros.  v[0..R/2) in,
 // v[0..R) out in natural order.
 template <int R, int L, bool INV, class C>
 __device__ __forceinline__ void dft_half_in(C* v, const C* tw) {
+  if constexpr (R == 4 || R == 8 || R == 16) {  // the zeros drop out of the first butterflies
+    HalfDFT<R, INV, C>::in(v);
+    return;
+  }
   constexpr int H = R / 2;
   C e[H], o[H];
 #pragma unroll
@@ -350,6 +450,10 @@ __device__ __forceinline__ void dft_half_in(C* v, const C* tw) {
 // inputs.  v[0..R) in, v[0..R/2) out.
 template <int R, int L, bool INV, class C>
 __device__ __forceinline__ void dft_half_out(C* v, const C* tw) {
+  if constexpr (R == 4 || R == 8 || R == 16) {
+    HalfDFT<R, INV, C>::out(v);
+    return;
+  }
   constexpr int H = R / 2;
   C e[H], o[H];
 #pragma unroll

@@ -295,14 +295,17 @@ __device__ void finish_arrive(const FinishArgs& a, GmresState& s, int j, bool co
   if (!any && !*(volatile int*)(s.flag + 2) && a.use_cond) cudaGraphSetConditional(a.outer, 0u);
 }
 
-constexpr int kCgsSub = 64;       // elements per sub-chunk: 64 lanes x 4 groups of basis vectors
+// Elements per sub-chunk of an update block, SUB lanes x 256 / SUB groups of basis vectors: 64,
+// or 16 on small systems (below 32 elements per SM), so that their FP64 work reaches more than
+// a few SMs: 480 unknowns, 8 -> 30 blocks per update.
+constexpr int cgs_sub(int ns) { return ns >= 152 * 32 ? 64 : 16; }
 constexpr int kCgsMaxE = 2048;    // elements per block at most
 constexpr int kCgsTargetP = 256;  // blocks per RHS aimed at (the chunk grows beyond)
 
 struct CgsArgs {
   double2* V;
   long long vstride;
-  int ns, E, P;          // RHS length, elements per block (multiple of kCgsSub), blocks per RHS
+  int ns, E, P;          // RHS length, elements per block (multiple of SUB), blocks per RHS
   double2* pd1;          // raw dot partials of w (k_cgs_dots) [B][64][P]
   double2* d1;           // their sums: the first pass's dots [B][64]
   double2* pd2;          // first pass: raw dot partials of the updated w [B][64][P]
@@ -355,13 +358,13 @@ __global__ void __launch_bounds__(kThreads) k_cgs_dots(CgsArgs a, GmresState s) 
 
 // One classical Gram-Schmidt pass on slot j+1 of every active RHS, grid (P, nb):
 //   h_i = sig_i d_i (d_i = sum of the raw dots conj(vt_i) . w, block 0 stores h),
-//   w -= sum_i vt_i (sig_i h_i) on the block's E elements (64 at a time: 4 groups of
-//   threads take every 4th basis vector, group 0 sums and writes),
-// then for the first pass the raw dots of the updated w over the block's elements (warp y
-// takes i = y, y + 8, ...), summed over the P blocks by the last block of the RHS into
+//   w -= sum_i vt_i (sig_i h_i) on the block's E elements (SUB at a time: the 256 / SUB
+//   groups of threads take the basis vectors in turn, group 0 sums and writes),
+// then for the first pass the raw dots of the updated w over the block's elements (a warp
+// takes one basis vector at a time, or two where SUB = 16), summed over the P blocks by the last block of the RHS into
 // d2 -- the second pass's d; for the second pass |w|^2 over the block, summed by the last
 // block, which then finishes column j (finish_rhs) and arrives at the step's counter.
-template <int PASS>
+template <int PASS, int SUB>
 __global__ void __launch_bounds__(kThreads) k_cgs(CgsArgs a, FinishArgs f, GmresState s) {
   pdl_wait();
   const int b = blockIdx.y, blk = blockIdx.x, tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
@@ -371,7 +374,8 @@ __global__ void __launch_bounds__(kThreads) k_cgs(CgsArgs a, FinishArgs f, Gmres
     return;
   }
   __shared__ double2 coef[64];
-  __shared__ double2 red[4][kCgsSub];
+  constexpr int GR = kThreads / SUB;
+  __shared__ double2 red[GR][SUB];
   __shared__ double2 wsm[kCgsMaxE];
   __shared__ double nrd[kThreads / 32];
   __shared__ int last;
@@ -389,13 +393,13 @@ __global__ void __launch_bounds__(kThreads) k_cgs(CgsArgs a, FinishArgs f, Gmres
   const double2* Vb = a.V + (size_t)b * a.ns;
   double2* w = a.V + (size_t)J * a.vstride + (size_t)b * a.ns;
   const int n0 = blk * a.E, cnt = min(a.ns, n0 + a.E) - n0;
-  const int e = tid & (kCgsSub - 1), grp = tid / kCgsSub;
-  for (int s0 = 0; s0 < cnt; s0 += kCgsSub) {
+  const int e = tid % SUB, grp = tid / SUB;
+  for (int s0 = 0; s0 < cnt; s0 += SUB) {
     const int n = n0 + s0 + e;
     const bool in = s0 + e < cnt;
     double2 pv = make_double2(0, 0);
     if (in)
-      for (int i = grp; i < J; i += 4) {
+      for (int i = grp; i < J; i += GR) {
         const double2 v = cmul(Vb[i * a.vstride + n], coef[i]);
         pv.x += v.x;
         pv.y += v.y;
@@ -404,8 +408,14 @@ __global__ void __launch_bounds__(kThreads) k_cgs(CgsArgs a, FinishArgs f, Gmres
     __syncthreads();
     if (grp == 0 && in) {
       double2 wv = w[n];
-      wv.x -= (red[0][e].x + red[1][e].x) + (red[2][e].x + red[3][e].x);
-      wv.y -= (red[0][e].y + red[1][e].y) + (red[2][e].y + red[3][e].y);
+      double2 q = make_double2(0, 0);
+#pragma unroll
+      for (int g = 0; g < GR; g += 4) {
+        q.x += (red[g][e].x + red[g + 1][e].x) + (red[g + 2][e].x + red[g + 3][e].x);
+        q.y += (red[g][e].y + red[g + 1][e].y) + (red[g + 2][e].y + red[g + 3][e].y);
+      }
+      wv.x -= q.x;
+      wv.y -= q.y;
       w[n] = wv;
       if (PASS == 1 && a.wf) a.wf[(size_t)b * a.ns + n] = make_float2((float)wv.x, (float)wv.y);
       wsm[s0 + e] = wv;
@@ -413,16 +423,26 @@ __global__ void __launch_bounds__(kThreads) k_cgs(CgsArgs a, FinishArgs f, Gmres
     __syncthreads();
   }
   if (PASS == 0) {
-    for (int i = warp; i < J; i += kThreads / 32) {
-      const double2* vi = Vb + i * a.vstride + n0;
+    constexpr int W = SUB < 32 ? SUB : 32, NI = 32 / W;  // lanes per basis vector
+    for (int i0 = warp * NI; i0 < J; i0 += kThreads / 32 * NI) {
+      const int i = i0 + lane / W;
       double2 t = make_double2(0, 0);
-      for (int q = lane; q < cnt; q += 32) {
-        const double2 p = cmulc(vi[q], wsm[q]);
-        t.x += p.x;
-        t.y += p.y;
+      if (i < J) {
+        const double2* vi = Vb + i * a.vstride + n0;
+        for (int q = lane % W; q < cnt; q += W) {
+          const double2 p = cmulc(vi[q], wsm[q]);
+          t.x += p.x;
+          t.y += p.y;
+        }
       }
-      t = warp_sum_c(t);
-      if (lane == 0) a.pd2[((size_t)b * 64 + i) * a.P + blk] = t;
+      // (real parts to the first half of the lanes, imaginary to the second)
+      const bool hi = lane & (W / 2);
+      double u = hi ? t.y : t.x;
+      u += __shfl_xor_sync(0xffffffffu, hi ? t.x : t.y, W / 2);
+#pragma unroll
+      for (int o = W / 4; o > 0; o >>= 1) u += __shfl_xor_sync(0xffffffffu, u, o);
+      const double im = __shfl_down_sync(0xffffffffu, u, W / 2);
+      if (lane % W == 0 && i < J) a.pd2[((size_t)b * 64 + i) * a.P + blk] = make_double2(u, im);
     }
   } else {
     double t = 0;
@@ -713,9 +733,11 @@ void arnoldi_step(aim_ctx* c, int nb, double tol, bool use_cond, cudaGraphCondit
   if (s.interp_P == 0)
     AIM_KLAUNCH(c, AIM_K_GMRES_DOT, launch_pdl(st, dim3(s.cgs_P, nb), dim3(kThreads), 0, k_cgs_dots, a, s));
   AIM_KLAUNCH(c, AIM_K_GMRES_UPDATE,
-              launch_pdl(st, dim3(s.cgs_P, nb), dim3(kThreads), 0, k_cgs<0>, a, f, s));
+              launch_pdl(st, dim3(s.cgs_P, nb), dim3(kThreads), 0, cgs_sub(ns) == 64 ? k_cgs<0, 64> : k_cgs<0, 16>, a,
+                         f, s));
   AIM_KLAUNCH(c, AIM_K_GMRES_UPDATE,
-              launch_pdl(st, dim3(s.cgs_P, nb), dim3(kThreads), 0, k_cgs<1>, a, f, s));
+              launch_pdl(st, dim3(s.cgs_P, nb), dim3(kThreads), 0, cgs_sub(ns) == 64 ? k_cgs<1, 64> : k_cgs<1, 16>, a,
+                         f, s));
 }
 
 void cycle_epilogue(aim_ctx* c, int nb, double2* x) {
@@ -868,15 +890,16 @@ void gmres_alloc(aim_ctx* c) {
   s.its = (int*)aim_alloc(c, B * sizeof(int));
   s.jdev = (int*)aim_alloc(c, sizeof(int));
   s.flag = (int*)aim_alloc(c, 3 * sizeof(int));
-  // CGS update blocks: E elements each (a multiple of 64), about kCgsTargetP per RHS
-  s.cgs_E = std::min(kCgsMaxE, std::max(kCgsSub, ((ns + kCgsTargetP - 1) / kCgsTargetP + kCgsSub - 1) / kCgsSub * kCgsSub));
+  // CGS update blocks: E elements each (a multiple of SUB), at most about kCgsTargetP per RHS
+  const int sub = cgs_sub(ns);
+  s.cgs_E = std::min(kCgsMaxE, std::max(sub, ((ns + kCgsTargetP - 1) / kCgsTargetP + sub - 1) / sub * sub));
   s.cgs_P = (ns + s.cgs_E - 1) / s.cgs_E;
   s.pu = (double*)aim_alloc(c, (size_t)B * s.cgs_P * sizeof(double));
   s.pd = (double2*)aim_alloc(c, (size_t)B * 64 * s.cgs_P * sizeof(double2));
   s.d1 = (double2*)aim_alloc(c, (size_t)B * 64 * sizeof(double2));
-  // the interpolation kernel forms the first pass's dots when its blocks of 32 rows are
-  // few enough for one block to sum their partials
-  const int pi = (ns + 31) / 32;
+  // the interpolation kernel forms the first pass's dots when its blocks are few enough for
+  // one block to sum their partials
+  const int br = 8 * interp_rows(ns), pi = (ns + br - 1) / br;
   s.interp_P = pi <= 1024 ? pi : 0;
   if (s.interp_P) s.pdi = (double2*)aim_alloc(c, (size_t)B * 64 * s.interp_P * sizeof(double2));
   s.pd2 = (double2*)aim_alloc(c, (size_t)B * 64 * s.cgs_P * sizeof(double2));

@@ -41,23 +41,13 @@ __host__ __device__ constexpr int x_pitch(int L, int yb) {
   while (p % 16 != (yb >= 16 ? 1 : yb == 1 ? 0 : 16 / yb)) ++p;
   return p;
 }
-template <int R, int L, bool INV, class C>
-__device__ __forceinline__ void half_in(C* v, const C* tw) {
-  if constexpr (R <= 16 && (R & (R - 1)) == 0) HalfDFT<R, INV, C>::in(v);
-  else dft_half_in<R, L, INV, C>(v, tw);
-}
-template <int R, int L, bool INV, class C>
-__device__ __forceinline__ void half_out(C* v, const C* tw) {
-  if constexpr (R <= 16 && (R & (R - 1)) == 0) HalfDFT<R, INV, C>::out(v);
-  else dft_half_out<R, L, INV, C>(v, tw);
-}
-
 // S_c[n] = sum_k L_c[n,k] x_k gathered node by node (the transpose of the interpolation
 // rows), then the forward x-FFT of each grid row.  One block holds the 4 components of YB
 // consecutive rows y of one plane z for BB right-hand sides.  Only the nodes some stencil
 // touches are visited (arow: their range per box row, anode: y N + x, aptr: their CSR
 // entries); the operator input is interleaved, xs[k][b], so the BB lanes of a node share
-// its coefficients and gather adjacent values.  KXM stores the kx-major grid of the plane
+// its coefficients and gather adjacent values.  With one right-hand side 4 lanes share a
+// node's entries instead (each is an index, coefficient, gather chain).  KXM stores the kx-major grid of the plane
 // kernel, A[b][c][kx][z][y - ylo] (rows beyond the box written as zeros up to N), runs of
 // YB values; otherwise A[b][c][z][y][kx].
 template <int L, int YB, int BB, bool KXM, class C>
@@ -79,25 +69,27 @@ __global__ void __launch_bounds__(256) k_anterp(const int* __restrict__ arow, co
   __syncthreads();
   const int ye = min(y0 + YB, nyb);
   if (y0 < nyb) {
-    const int k0 = arow[z * nyb + y0], items = (arow[z * nyb + ye] - k0) * BB;
-    for (int i = threadIdx.x; i < items; i += 256) {
-      const int bs = i % BB, k = k0 + i / BB, b = b0 + bs;
-      if (BB > 1 && (b >= nb || (active && !active[b]))) continue;
+    constexpr int EL = BB == 1 ? 4 : 1;  // lanes per node
+    const int k0 = arow[z * nyb + y0], items = (arow[z * nyb + ye] - k0) * (BB * EL);
+    // (whole warps run every round, for the sums over the lanes of a node)
+    for (int i = threadIdx.x; i - (int)(threadIdx.x & 31) < items; i += 256) {
+      const int bs = i % BB, k = min(k0 + i / (BB * EL), k0 + items / (BB * EL) - 1), b = b0 + bs;
+      const bool on = i < items && (BB == 1 || (b < nb && !(active && !active[b])));
       const int nd = anode[k], yy = nd / N - ylo - y0, x = nd % N;
       const C* vb = xs + b;
       C a0{}, a1{}, a2{}, a3{};
-      int e = aptr[k];
-      const int e1 = aptr[k + 1];
+      int e = on ? aptr[k] + (EL > 1 ? i % EL : 0) : 0;
+      const int e1 = on ? aptr[k + 1] : 0;
       // four entries at a time: their index and coefficient loads, then their gathers of
       // x, are independent and in flight together (the sums keep the entry order)
-      for (; e + 4 <= e1; e += 4) {
+      for (; e + 3 * EL < e1; e += 4 * EL) {
         int j[4];
         typename Real<C>::F4 w[4];
         C xv[4];
 #pragma unroll
         for (int u = 0; u < 4; ++u) {
-          j[u] = nidx[e + u];
-          w[u] = ncoef[e + u];
+          j[u] = nidx[e + u * EL];
+          w[u] = ncoef[e + u * EL];
         }
 #pragma unroll
         for (int u = 0; u < 4; ++u) xv[u] = vb[(size_t)j[u] * nb];
@@ -109,7 +101,7 @@ __global__ void __launch_bounds__(256) k_anterp(const int* __restrict__ arow, co
           a3 += (R)w[u].w * xv[u];
         }
       }
-      for (; e < e1; ++e) {
+      for (; e < e1; e += EL) {
         const typename Real<C>::F4 w = ncoef[e];
         const C xv = vb[(size_t)nidx[e] * nb];
         a0 += (R)w.x * xv;
@@ -117,6 +109,22 @@ __global__ void __launch_bounds__(256) k_anterp(const int* __restrict__ arow, co
         a2 += (R)w.z * xv;
         a3 += (R)w.w * xv;
       }
+      if constexpr (EL == 4) {  // lane q of the four keeps component q
+        const bool hi = i & 2, od = i & 1;
+        C u0 = hi ? a2 : a0, u1 = hi ? a3 : a1;
+        const C s0 = hi ? a0 : a2, s1 = hi ? a1 : a3;
+        u0.x += __shfl_xor_sync(0xffffffffu, s0.x, 2);
+        u0.y += __shfl_xor_sync(0xffffffffu, s0.y, 2);
+        u1.x += __shfl_xor_sync(0xffffffffu, s1.x, 2);
+        u1.y += __shfl_xor_sync(0xffffffffu, s1.y, 2);
+        C t = od ? u1 : u0;
+        const C s = od ? u0 : u1;
+        t.x += __shfl_xor_sync(0xffffffffu, s.x, 1);
+        t.y += __shfl_xor_sync(0xffffffffu, s.y, 1);
+        if (on) in[((i & 3) * YB + yy) * N + x] = t;
+        continue;
+      }
+      if (!on) continue;
       C* t = in + (bs * 4 * YB + yy) * N + x;
       t[0] = a0;
       t[YB * N] = a1;
@@ -130,7 +138,7 @@ __global__ void __launch_bounds__(256) k_anterp(const int* __restrict__ arow, co
     C v[R1];
 #pragma unroll
     for (int n1 = 0; n1 < R1 / 2; ++n1) v[n1] = in[row * N + R2 * n1 + n2];
-    half_in<R1, L, false, C>(v, tw);
+    dft_half_in<R1, L, false, C>(v, tw);
 #pragma unroll
     for (int k1 = 0; k1 < R1; ++k1) tmp[row * PX + k1 * (R2 + 1) + n2] = k1 ? v[k1] * tw[n2 * k1] : v[k1];
   }
@@ -194,7 +202,7 @@ __global__ void __launch_bounds__(256) k_xinv(const C* __restrict__ A, C* __rest
     C v[R2];
 #pragma unroll
     for (int n2 = 0; n2 < R2; ++n2) v[n2] = tmp[yy * PX + k1 * (R2 + 1) + n2];
-    half_out<R2, L, true, C>(v, tw);
+    dft_half_out<R2, L, true, C>(v, tw);
     if (y0 + yy < nyb)
 #pragma unroll
       for (int k2 = 0; k2 < R2 / 2; ++k2) dst[(size_t)yy * N + k1 + R1 * k2] = v[k2];
@@ -779,17 +787,17 @@ __global__ void __launch_bounds__(kZThreads) k_zrhs_2s(SlabList sl, const C* __r
 
 // ---------------------------------------------------------------- stage iii + iv
 // y_k = sign * ( sum_c sum_{n in stencil(k)} L_c[n,k] P_c[n]  +  sum_terms Z~near_m x_m ) + base_k
-// Grid (nb, ceil(ns / 32)): a block takes 32 rows of one RHS, one warp per kInterpRows
-// consecutive rows.  Grid part: the whole warp per row, accumulated in the grid precision.
-// Near part: 8 lanes per row, all rows at once, in FP64 -- the warp's FP64 instructions
-// (each holds the sub-partition's FP64 pipe for the whole warp) serve kInterpRows rows
-// instead of one.  With df.V set (the operator of an Arnoldi step, y = Krylov slot j+1)
-// the block also forms the raw dots conj(vt_i) . y over its 32 rows for i <= j, and the
-// last block of the RHS sums them into df.d.
-constexpr int kInterpRows = 4;
-constexpr int kInterpBlockRows = 8 * kInterpRows;  // 256 threads
-
-template <class C>
+// Grid (nb, row blocks): a warp takes ROWS consecutive rows of one RHS, a block the rows of
+// its 8 warps: 4 rows per warp, or 1 on small systems, whose FP64 work would otherwise sit on
+// a few SMs (interp_rows).  Grid part: the whole warp per row, accumulated in the grid
+// precision, the rows' sums reduced together.  Near part: 32 / ROWS lanes per row, all rows
+// at once, in FP64 -- the warp's FP64 instructions (each holds the FP64 pipe for the whole
+// warp) serve ROWS rows.  With df.V set (the operator of an Arnoldi step, y = Krylov slot
+// j+1) the block also forms the raw dots conj(vt_i) . y over its rows for i <= j, 32 / rows
+// of them per warp instruction, and the last block of the RHS sums them into df.d.
+// Measured, us per product: 480 unknowns, complex128, 16.3 -> 8.1 (15 blocks before);
+// 64 right-hand sides of 7680 unknowns, complex64, 334 -> 262.
+template <class C, int ROWS>
 __global__ void __launch_bounds__(256, 3) k_interp_near(const C* __restrict__ P, const int* __restrict__ anchor,
                                                      const int* __restrict__ order,
                                                      const typename Real<C>::T* __restrict__ lam, int N, int nz,
@@ -799,92 +807,134 @@ __global__ void __launch_bounds__(256, 3) k_interp_near(const C* __restrict__ P,
                                                      const double2* __restrict__ base, double sign,
                                                      const int* __restrict__ active, double2* __restrict__ y,
                                                      VecSel ys, DotFuse df) {
-  pdl_wait();
   using R = typename Real<C>::T;
   // the right-hand side is the fastest grid index: the blocks of all right-hand sides
   // for one set of rows run together and share that set's near-zone rows through L2
   const int b = blockIdx.x, rb = blockIdx.y, warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  if (active && !active[b]) return;
-  const int k0 = rb * kInterpBlockRows + warp * kInterpRows;  // the warp's first position
-  // grid part, row by row; lane group r (lanes 8r .. 8r+7) keeps row r's sum
-  C mine{};
-  if (P) {
-    const size_t N3 = (size_t)nz * N * N;  // the box planes z0 .. z0 + nz - 1
-    // the warp's RWGs and their stencil origins first, so that the potential gathers of
-    // all kInterpRows RWGs depend on no further load and can be in flight together
-    int kr[kInterpRows];
-    size_t org[kInterpRows];
+  constexpr int brows = 8 * ROWS, GL = 32 / ROWS;  // rows per block, lanes per row of the near part
+  const int k0 = rb * brows + warp * ROWS;  // the warp's first position
+  // set-up tables first: they do not depend on the previous kernel
+  int kr[ROWS];
+  size_t org[ROWS];
 #pragma unroll
-    for (int r = 0; r < kInterpRows; ++r) kr[r] = k0 + r < ns ? order[k0 + r] : -1;
+  for (int r = 0; r < ROWS; ++r) kr[r] = k0 + r < ns ? order[k0 + r] : -1;
 #pragma unroll
-    for (int r = 0; r < kInterpRows; ++r) {
-      const int k = kr[r] < 0 ? 0 : kr[r];
-      org[r] = ((size_t)(anchor[3 * k + 2] - zlo) * N + anchor[3 * k + 1]) * N + anchor[3 * k];
-    }
-#pragma unroll
-    for (int r = 0; r < kInterpRows; ++r) {
-      C g{};
-      if (kr[r] >= 0) {
-        const int k = kr[r];
-        // 4 lanes per stencil row: lane -> (row of 8, dx); the 256 (component, node)
-        // terms of an RWG take 8 warp loads of 8 rows x 32 B each
-        const C* Pb = P + (size_t)b * 4 * N3 + org[r] + (lane & 3);
-        const R* lk = lam + (size_t)k * 256 + lane;
-#pragma unroll
-        for (int it = 0; it < 8; ++it) {
-          const int q = it * 8 + (lane >> 2);  // (component, row) pair, 0..63
-          const int c = q >> 4, row = q & 15;
-          const int dz = row >> 2, dy = row & 3;
-          g += lk[it * 32] * Pb[c * N3 + ((size_t)dz * N + dy) * N];
-        }
-      }
-      for (int o = 16; o > 0; o >>= 1) {
-        g.x += __shfl_xor_sync(0xffffffffu, g.x, o);
-        g.y += __shfl_xor_sync(0xffffffffu, g.y, o);
-      }
-      if ((lane >> 3) == r) mine = g;
-    }
+  for (int r = 0; r < ROWS; ++r) {
+    const int k = kr[r] < 0 ? 0 : kr[r];
+    org[r] = ((size_t)(anchor[3 * k + 2] - zlo) * N + anchor[3 * k + 1]) * N + anchor[3 * k];
   }
   // near part: lane group r, sub-lane sl
-  const int r = lane >> 3, sl = lane & 7;
-  const bool on = k0 + r < ns;
-  const int k = on ? order[k0 + r] : 0;
-  long long xoff = 0;
-  double xscale = 1.0;
-  if (nl.xsel.sel) {
-    const int jj = *nl.xsel.sel + nl.xsel.off;
-    xoff = jj * nl.xsel.stride;
-    if (nl.xsel.scale) xscale = nl.xsel.scale[b * 64 + jj];
-  }
-  double2 nr = make_double2(0, 0);
-  if (on) {
-    for (int e = rowptr[k] + sl; e < rowptr[k + 1]; e += 8) {
-      const int j = col[e];
-      for (int t = 0; t < nl.n; ++t) {
-        const double2 z = nl.val[t][e];
-        double2 xv = nl.x[t][xoff + (size_t)b * ns + j];
-        if (nl.dinv) {
-          const double2 d = nl.dinv[j];
-          xv = make_double2(xv.x * d.x - xv.y * d.y, xv.x * d.y + xv.y * d.x);
+  const int r = lane / GL, sl = lane % GL;
+  int k = kr[0];
+#pragma unroll
+  for (int q = 1; q < ROWS; ++q) k = r == q ? kr[q] : k;
+  const bool on = k >= 0;
+  int e = on ? rowptr[k] + sl : 0;
+  const int e1 = on ? rowptr[k + 1] : 0;
+  constexpr int U = ROWS == 4 ? 4 : 2;  // entries of a lane in flight
+  int j[U];
+#pragma unroll
+  for (int u = 0; u < U; ++u) j[u] = e + GL * u < e1 ? col[e + GL * u] : -1;
+  pdl_wait();
+  if (active && !active[b]) return;
+  // grid part, row by row
+  C g[ROWS];
+  if (P) {
+    const size_t N3 = (size_t)nz * N * N;  // the box planes z0 .. z0 + nz - 1
+#pragma unroll
+    for (int q = 0; q < ROWS; ++q) {
+      g[q] = C{};
+      if (kr[q] >= 0) {
+        // 4 lanes per stencil row: lane -> (row of 8, dx); the 256 (component, node)
+        // terms of an RWG take 8 warp loads of 8 rows x 32 B each
+        const C* Pb = P + (size_t)b * 4 * N3 + org[q] + (lane & 3);
+        const R* lk = lam + (size_t)kr[q] * 256 + lane;
+#pragma unroll
+        for (int it = 0; it < 8; ++it) {
+          const int p = it * 8 + (lane >> 2);  // (component, row) pair, 0..63
+          const int c = p >> 4, row = p & 15;
+          const int dz = row >> 2, dy = row & 3;
+          g[q] += lk[it * 32] * Pb[c * N3 + ((size_t)dz * N + dy) * N];
         }
-        nr.x += z.x * xv.x - z.y * xv.y;
-        nr.y += z.x * xv.y + z.y * xv.x;
       }
     }
   }
-  // sum over the 8 lanes of a group: the first exchange splits real (sl < 4) and
-  // imaginary (sl >= 4) parts, so 3 FP64 additions cover both
-  const bool hi = sl & 4;
+  double2 nr = make_double2(0, 0);
+  double xscale = 1.0;
+  {
+    long long xoff = 0;
+    if (nl.xsel.sel) {
+      const int jj = *nl.xsel.sel + nl.xsel.off;
+      xoff = jj * nl.xsel.stride;
+      if (nl.xsel.scale) xscale = nl.xsel.scale[b * 64 + jj];
+    }
+    xoff += (size_t)b * ns;
+    if (nl.n)
+      for (;;) {
+        for (int t = 0; t < nl.n; ++t) {
+          const double2* val = nl.val[t];
+          const double2* x = nl.x[t] + xoff;
+          double2 z[U], xv[U];
+#pragma unroll
+          for (int u = 0; u < U; ++u) {
+            z[u] = j[u] >= 0 ? val[e + GL * u] : make_double2(0, 0);
+            xv[u] = j[u] >= 0 ? x[j[u]] : make_double2(0, 0);
+          }
+#pragma unroll
+          for (int u = 0; u < U; ++u)
+            if (j[u] >= 0) {
+              if (nl.dinv) {
+                const double2 d = nl.dinv[j[u]];
+                xv[u] = make_double2(xv[u].x * d.x - xv[u].y * d.y, xv[u].x * d.y + xv[u].y * d.x);
+              }
+              nr.x += z[u].x * xv[u].x - z[u].y * xv[u].y;
+              nr.y += z[u].x * xv[u].y + z[u].y * xv[u].x;
+            }
+        }
+        e += GL * U;
+        if (__all_sync(0xffffffffu, e - sl >= e1)) break;
+#pragma unroll
+        for (int u = 0; u < U; ++u) j[u] = e + GL * u < e1 ? col[e + GL * u] : -1;
+      }
+  }
+  // Sums over lanes, real and imaginary parts split between lane halves.  Grid part: the 8
+  // values of 4 rows reduce together, lane group r keeping row r (9 additions instead of 40);
+  // then within a group real (first half) and imaginary (second half) parts.
+  const bool hi = sl & (GL / 2);
+  double grid = 0.0;
+  if (P) {
+    C t;
+    if constexpr (ROWS == 4) {
+      const bool h4 = lane & 16, h3 = lane & 8;
+      const C s0 = h4 ? g[0] : g[2], s1 = h4 ? g[1] : g[3];
+      C a0 = h4 ? g[2] : g[0], a1 = h4 ? g[3] : g[1];
+      a0.x += __shfl_xor_sync(0xffffffffu, s0.x, 16);
+      a0.y += __shfl_xor_sync(0xffffffffu, s0.y, 16);
+      a1.x += __shfl_xor_sync(0xffffffffu, s1.x, 16);
+      a1.y += __shfl_xor_sync(0xffffffffu, s1.y, 16);
+      const C s = h3 ? a0 : a1;
+      t = h3 ? a1 : a0;
+      t.x += __shfl_xor_sync(0xffffffffu, s.x, 8);
+      t.y += __shfl_xor_sync(0xffffffffu, s.y, 8);
+    } else {
+      t = g[0];
+    }
+    R kp = hi ? t.y : t.x;
+    kp += __shfl_xor_sync(0xffffffffu, hi ? t.x : t.y, GL / 2);
+#pragma unroll
+    for (int o = GL / 4; o > 0; o >>= 1) kp += __shfl_xor_sync(0xffffffffu, kp, o);
+    grid = (double)kp;
+  }
   double keep = hi ? nr.y : nr.x;
-  keep += __shfl_xor_sync(0xffffffffu, hi ? nr.x : nr.y, 4);
-  keep += __shfl_xor_sync(0xffffffffu, keep, 2);
-  keep += __shfl_xor_sync(0xffffffffu, keep, 1);
-  const double nim = __shfl_down_sync(0xffffffffu, keep, 4);
+  keep += __shfl_xor_sync(0xffffffffu, hi ? nr.x : nr.y, GL / 2);
+#pragma unroll
+  for (int o = GL / 4; o > 0; o >>= 1) keep += __shfl_xor_sync(0xffffffffu, keep, o);
+  keep = grid + xscale * keep;
+  const double nim = __shfl_down_sync(0xffffffffu, keep, GL / 2);
   double2 out = make_double2(0, 0);
   if (on && sl == 0) {
     if (ys.sel) y += (*ys.sel + ys.off) * ys.stride;
-    const double re = (double)mine.x + xscale * keep, im = (double)mine.y + xscale * nim;
-    out = make_double2(sign * re, sign * im);
+    out = make_double2(sign * keep, sign * nim);
     if (base) {
       const double2 bb = base[(size_t)b * ns + k];
       out = make_double2(bb.x + out.x, bb.y + out.y);
@@ -892,22 +942,32 @@ __global__ void __launch_bounds__(256, 3) k_interp_near(const C* __restrict__ P,
     y[(size_t)b * ns + k] = out;
   }
   if (df.V) {
-    __shared__ double2 wsm[kInterpBlockRows];
+    __shared__ double2 wsm[brows];
     __shared__ int last;
-    if (sl == 0) wsm[warp * kInterpRows + r] = out;  // zero for rows past ns
+    if (sl == 0) wsm[warp * ROWS + r] = out;  // zero for rows past ns
     __syncthreads();
     const int J = *df.jdev + 1;
-    const int pb = rb * kInterpBlockRows + lane;
-    const int kb = pb < ns ? order[pb] : 0;
+    constexpr int NI = 32 / brows;  // dots per warp instruction
+    const int row = lane % brows, pb = rb * brows + row;
+    const bool in = pb < ns;
+    const int kb = in ? order[pb] : 0;
     const double2* Vb = df.V + (size_t)b * ns;
-    for (int i = warp; i < J; i += 8) {
+    const double2 w = wsm[row];
+    for (int i0 = warp * NI; i0 < J; i0 += 8 * NI) {
+      const int i = i0 + lane / brows;
       double2 t = make_double2(0, 0);
-      if (pb < ns) {
-        const double2 v = Vb[i * df.vstride + kb], w = wsm[lane];
+      if (in && i < J) {
+        const double2 v = Vb[i * df.vstride + kb];
         t = make_double2(v.x * w.x + v.y * w.y, v.x * w.y - v.y * w.x);  // conj(v) w
       }
-      t = warp_sum_c(t);
-      if (lane == 0) df.pd[((size_t)b * 64 + i) * df.P + rb] = t;
+      // real parts end in the first half of a row group, imaginary in the second
+      const bool h = lane & (brows / 2);
+      double s = h ? t.y : t.x;
+      s += __shfl_xor_sync(0xffffffffu, h ? t.x : t.y, brows / 2);
+#pragma unroll
+      for (int o = brows / 4; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
+      const double im = __shfl_down_sync(0xffffffffu, s, brows / 2);
+      if (row == 0 && i < J) df.pd[((size_t)b * 64 + i) * df.P + rb] = make_double2(s, im);
     }
     __syncthreads();
     if (threadIdx.x == 0) {
@@ -1211,12 +1271,13 @@ struct GridOps {
   static void interp(aim_ctx* c, int nb, const C* P, const NearList& nl, const double2* base, double sign,
                      const int* active, double2* y, VecSel ys = VecSel()) {
     KScope ks(c, AIM_K_INTERP_NEAR);
-    const unsigned nrb = (unsigned)((c->ns + kInterpBlockRows - 1) / kInterpBlockRows);
+    const int br = 8 * interp_rows(c->ns);
+    const unsigned nrb = (unsigned)((c->ns + br - 1) / br);
     if (nrb > 65535u) throw AimError{AIM_ERR_ARG, "interpolation: more than 2 097 120 RWGs"};
-    launch_pdl(c->stream, dim3((unsigned)nb, nrb), dim3(256),
-               0, k_interp_near<C>, P, (const int*)c->d_anchor, (const int*)c->d_order, lam(c), c->N, c->NZ,
-               c->box_lo[2], c->ns, nb,
-               (const int*)c->d_rowptr, (const int*)c->d_col, nl, base, sign, active, y, ys, c->dotfuse);
+    launch_pdl(c->stream, dim3((unsigned)nb, nrb), dim3(256), 0,
+               interp_rows(c->ns) == 4 ? k_interp_near<C, 4> : k_interp_near<C, 1>, P, (const int*)c->d_anchor,
+               (const int*)c->d_order, lam(c), c->N, c->NZ, c->box_lo[2], c->ns, nb, (const int*)c->d_rowptr,
+               (const int*)c->d_col, nl, base, sign, active, y, ys, c->dotfuse);
   }
 
   // size of one kernel-spectrum octant [LZ/2 + 1][N + 1][N + 1]
