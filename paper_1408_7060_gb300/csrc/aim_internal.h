@@ -301,6 +301,9 @@ struct aim_ctx {
   bool ring_tma = false;
   int* d_err = nullptr;        // device error flag (a bounded wait gave up)
   void* d_xs = nullptr;        // [ns][nb] prepared operator input, grid precision (nb of the call)
+  void* d_Ab = nullptr;        // kx-major grids and inputs of up to batch_cap vectors: several delays
+  void* d_xsb = nullptr;       // of aim_rhs in one launch of each pass (null: one at a time)
+  int batch_cap = 0;
   double2* d_xd = nullptr;     // [B][ns] prepared operator input, FP64 (near zone)
   DotFuse dotfuse;             // set by the Arnoldi step around its operator application
   float2* d_vf = nullptr;      // [B][ns] complex64 copy of the Krylov vector the next SAI application

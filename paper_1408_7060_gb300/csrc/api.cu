@@ -63,6 +63,8 @@ T* upload(aim_ctx* c, const std::vector<T>& v) {
   return d;
 }
 
+constexpr size_t kBatchBytes = size_t(64) << 20;  // x-transformed grids of a batch of delays
+
 size_t grid_elem(const aim_ctx* c) { return c->precision == AIM_C64 ? sizeof(float2) : sizeof(double2); }
 
 // z transform length for nz box planes: the shortest length of the z pass >= 2 nz (at most
@@ -214,6 +216,15 @@ void setup_impl(aim_ctx* c, const aim_mesh* mesh, const aim_grid* grid, double n
   c->d_A = aim_alloc(c, grid_a_elems(c, B) * es);
   c->d_Bf = aim_alloc(c, grid_bf_elems(c, B) * es);
   c->d_P = aim_alloc(c, grid_p_elems(c, B) * es);
+  if (op_plane(c)) {
+    const size_t per = grid_a_elems(c, 1) * es;
+    const int cap = (int)std::min<size_t>((size_t)ng * B, kBatchBytes / per);
+    if (cap >= 2 * B || (B == 1 && cap >= 2)) {
+      c->d_Ab = aim_alloc(c, cap * per);
+      c->d_xsb = aim_alloc(c, (size_t)cap * ns * es);
+      c->batch_cap = cap;
+    }
+  }
   c->d_xs = aim_alloc(c, (size_t)B * ns * es);
   c->d_xd = (double2*)aim_alloc(c, (size_t)B * ns * sizeof(double2));
   c->d_vf = (float2*)aim_alloc(c, (size_t)B * ns * sizeof(float2));
@@ -552,12 +563,11 @@ int aim_rhs(aim_ctx* c, int32_t l, int32_t nb, const aim_c128* hist, aim_c128* r
     const size_t slab = op_slab_bytes(c, c->batch_max);
     SlabList sl{};
     NearList nl{};
+    op_forward_slabs(c, std::min(ng, l - 1), nb, hs, c->d_ring, slab);  // I_{l-m}, m < l
     for (int m = 1; m <= ng; ++m) {
       if (l - m < 1) continue;
       const double2* I = hs + (size_t)(m - 1) * n;
-      void* dst = (char*)c->d_ring + (size_t)(m - 1) * slab;
-      op_forward_slab(c, nb, I, dst);
-      sl.p[sl.n] = dst;
+      sl.p[sl.n] = (char*)c->d_ring + (size_t)(m - 1) * slab;
       sl.m[sl.n] = m;
       sl.n++;
       if (c->nnz > 0) {

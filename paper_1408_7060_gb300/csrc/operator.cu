@@ -17,6 +17,8 @@ void body_apply(aim_ctx*, int, int, const double2*, const double2*, const double
 template <class C>
 void body_forward_slab(aim_ctx*, int, const double2*, void*);
 template <class C>
+void body_forward_slots(aim_ctx*, int, int, const double2*, void*, size_t);
+template <class C>
 void body_apply_rhs(aim_ctx*, int, const SlabList&, void*, const NearList&, const double2*, double, double2*);
 template <class C>
 void body_apply_rhs_pending(aim_ctx*, int, void*, const NearList&, const double2*, double, double2*);
@@ -73,6 +75,26 @@ void op_forward_slab(aim_ctx* c, int nb, const double2* v, void* dst) {
     body_forward_slab<float2>(c, nb, v, dst);
   else
     body_forward_slab<double2>(c, nb, v, dst);
+}
+
+// Several delays go through each pass together where the batch buffers hold them (a single
+// vector of a small grid leaves most of the chip idle: 512 planes for 152 SMs on a 64^3
+// grid), as many as keep the x-transformed grids within kBatchBytes, i.e. in L2.
+void op_forward_slabs(aim_ctx* c, int count, int nb, const double2* v, void* dst, size_t stride) {
+  const int most = op_plane(c) && c->d_Ab ? c->batch_cap / nb : 1;
+  const size_t es = c->precision == AIM_C64 ? sizeof(float2) : sizeof(double2);
+  for (int i = 0; i < count;) {
+    const int n = std::min(count - i, std::max(1, most));
+    const double2* vi = v + (size_t)i * nb * c->ns;
+    char* d = (char*)dst + (size_t)i * stride;
+    if (n == 1)
+      op_forward_slab(c, nb, vi, d);
+    else if (c->precision == AIM_C64)
+      body_forward_slots<float2>(c, n, nb, vi, d, stride / es);
+    else
+      body_forward_slots<double2>(c, n, nb, vi, d, stride / es);
+    i += n;
+  }
 }
 
 void op_apply_rhs(aim_ctx* c, int nb, const SlabList& sl, void* scratch, const NearList& nl, const double2* base,

@@ -57,6 +57,8 @@ void op_apply(aim_ctx* c, int m, int nb, const double2* v, const double2* dinv, 
 void op_apply_f64(aim_ctx* c, int m, int nb, const double2* v, const double2* base, double sign, double2* y);
 // slab of one current vector (anterpolation + forward x and y passes) written to dst
 void op_forward_slab(aim_ctx* c, int nb, const double2* v, void* dst);
+// the slabs of `count` vectors v[count][nb][ns], `stride` bytes apart from dst on
+void op_forward_slabs(aim_ctx* c, int count, int nb, const double2* v, void* dst, size_t stride);
 // y = base + sign * [ sum_s Z~FFT_{m_s} (slab_s) + near terms ]; scratch: a ring slot whose
 // contents are not needed afterwards (it may be one of the slabs), for the delay sum of
 // plane-kernel contexts
@@ -74,9 +76,10 @@ int op_kernel_count(const aim_ctx* c);
 bool op_plane(const aim_ctx* c);
 // decide that, and tabulate the plane kernel's spectra (after the octants)
 void plane_setup(aim_ctx* c);
-// one launch of the plane kernel (mode: PLANE_* of plane.cuh) on d_A
+// one launch of the plane kernel (mode: PLANE_* of plane.cuh) on d_A, for `slots` spectra of
+// nb right-hand sides each, slot_elems apart from S on
 template <class C>
-void plane_launch(aim_ctx* c, int nb, int mode, int m, const int* active, C* S);
+void plane_launch(aim_ctx* c, int nb, int mode, int m, const int* active, C* S, int slots, size_t slot_elems);
 // d_A = inverse of the delay sum over the z-spectra sl (S: scratch for one spectrum)
 template <class C>
 void plane_rhs(aim_ctx* c, int nb, const SlabList& sl, C* S);

@@ -48,6 +48,11 @@ void body_forward_slab(aim_ctx* c, int nb, const double2* v, void* dst) {
 }
 
 template <class C>
+void body_forward_slots(aim_ctx* c, int slots, int nb, const double2* v, void* dst, size_t slot_elems) {
+  AIM_DISPATCH_L(c->L, (GridOps<LL, C>::forward_slots(c, slots, nb, v, reinterpret_cast<C*>(dst), slot_elems)));
+}
+
+template <class C>
 void body_apply_rhs(aim_ctx* c, int nb, const SlabList& sl, void* scratch, const NearList& nl, const double2* base,
                     double sign, double2* y) {
   AIM_DISPATCH_L(c->L, {
@@ -96,6 +101,7 @@ void body_plan_fill(aim_ctx* c) {
   template void body_apply<C>(aim_ctx*, int, int, const double2*, const double2*, const double2*, double,       \
                               const int*, double2*, VecSel, VecSel);                                             \
   template void body_forward_slab<C>(aim_ctx*, int, const double2*, void*);                                     \
+  template void body_forward_slots<C>(aim_ctx*, int, int, const double2*, void*, size_t);                       \
   template void body_apply_rhs<C>(aim_ctx*, int, const SlabList&, void*, const NearList&, const double2*,       \
                                   double, double2*);                                                           \
   template void body_apply_rhs_pending<C>(aim_ctx*, int, void*, const NearList&, const double2*, double,        \

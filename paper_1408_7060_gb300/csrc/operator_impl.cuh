@@ -1260,6 +1260,27 @@ struct GridOps {
     if (!kxm(c)) y_fwd(c, nb, slab);
   }
 
+  // the spectra of `slots` vectors v[slots][nb][ns] in one launch of each pass (kx-major
+  // grids; their grid stages use the batch buffers d_Ab, d_xsb)
+  static void forward_slots(aim_ctx* c, int slots, int nb, const double2* v, C* dst, size_t slot_elems) {
+    struct Swap {  // the batch buffers stand in for the context's for the duration
+      aim_ctx* c;
+      void *A, *xs;
+      explicit Swap(aim_ctx* c_) : c(c_), A(c_->d_A), xs(c_->d_xs) {
+        c->d_A = c->d_Ab;
+        c->d_xs = c->d_xsb;
+      }
+      ~Swap() {
+        c->d_A = A;
+        c->d_xs = xs;
+      }
+    } sw(c);
+    prep(c, slots * nb, v, nullptr, VecSel(), nullptr, false);
+    anterp_x(c, slots * nb, nullptr);
+    KScope ks(c, AIM_K_ZFWD);
+    plane_launch<C>(c, nb, PLANE_FWD, 0, nullptr, dst, slots, slot_elems);
+  }
+
   // inverse y and x passes: Bf slab -> P, then interpolation + near terms
   static void backward(aim_ctx* c, int nb, const NearList& nl, const double2* base, double sign, const int* active,
                        double2* y, VecSel ys = VecSel()) {
@@ -1285,7 +1306,7 @@ struct GridOps {
 
   static void zconv(aim_ctx* c, int nb, int m, const int* active) {
     KScope ks(c, AIM_K_ZCONV);
-    if (kxm(c)) return plane_launch<C>(c, nb, PLANE_CONV, m, active, nullptr);
+    if (kxm(c)) return plane_launch<C>(c, nb, PLANE_CONV, m, active, nullptr, 1, 0);
     C* Bf = reinterpret_cast<C*>(c->d_Bf);
     const C* G = kspec(c) + (size_t)m * 2 * octant(c);
     with_zlen(c->LZ, [&](auto lz) {
@@ -1366,7 +1387,7 @@ struct GridOps {
   static void zfwd(aim_ctx* c, int nb, C* dst) {
     if (kxm(c)) {
       KScope ks(c, AIM_K_ZFWD);
-      return plane_launch<C>(c, nb, PLANE_FWD, 0, nullptr, dst);
+      return plane_launch<C>(c, nb, PLANE_FWD, 0, nullptr, dst, 1, 0);
     }
     with_zlen(c->LZ, [&](auto lz) {
       constexpr int LZ = decltype(lz)::value;
@@ -1440,7 +1461,7 @@ struct GridOps {
   static void zinv_pending(aim_ctx* c, int nb, C* S) {
     if (kxm(c)) {
       KScope ks(c, AIM_K_ZINV_PENDING);
-      return plane_launch<C>(c, nb, PLANE_PENDING, 0, nullptr, S);
+      return plane_launch<C>(c, nb, PLANE_PENDING, 0, nullptr, S, 1, 0);
     }
     with_zlen(c->LZ, [&](auto lz) {
       constexpr int LZ = decltype(lz)::value;

@@ -293,6 +293,8 @@ struct PlaneArgs {
   C* A;              // [nb * 4][L][nz][N]
   C* S;              // FWD: spectra out; INV, PENDING: spectra in
   const C* G;        // CONV: the tabulated spectrum of the delay
+  int sbc;           // (right-hand side, component) pairs per spectrum; further ones go on
+  size_t sstride;    // sstride elements after it (several delays in one launch)
   const int* active;
   const C* twy;
   const C* twz;
@@ -324,7 +326,7 @@ __global__ void __launch_bounds__(32 * PlaneCfg<L, LZ, C>::NW, (PlaneCfg<L, LZ, 
   C* A = a.A + ((size_t)bc * L + kx) * a.nz * N;
   const int kind = (bc & 3) == 3 ? 1 : 0;
   const size_t goff = ((size_t)kind * (N + 1) + (kx <= N ? kx : L - kx)) * plane_g_elems(o);
-  const size_t soff = ((size_t)bc * L + kx) * ((size_t)L * LZ);
+  const size_t soff = (size_t)(bc / a.sbc) * a.sstride + ((size_t)(bc % a.sbc) * L + kx) * ((size_t)L * LZ);
   __syncthreads();
   if (MODE == PLANE_CONV || MODE == PLANE_FWD) {
     for (int z0 = warp * F::RW; z0 < a.nz; z0 += F::NW * F::RW) F::y_forward(A, slab, twy, z0, a.nz);

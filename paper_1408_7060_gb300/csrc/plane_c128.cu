@@ -1,5 +1,5 @@
 // complex128 plane kernel
 #include "plane_launch.cuh"
-template void plane_launch<double2>(aim_ctx*, int, int, int, const int*, double2*);
+template void plane_launch<double2>(aim_ctx*, int, int, int, const int*, double2*, int, size_t);
 template void plane_rhs<double2>(aim_ctx*, int, const SlabList&, double2*);
 template bool plane_tables<double2>(aim_ctx*, int, const double2*, double2**);

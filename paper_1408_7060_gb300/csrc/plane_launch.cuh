@@ -26,19 +26,19 @@ static void plane_with_l(int l, F&& f) {
 }
 
 template <class C>
-void plane_launch(aim_ctx* c, int nb, int mode, int m, const int* active, C* S) {
+void plane_launch(aim_ctx* c, int nb, int mode, int m, const int* active, C* S, int slots, size_t slot_elems) {
   plane_with_l(c->L, [&](auto lt) {
     constexpr int L = decltype(lt)::value;
     plane_with_z<L>(c->LZ, [&](auto zt) {
       constexpr int LZ = decltype(zt)::value;
       if constexpr (plane_fits<L, LZ, C>()) {
-        PlaneArgs<C> a{reinterpret_cast<C*>(c->d_A), S, sel_plane(c, (C*)nullptr), active, sel_tw(c, (C*)nullptr),
-                       sel_twz(c, (C*)nullptr), c->NZ};
+        PlaneArgs<C> a{reinterpret_cast<C*>(c->d_A), S, sel_plane(c, (C*)nullptr), nb * 4, slot_elems, active,
+                       sel_tw(c, (C*)nullptr), sel_twz(c, (C*)nullptr), c->NZ};
         a.G += (size_t)m * plane_spec_elems(plane_order<L, LZ, C>());
         constexpr size_t sm = PlaneCfg<L, LZ, C>::smem;
         auto go = [&](auto kern) {
           smem_opt_in(kern, sm);
-          launch_pdl(c->stream, dim3(nb * 4, L), dim3(32 * PlaneCfg<L, LZ, C>::NW), sm, kern, a);
+          launch_pdl(c->stream, dim3(slots * nb * 4, L), dim3(32 * PlaneCfg<L, LZ, C>::NW), sm, kern, a);
         };
         switch (mode) {
           case PLANE_CONV: go(k_plane<L, LZ, C, PLANE_CONV>); break;
@@ -68,7 +68,7 @@ void plane_rhs(aim_ctx* c, int nb, const SlabList& sl, C* S) {
       }
     });
   });
-  plane_launch<C>(c, nb, PLANE_INV, 0, nullptr, S);
+  plane_launch<C>(c, nb, PLANE_INV, 0, nullptr, S, 1, 0);
 }
 
 // Whether grids of this size run the plane kernel, and its spectra of nm delays from the
