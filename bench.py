@@ -217,16 +217,18 @@ def log(*a):
 
 # --------------------------------------------------------------------------- memory plan
 
-Z_LENGTHS = (16, 32, 64, 128, 192, 256, 768)   # z transform lengths the library is built for
+Z_LENGTHS = (16, 32, 64, 128, 144, 192, 256, 768)   # z transform lengths the library is built for
 
 
 def box_depth(w):
-    """Estimated z-planes of the active box (the stencils of edges between the mesh's
-    lowest and highest vertices, 4 nodes each) and the z transform length the context
-    picks for it (the shortest built length >= 2 nz)."""
-    V = w.mesh[0]
+    """z-planes of the active box (4-node stencils anchored at the midpoints of the mesh's
+    edges) and the z transform length the context picks for it (the shortest built length
+    >= 2 nz)."""
+    V, F = w.mesh
     N, L = w.grid_n, 2 * w.grid_n
-    nz = min(N, int((V[:, 2].max() - V[:, 2].min()) / w.h) + 5)
+    z = 0.5 * (V[F, 2] + V[F[:, [1, 2, 0]], 2])
+    az = np.clip(np.floor((z - w.origin[2]) / w.h) - 1, 0, N - 4)
+    nz = int(az.max() - az.min()) + 4
     lz = next((n for n in Z_LENGTHS if 2 * nz <= n <= L), L)
     return nz, lz
 

@@ -70,7 +70,7 @@ size_t grid_elem(const aim_ctx* c) { return c->precision == AIM_C64 ? sizeof(flo
 // z transform length for nz box planes: the shortest length of the z pass >= 2 nz (at most
 // the padded length L = 2N >= 2 nz)
 static int z_length(int nz, int L) {
-  for (int lz : {16, 32, 64, 128, 192, 256, 768})
+  for (int lz : {16, 32, 64, 128, 144, 192, 256, 768})
     if (lz >= 2 * nz && lz <= L) return lz;
   return L;
 }

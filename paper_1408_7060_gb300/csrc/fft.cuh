@@ -355,6 +355,22 @@ struct HalfDFT {
       v[1] = e1 + w1; v[5] = e1 - w1;
       v[2] = e2 + w2; v[6] = e2 - w2;
       v[3] = e3 + w3; v[7] = e3 - w3;
+    } else if constexpr (R == 12) {  // 4 x 3, n = 3 na + nb, na < 2
+      C t[12];
+#pragma unroll
+      for (int nb = 0; nb < 3; ++nb) dft4_half_in<INV>(v[nb], v[3 + nb], t[nb], t[3 + nb], t[6 + nb], t[9 + nb]);
+#pragma unroll
+      for (int ka = 0; ka < 4; ++ka) {
+        C b[3] = {t[3 * ka], t[3 * ka + 1], t[3 * ka + 2]};
+        if (ka) {
+          b[1] = mul_root<12, INV, C>(b[1], ka);
+          b[2] = mul_root<12, INV, C>(b[2], 2 * ka);
+        }
+        DFT<3, INV, C>::run(b);
+        v[ka] = b[0];
+        v[ka + 4] = b[1];
+        v[ka + 8] = b[2];
+      }
     } else {
       static_assert(R == 16, "half-input radix");
       C t[16];
@@ -396,6 +412,27 @@ struct HalfDFT {
       v[1] = e1 + w1;
       v[2] = e2 + w2;
       v[3] = e3 + w3;
+    } else if constexpr (R == 12) {  // outputs ka + 4 kb < 6
+#pragma unroll
+      for (int nb = 0; nb < 3; ++nb) dft4<INV>(v[nb], v[3 + nb], v[6 + nb], v[9 + nb]);
+      C t[6];
+#pragma unroll
+      for (int ka = 0; ka < 4; ++ka) {
+        C b[3] = {v[3 * ka], v[3 * ka + 1], v[3 * ka + 2]};
+        if (ka) {
+          b[1] = mul_root<12, INV, C>(b[1], ka);
+          b[2] = mul_root<12, INV, C>(b[2], 2 * ka);
+        }
+        if (ka < 2) {
+          DFT<3, INV, C>::run(b);
+          t[ka] = b[0];
+          t[ka + 4] = b[1];
+        } else {
+          t[ka] = b[0] + (b[1] + b[2]);
+        }
+      }
+#pragma unroll
+      for (int q = 0; q < 6; ++q) v[q] = t[q];
     } else {
       static_assert(R == 16, "half-output radix");
 #pragma unroll
@@ -425,7 +462,7 @@ struct HalfDFT {
 // v[0..R) out in natural order.
 template <int R, int L, bool INV, class C>
 __device__ __forceinline__ void dft_half_in(C* v, const C* tw) {
-  if constexpr (R == 4 || R == 8 || R == 16) {  // the zeros drop out of the first butterflies
+  if constexpr (R == 4 || R == 8 || R == 12 || R == 16) {  // the zeros drop out of the first butterflies
     HalfDFT<R, INV, C>::in(v);
     return;
   }
@@ -450,7 +487,7 @@ __device__ __forceinline__ void dft_half_in(C* v, const C* tw) {
 // inputs.  v[0..R) in, v[0..R/2) out.
 template <int R, int L, bool INV, class C>
 __device__ __forceinline__ void dft_half_out(C* v, const C* tw) {
-  if constexpr (R == 4 || R == 8 || R == 16) {
+  if constexpr (R == 4 || R == 8 || R == 12 || R == 16) {
     HalfDFT<R, INV, C>::out(v);
     return;
   }
@@ -473,11 +510,14 @@ __device__ __forceinline__ void dft_half_out(C* v, const C* tw) {
 // Step A: one radix-R1 DFT per (line, n2) and the twiddles W_L^{n2 k1};
 // step B: one radix-R2 DFT per (line, k1).  Each step reads and writes shared memory once.
 __host__ __device__ constexpr bool pow2_len(int L) { return L == 16 || L == 32 || L == 64 || L == 128 || L == 256 || L == 512; }
-// lengths with a two-step plan: the powers of two and 96 = 8 x 12, 192 = 16 x 12, 768 = 32 x 24
-__host__ __device__ constexpr bool two_step_len(int L) { return pow2_len(L) || L == 96 || L == 192 || L == 768; }
+// lengths with a two-step plan: the powers of two and 96 = 8 x 12, 144 = 12 x 12, 192 = 16 x 12,
+// 768 = 32 x 24
+__host__ __device__ constexpr bool two_step_len(int L) {
+  return pow2_len(L) || L == 96 || L == 144 || L == 192 || L == 768;
+}
 __host__ __device__ constexpr int split_r1(int L) {
   return L == 16 ? 4 : L == 32 ? 8 : L == 64 ? 8 : L == 128 ? 8 : L == 256 ? 16 : L == 512 ? 16
-       : L == 96 ? 8 : L == 192 ? 16 : L == 768 ? 32 : 0;
+       : L == 96 ? 8 : L == 144 ? 12 : L == 192 ? 16 : L == 768 ? 32 : 0;
 }
 
 // Column tile: W lines, element i of line l at a[i*W + l].  Result in natural order in a.

@@ -30,6 +30,16 @@ __device__ __forceinline__ int zpass_row(int j, int N) {
   return (j & 1) ? 2 * N - k : k;
 }
 
+// The twiddles of a two-step transform, tw[k1 (R2 + 1) + n2] = W_L^{n2 k1}: lanes that walk n2
+// or k1 read different banks (W_L^{n2 k1} in a table of L entries puts all lanes of a warp in
+// one bank for k1 = 16), and the offsets of an unrolled k1 or n2 are immediates.
+template <int R1, int R2>
+constexpr int kTw2 = R1 * (R2 + 1);
+template <int R1, int R2, class C>
+__device__ __forceinline__ void load_twiddles2(C* tw, const C* __restrict__ twg) {
+  for (int i = threadIdx.x; i < R1 * R2; i += blockDim.x) tw[(i / R2) * (R2 + 1) + i % R2] = twg[(i / R2) * (i % R2)];
+}
+
 // Transform the lines of a tile (after a __syncthreads that publishes a); returns
 // the buffer holding the natural-order result.  Lengths with a two-step plan use the
 // two-step transform, any other the Stockham passes.
@@ -105,8 +115,8 @@ __global__ void __launch_bounds__(256) k_rows_p2(const C* __restrict__ in, C* __
   pdl_wait();
   constexpr int R1 = split_r1(L), R2 = L / R1, P = row_tmp_pitch<L>();
   C* tw = reinterpret_cast<C*>(aim_smem);
-  C* t = tw + L;
-  load_twiddles(tw, twg, L);
+  C* t = tw + kTw2<R1, R2>;
+  load_twiddles2<R1, R2>(tw, twg);
   __syncthreads();
   const int r0 = blockIdx.x * rpb;
   const int nr = min(rpb, nrows - r0);
@@ -123,8 +133,8 @@ __global__ void __launch_bounds__(256) k_rows_p2(const C* __restrict__ in, C* __
 #pragma unroll
     for (int k1 = 0; k1 < R1; ++k1) {
       C x = v[k1];
-      if (k1 && n2) {
-        const C w = tw[n2 * k1];
+      if (k1) {
+        const C w = tw[k1 * (R2 + 1) + n2];
         x = x * (INV ? conjc(w) : w);
       }
       t[r * P + k1 * (R2 + 1) + n2] = x;

@@ -59,9 +59,9 @@ __global__ void __launch_bounds__(256) k_anterp(const int* __restrict__ arow, co
   using R = typename Real<C>::T;
   constexpr int N = L / 2, R1 = x_r1(L), R2 = x_r2(L), PX = x_pitch(L, KXM ? YB : 1), ROWS = 4 * YB * BB;
   C* tw = reinterpret_cast<C*>(aim_smem);
-  C* in = tw + L;             // [bs][c][yy][N]
+  C* in = tw + kTw2<R1, R2>;  // [bs][c][yy][N]
   C* tmp = in + ROWS * N;     // [bs][c][yy][PX]
-  load_twiddles(tw, twg, L);
+  load_twiddles2<R1, R2>(tw, twg);
   for (int i = threadIdx.x; i < ROWS * N; i += 256) in[i] = C{};
   pdl_wait();
   const int b0 = blockIdx.x * BB, y0 = blockIdx.y * YB, z = blockIdx.z;  // y relative to the box
@@ -140,7 +140,7 @@ __global__ void __launch_bounds__(256) k_anterp(const int* __restrict__ arow, co
     for (int n1 = 0; n1 < R1 / 2; ++n1) v[n1] = in[row * N + R2 * n1 + n2];
     dft_half_in<R1, L, false, C>(v, tw);
 #pragma unroll
-    for (int k1 = 0; k1 < R1; ++k1) tmp[row * PX + k1 * (R2 + 1) + n2] = k1 ? v[k1] * tw[n2 * k1] : v[k1];
+    for (int k1 = 0; k1 < R1; ++k1) tmp[row * PX + k1 * (R2 + 1) + n2] = k1 ? v[k1] * tw[k1 * (R2 + 1) + n2] : v[k1];
   }
   __syncthreads();
   for (int u = threadIdx.x; u < ROWS * R1; u += 256) {
@@ -179,8 +179,8 @@ __global__ void __launch_bounds__(256) k_xinv(const C* __restrict__ A, C* __rest
                                               const C* __restrict__ twg, int ylo, int nyb, int nz) {
   constexpr int N = L / 2, R1 = x_r1(L), R2 = x_r2(L), PX = x_pitch(L, YB);
   C* tw = reinterpret_cast<C*>(aim_smem);
-  C* tmp = tw + L;
-  load_twiddles(tw, twg, L);
+  C* tmp = tw + kTw2<R1, R2>;
+  load_twiddles2<R1, R2>(tw, twg);
   pdl_wait();
   __syncthreads();
   const int y0 = blockIdx.x * YB, z = blockIdx.y, bc = blockIdx.z;
@@ -193,7 +193,7 @@ __global__ void __launch_bounds__(256) k_xinv(const C* __restrict__ A, C* __rest
     DFTL<R1, L, true, C>::run(v, tw);
 #pragma unroll
     for (int k1 = 0; k1 < R1; ++k1)
-      tmp[yy * PX + k1 * (R2 + 1) + n2] = k1 ? v[k1] * conjc(tw[n2 * k1]) : v[k1];
+      tmp[yy * PX + k1 * (R2 + 1) + n2] = k1 ? v[k1] * conjc(tw[k1 * (R2 + 1) + n2]) : v[k1];
   }
   __syncthreads();
   C* dst = P + ((size_t)bc * nz + z) * N * N + (size_t)(ylo + y0) * N;
@@ -454,6 +454,288 @@ __global__ void __launch_bounds__(kZThreads) k_zconv_p2(C* __restrict__ Bf, cons
   __syncthreads();
   zcol_step_c<LZ, W, C>(t, tw, col, es, g.nz);
   pdl_trigger();
+}
+
+// The y passes of large complex64 grids (those the plane kernel does not hold): W adjacent
+// lines per tile, two-step transform L = R1 R2 as in k_cols_p2, each block running through
+// many tiles with the next tile's rows on their way (cp.async) while the current one is
+// transformed, so loads, butterflies and stores overlap.  Rows outside [in_lo, in_hi] are
+// zero (the stage keeps zeros there), outputs outside [out_lo, out_hi] are not stored.
+// Measured, 4 waves on the 384^3 grid, per launch: forward 2.00 -> 1.52 ms, inverse 2.24 ->
+// 1.39 ms against k_cols_p2; floor 1.2 ms of HBM traffic each.
+template <int L, bool INV>
+struct YPipe {
+  static constexpr int R1 = split_r1(L), R2 = L / R1, W = L == 768 ? 8 : 16, NT = 256;
+  static constexpr int ROWS = INV ? L : L / 2;  // rows of a staged tile
+  static constexpr size_t smem = (size_t)(kTw2<R1, R2> + ROWS * W + L * W) * sizeof(float2);
+  static constexpr int blocks = smem <= 72 * 1024 ? 3 : 2;
+  // exchange row (k1, n2); with 8 lines a half-warp spans two k1, put on rows of opposite parity
+  static __device__ __forceinline__ int row(int k1, int n2) { return k1 * R2 + (W == 8 ? n2 ^ (k1 & 1) : n2); }
+};
+template <int L, bool INV>
+__global__ void __launch_bounds__(256, (YPipe<L, INV>::blocks))
+    k_ypipe(const float2* __restrict__ in, float2* __restrict__ out, int ntiles, int in_lo, int in_hi, int out_lo,
+            int out_hi, long long plane_in, long long plane_out, const float2* __restrict__ twg) {
+  using Y = YPipe<L, INV>;
+  constexpr int R1 = Y::R1, R2 = Y::R2, W = Y::W, NT = Y::NT, CH = W / 2;  // 16-byte chunks per row
+  float2* tw = reinterpret_cast<float2*>(aim_smem);
+  float2* stage = tw + kTw2<R1, R2>;
+  float2* t = stage + Y::ROWS * W;
+  load_twiddles2<R1, R2>(tw, twg);
+  for (int i = threadIdx.x; i < Y::ROWS * W; i += NT)
+    if (i / W < in_lo || i / W > in_hi) stage[i] = make_float2(0, 0);
+  pdl_wait();
+  // tile = (plane, x tile), x fastest
+  auto fetch = [&](int tile) {
+    const float2* src = in + (tile / (L / W)) * plane_in + (tile % (L / W)) * W;
+    for (int i = threadIdx.x; i < (in_hi - in_lo + 1) * CH; i += NT) {
+      const int r = in_lo + i / CH, c = i % CH;
+      cp_async16(smem_addr(stage + r * W + 2 * c), src + (long long)r * L + 2 * c);
+    }
+    cp_async_commit();
+  };
+  int tile = blockIdx.x;
+  if (tile < ntiles) fetch(tile);
+  for (; tile < ntiles; tile += gridDim.x) {
+    cp_async_wait();
+    __syncthreads();
+    for (int u = threadIdx.x; u < W * R2; u += NT) {
+      const int l = u % W, n2 = u / W;
+      float2 v[R1];
+#pragma unroll
+      for (int n1 = 0; n1 < (INV ? R1 : R1 / 2); ++n1) v[n1] = stage[(R2 * n1 + n2) * W + l];
+      if constexpr (INV)
+        DFTL<R1, L, true, float2>::run(v, tw);
+      else
+        dft_half_in<R1, L, false, float2>(v, tw);
+#pragma unroll
+      for (int k1 = 0; k1 < R1; ++k1) {
+        const float2 w = tw[k1 * (R2 + 1) + n2];
+        t[Y::row(k1, n2) * W + l] = k1 ? v[k1] * (INV ? conjc(w) : w) : v[k1];
+      }
+    }
+    __syncthreads();  // the stage may be refilled
+    if (tile + (int)gridDim.x < ntiles) fetch(tile + gridDim.x);
+    float2* dst = out + (tile / (L / W)) * plane_out + (tile % (L / W)) * W;
+    for (int u = threadIdx.x; u < W * R1; u += NT) {
+      const int l = u % W, k1 = u / W;
+      float2 v[R2];
+#pragma unroll
+      for (int n2 = 0; n2 < R2; ++n2) v[n2] = t[Y::row(k1, n2) * W + l];
+      if constexpr (INV) {
+        dft_half_out<R2, L, true, float2>(v, tw);  // outputs below L / 2 only
+#pragma unroll
+        for (int k2 = 0; k2 < R2 / 2; ++k2) {
+          const int k = k1 + R1 * k2;
+          if (k >= out_lo && k <= out_hi) dst[(long long)k * L + l] = v[k2];
+        }
+      } else {
+        DFTL<R2, L, false, float2>::run(v, tw);
+#pragma unroll
+        for (int k2 = 0; k2 < R2; ++k2) dst[(long long)(k1 + R1 * k2) * L + l] = v[k2];
+      }
+    }
+  }
+  cp_async_wait();
+}
+
+// The z pass of the lengths with a factor 3 on large complex64 grids.  A warp takes CW = 8
+// adjacent columns, 32 lanes = (column, n2 or k1), and its own exchange buffer, so the block
+// never synchronises and every lane has work in each step (12 or 16 items per column).  The
+// columns of the next component (or, in Z_RHS, of the next delay) stream into the warp's tile
+// by cp.async while the current ones are transformed.  With MODE Z_CONV the warp runs through
+// all right-hand sides and components of its columns; where the lane's slice of the kernel
+// spectrum fits in registers (LZ = 144) it is read once per kernel kind instead of once per
+// component.  With MODE Z_RHS it sums the delays of one (right-hand side, component) in
+// registers.  Each 8-column run is two 32-byte sectors.
+// Measured, 4 waves on the 384^3 grid (72 box planes), per launch: block tiles of 32 columns
+// 4.94 ms at LZ = 192 (416 warp instructions per column, a quarter of the lanes idle in two of
+// the three steps); this kernel 3.2 ms at LZ = 144 (3.85 ms with register loads instead of
+// cp.async, waiting for memory).  Floors: 1.6 ms HBM, 1.7 ms FP32.
+enum { Z_CONV = 0, Z_RHS = 1 };
+template <int LZ>
+struct ZWarp {
+  static constexpr int R1 = zsplit_r1<LZ>(), R2 = LZ / R1, CW = 8, NW = 4;
+  static constexpr int QA = CW * R2 / 32, QB = CW * R1 / 32;
+  static constexpr bool HOLD = QB * R2 <= 36;
+  // column pitch 2 mod 16: the 8 columns of a half-warp fall in different banks
+  static constexpr int PZ = pl_round(R1 * (R2 + 1), 2);
+  static constexpr int TILE = LZ / 2 * CW, PER_WARP = TILE + CW * PZ;
+  static constexpr size_t smem = (size_t)(kTw2<R1, R2> + NW * PER_WARP) * sizeof(float2);
+  static constexpr int blocks = (int)((size_t)(228 * 1024) / (smem + 1024));
+  static_assert(CW * R1 % 32 == 0 && CW * R2 % 32 == 0, "whole warps");
+
+  // start copying the nz rows of 8 columns into the warp's tile [row][8]
+  static __device__ __forceinline__ void fetch(const float2* __restrict__ col, long long es, int nz, float2* tile) {
+    const int lane = threadIdx.x & 31;
+    const float2* s = col + (lane >> 2) * es + 2 * (lane & 3);
+    unsigned d = smem_addr(tile + 2 * lane);
+    for (int r = lane >> 2; r < nz; r += 8) {
+      cp_async16(d, s);
+      s += 8 * es;
+      d += 64 * sizeof(float2);
+    }
+    cp_async_commit();
+  }
+  static __device__ __forceinline__ void fetched() {
+    cp_async_wait();
+    __syncwarp();
+  }
+  static __device__ __forceinline__ void step_a(const float2* tile, float2* scr, const float2* tw) {
+    const int lane = threadIdx.x & 31, l = lane & 7;
+#pragma unroll
+    for (int q = 0; q < QA; ++q) {
+      const int n2 = (lane >> 3) + 4 * q;
+      float2 v[R1];
+#pragma unroll
+      for (int n1 = 0; n1 < R1 / 2; ++n1) v[n1] = tile[(R2 * n1 + n2) * CW + l];
+      dft_half_in<R1, LZ, false, float2>(v, tw);
+      float2* t = scr + l * PZ + n2;
+#pragma unroll
+      for (int k1 = 0; k1 < R1; ++k1) t[k1 * (R2 + 1)] = k1 ? v[k1] * tw[k1 * (R2 + 1) + n2] : v[k1];
+    }
+    __syncwarp();  // the tile may be refilled, the exchange buffer is complete
+  }
+  static __device__ __forceinline__ void step_c(float2* __restrict__ dst, long long es, int nz, const float2* scr,
+                                                const float2* tw) {
+    const int lane = threadIdx.x & 31, l = lane & 7;
+    __syncwarp();
+#pragma unroll
+    for (int q = 0; q < QA; ++q) {
+      const int n2 = (lane >> 3) + 4 * q;
+      const float2* t = scr + l * PZ + n2;
+      float2 v[R1];
+#pragma unroll
+      for (int k1 = 0; k1 < R1; ++k1) v[k1] = t[k1 * (R2 + 1)];
+      dft_half_out<R1, LZ, true, float2>(v, tw);
+      float2* d = dst + n2 * es + l;
+#pragma unroll
+      for (int n1 = 0; n1 < R1 / 2; ++n1) {
+        if (R2 * n1 + n2 < nz) *d = v[n1];
+        d += R2 * es;
+      }
+    }
+    __syncwarp();
+  }
+  // the lane's slice kz = k1 + R1 k2 of a spectrum octant: ascending below LZ/2, then descending
+  static __device__ __forceinline__ void load_g(const float2* __restrict__ G, size_t nn, int k1, float2 (&g)[R2]) {
+    const float2* p = G + (size_t)k1 * nn;
+#pragma unroll
+    for (int k2 = 0; k2 < R2 / 2; ++k2) {
+      g[k2] = __ldg(p);
+      p += R1 * nn;
+    }
+    p = G + (size_t)(LZ / 2 - k1) * nn;  // kz = LZ/2 + k1 + R1 (k2 - R2/2) mirrors LZ/2 - ...
+#pragma unroll
+    for (int k2 = R2 / 2; k2 < R2; ++k2) {
+      g[k2] = __ldg(p);
+      p -= R1 * nn;
+    }
+  }
+  static __device__ __forceinline__ void b_forward(const float2* t, const float2* tw, float2 (&v)[R2]) {
+#pragma unroll
+    for (int n2 = 0; n2 < R2; ++n2) v[n2] = t[n2];
+    DFTL<R2, LZ, false, float2>::run(v, tw);
+  }
+  static __device__ __forceinline__ void b_inverse(float2* t, const float2* tw, int k1, float2 (&v)[R2]) {
+    DFTL<R2, LZ, true, float2>::run(v, tw);
+#pragma unroll
+    for (int n2 = 0; n2 < R2; ++n2) t[n2] = n2 ? v[n2] * conjc(tw[k1 * (R2 + 1) + n2]) : v[n2];
+  }
+};
+
+// Grid (L / 32, L[, nb * 4 for Z_RHS]): 32 adjacent columns of row y (mirror order) per block.
+template <int LZ, int MODE>
+__global__ void __launch_bounds__(32 * ZWarp<LZ>::NW, ZWarp<LZ>::blocks)
+    k_zwarp(float2* __restrict__ Bf, const float2* __restrict__ kspec, ZGeom g, int nb, const int* __restrict__ active,
+            const float2* __restrict__ twg, const __grid_constant__ SlabList sl) {
+  using Z = ZWarp<LZ>;
+  constexpr int QB = Z::QB, R2 = Z::R2;
+  float2* tw = reinterpret_cast<float2*>(aim_smem);
+  load_twiddles2<Z::R1, Z::R2>(tw, twg);
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  float2* tile = tw + kTw2<Z::R1, Z::R2> + warp * Z::PER_WARP;
+  float2* scr = tile + Z::TILE;
+  for (int i = g.nz * Z::CW + lane; i < Z::TILE; i += 32) tile[i] = make_float2(0, 0);  // below the box
+  pdl_wait();
+  __syncthreads();
+  const int y = zpass_row(blockIdx.y, g.N), x0 = (blockIdx.x * Z::NW + warp) * Z::CW;
+  const long long es = (long long)g.L * g.L;
+  const size_t nn = (size_t)(g.N + 1) * (g.N + 1), oct = nn * (LZ / 2 + 1);
+  const size_t off = (size_t)y * g.L + x0, slab = (size_t)g.nz * es;
+  // step B: lane (column, k1 = lane / 8 + 4 q)
+  float2* tb = scr + (lane & 7) * Z::PZ;
+  if (MODE == Z_CONV) {
+    // components i: x, y, z of every right-hand side, then div of every right-hand side
+    const int n = 4 * nb;
+    auto comp = [&](int i) { return i < 3 * nb ? (i / 3) * 4 + i % 3 : (i - 3 * nb) * 4 + 3; };
+    auto next = [&](int i) {  // the first component from i on whose right-hand side takes part
+      while (i < n && active && !active[comp(i) >> 2]) ++i;
+      return i;
+    };
+    int i = next(0), loaded = -1;
+    if (i < n) Z::fetch(Bf + comp(i) * slab + off, es, g.nz, tile);
+    float2 gk[Z::HOLD ? QB : 1][R2];
+#pragma unroll 1
+    while (i < n) {
+      const int kind = i < 3 * nb ? 0 : 1;
+      const float2* G = kcol<LZ>(kspec, g, kind, x0 + (lane & 7), y);
+      if (Z::HOLD && kind != loaded) {
+#pragma unroll
+        for (int q = 0; q < (Z::HOLD ? QB : 0); ++q) Z::load_g(G, nn, (lane >> 3) + 4 * q, gk[q]);
+        loaded = kind;
+      }
+      Z::fetched();
+      Z::step_a(tile, scr, tw);
+      const int j = next(i + 1);
+      if (j < n) Z::fetch(Bf + comp(j) * slab + off, es, g.nz, tile);
+#pragma unroll
+      for (int q = 0; q < QB; ++q) {
+        const int k1 = (lane >> 3) + 4 * q;
+        float2* t = tb + k1 * (R2 + 1);
+        float2 v[R2];
+        if constexpr (!Z::HOLD) Z::load_g(G, nn, k1, gk[0]);
+        Z::b_forward(t, tw, v);
+#pragma unroll
+        for (int k2 = 0; k2 < R2; ++k2) v[k2] = v[k2] * gk[Z::HOLD ? q : 0][k2];
+        Z::b_inverse(t, tw, k1, v);
+      }
+      Z::step_c(Bf + comp(i) * slab + off, es, g.nz, scr, tw);
+      i = j;
+    }
+  } else {
+    const int bc = blockIdx.z;
+    auto col = [&](int s) { return reinterpret_cast<const float2*>(sl.p[s]) + bc * slab + off; };
+    float2 acc[QB][R2];
+#pragma unroll
+    for (int q = 0; q < QB; ++q)
+#pragma unroll
+      for (int k2 = 0; k2 < R2; ++k2) acc[q][k2] = make_float2(0, 0);
+    if (sl.n > 0) Z::fetch(col(0), es, g.nz, tile);
+#pragma unroll 1
+    for (int s = 0; s < sl.n; ++s) {
+      const float2* G = kcol<LZ>(kspec + (size_t)sl.m[s] * 2 * oct, g, (bc & 3) == 3 ? 1 : 0, x0 + (lane & 7), y);
+      Z::fetched();
+      Z::step_a(tile, scr, tw);
+      if (s + 1 < sl.n) Z::fetch(col(s + 1), es, g.nz, tile);
+#pragma unroll
+      for (int q = 0; q < QB; ++q) {
+        const int k1 = (lane >> 3) + 4 * q;
+        float2 v[R2], gk[R2];
+        Z::load_g(G, nn, k1, gk);
+        Z::b_forward(tb + k1 * (R2 + 1), tw, v);
+#pragma unroll
+        for (int k2 = 0; k2 < R2; ++k2) acc[q][k2] += v[k2] * gk[k2];
+      }
+      __syncwarp();
+    }
+#pragma unroll
+    for (int q = 0; q < QB; ++q) {
+      const int k1 = (lane >> 3) + 4 * q;
+      Z::b_inverse(tb + k1 * (R2 + 1), tw, k1, acc[q]);
+    }
+    Z::step_c(Bf + bc * slab + off, es, g.nz, scr, tw);
+  }
 }
 
 // History slabs of power-of-two z length are kept z-transformed: S[bc][kz][y][x], all LZ
@@ -1035,6 +1317,7 @@ inline void with_zlen(int lz, F&& f) {
     case 32: f(std::integral_constant<int, 32>{}); break;
     case 64: f(std::integral_constant<int, 64>{}); break;
     case 128: f(std::integral_constant<int, 128>{}); break;
+    case 144: f(std::integral_constant<int, 144>{}); break;
     case 192: f(std::integral_constant<int, 192>{}); break;
     case 256: f(std::integral_constant<int, 256>{}); break;
     case 768: f(std::integral_constant<int, 768>{}); break;
@@ -1048,6 +1331,18 @@ constexpr size_t kPlanSmemMax = 220 * 1024;  // dynamic shared memory a plan may
 template <int L, int LZ, class C>
 constexpr bool plane_always() {
   return plane_fits<L, LZ, C>() && pow2_len(LZ);
+}
+
+// z lengths with a factor 3 in complex64 whose exchange fits a warp's buffer: k_zwarp
+template <int L, int LZ, class C>
+constexpr bool zwarp_len() {
+  return sizeof(C) == 8 && LZ <= L && L % 64 == 0 && (LZ == 144 || LZ == 192);
+}
+
+// padded lengths whose separate y passes run in k_ypipe (FP64 lines are bound by arithmetic)
+template <int L, class C>
+constexpr bool ypipe_len() {
+  return sizeof(C) == 8 && (L == 192 || L == 256 || L == 768);
 }
 
 template <int L, class C>
@@ -1066,7 +1361,7 @@ struct GridOps {
     return fill_rows(c, 16, (long long)c->batch_max * 4 * c->NZ);
   }
   static int def_ypb(const aim_ctx* c) {
-    return kxm(c) ? fill_rows(c, 8, (long long)c->NZ * ((c->batch_max + 1) / 2)) : 1;
+    return kxm(c) ? fill_rows(c, c->batch_max > 1 ? 4 : 8, (long long)c->NZ * ((c->batch_max + 1) / 2)) : 1;
   }
   // the most rows per block (a power of two up to `most`) that still give every SM two blocks
   static int fill_rows(const aim_ctx* c, int most, long long others) {
@@ -1076,11 +1371,15 @@ struct GridOps {
   }
   static size_t smem_z(int lz, int w) { return (size_t)(lz + lz * w) * sizeof(C); }
   static size_t smem_y(int w) { return (size_t)(L + L * w) * sizeof(C); }
-  static size_t smem_x(int rp) { return (size_t)(L + rp * row_tmp_pitch<L>()) * sizeof(C); }
-  static size_t smem_anterp(int yb, int bb, bool k) {
-    return (L + (size_t)4 * yb * bb * (L / 2 + x_pitch(L, k ? yb : 1))) * sizeof(C);
+  static size_t smem_x(int rp) {
+    return (size_t)(row_tmp_pitch<L>() + rp * row_tmp_pitch<L>()) * sizeof(C);
   }
-  static size_t smem_xinv(int yb) { return (L + (size_t)yb * x_pitch(L, yb)) * sizeof(C); }
+  static size_t smem_anterp(int yb, int bb, bool k) {
+    return (x_r1(L) * (x_r2(L) + 1) + (size_t)4 * yb * bb * (L / 2 + x_pitch(L, k ? yb : 1))) * sizeof(C);
+  }
+  static size_t smem_xinv(int yb) {
+    return (x_r1(L) * (x_r2(L) + 1) + (size_t)yb * x_pitch(L, yb)) * sizeof(C);
+  }
   // the plan holds the shapes of the context's own precision (the FP64 residual of the
   // refinement on the complex64 path runs with the defaults)
   static bool own(const aim_ctx* c) { return (c->precision == AIM_C64) == (sizeof(C) == sizeof(float2)); }
@@ -1155,8 +1454,12 @@ struct GridOps {
   template <bool KXM>
   static void anterp_as(aim_ctx* c, int nb, const int* active) {
     const int most = std::min(8, L / 2), nyb = nbox(c, 1);
-    // a batch in pairs: two right-hand sides per block share the coefficient loads
-    const int bb = nb > 1 ? 2 : 1;
+    // a batch in pairs (two right-hand sides per block share the coefficient loads) where the
+    // pairs fill the chip four times with 4 rows per block (whatever the plan's rows: the order
+    // of the sums depends on this); else 4 lanes per node (3 waves, 1160 unknowns: 8.6 us
+    // against 12.7 in pairs; 64 waves, 7680 unknowns: 533 against 469)
+    const long long pairs = (long long)((nb + 1) / 2) * c->NZ * ((nyb + 3) / 4);
+    const int bb = nb > 1 && pairs >= 4 * 152 ? 2 : 1;
     int yp = ypb(c);
     while (yp > 1 && smem_anterp(yp, bb, KXM) > (size_t)kPlaneSmemMax) yp /= 2;
     with_rows(yp, most, [&](auto yt) {
@@ -1186,12 +1489,24 @@ struct GridOps {
     anterp_as<false>(c, nb, active);
   }
 
+  template <bool INV>
+  static void ypipe(aim_ctx* c, int nb, const float2* in, float2* out) {
+    using Y = YPipe<L, INV>;
+    const int ntiles = nb * 4 * c->NZ * (L / Y::W), lo = c->box_lo[1], hi = c->box_hi[1];
+    const long long half = (long long)c->N * L, full = (long long)L * L;
+    auto kern = k_ypipe<L, INV>;
+    smem_opt_in(kern, Y::smem);
+    launch_pdl(c->stream, dim3(std::min(ntiles, 152 * Y::blocks)), dim3(Y::NT), Y::smem, kern, in, out, ntiles,
+               INV ? 0 : lo, INV ? L - 1 : hi, lo, hi, INV ? full : half, INV ? half : full, twiddles(c));
+  }
+
   // forward y pass (pruned input): A -> slab
   static void y_fwd(aim_ctx* c, int nb, C* slab) {
     static_assert(two_step_len(L), "every supported padded length has a two-step plan");
     const int N = c->N, nz = c->NZ;
     const C* A = reinterpret_cast<const C*>(c->d_A);
     KScope ks(c, AIM_K_YFFT_FWD);
+    if constexpr (ypipe_len<L, C>()) return ypipe<false>(c, nb, A, slab);
     with_width(cw(c), [&](auto wt) {
       constexpr int CW = decltype(wt)::value;
       if constexpr (CW <= L) {
@@ -1211,6 +1526,8 @@ struct GridOps {
   static void y_inv(aim_ctx* c, int nb) {
     const int N = c->N, nz = c->NZ;
     KScope ks(c, AIM_K_YFFT_INV);
+    if constexpr (ypipe_len<L, C>())
+      return ypipe<true>(c, nb, reinterpret_cast<const C*>(c->d_Bf), reinterpret_cast<C*>(c->d_A));
     with_width(cw(c), [&](auto wt) {
       constexpr int CW = decltype(wt)::value;
       if constexpr (CW <= L) {
@@ -1311,7 +1628,13 @@ struct GridOps {
     const C* G = kspec(c) + (size_t)m * 2 * octant(c);
     with_zlen(c->LZ, [&](auto lz) {
       constexpr int LZ = decltype(lz)::value;
-      if constexpr (LZ <= L && !plane_always<L, LZ, C>()) {
+      if constexpr (zwarp_len<L, LZ, C>()) {
+        constexpr size_t sm = ZWarp<LZ>::smem;
+        smem_opt_in(k_zwarp<LZ, Z_CONV>, sm);
+        launch_pdl(c->stream, dim3(L / (ZWarp<LZ>::CW * ZWarp<LZ>::NW), L), dim3(32 * ZWarp<LZ>::NW), sm,
+                   k_zwarp<LZ, Z_CONV>, Bf, G, zgeom(c), nb, active,
+                   ztwiddles(c), SlabList{});
+      } else if constexpr (LZ <= L && !plane_always<L, LZ, C>()) {
         with_width(zw(c), [&](auto wt) {
           constexpr int ZW = decltype(wt)::value;
           if constexpr (ZW <= L) {
@@ -1411,7 +1734,13 @@ struct GridOps {
     if (kxm(c)) return plane_rhs<C>(c, nb, sl, scratch);
     with_zlen(c->LZ, [&](auto lz) {
       constexpr int LZ = decltype(lz)::value;
-      if constexpr (LZ <= L && !plane_always<L, LZ, C>()) {
+      if constexpr (zwarp_len<L, LZ, C>()) {
+        constexpr size_t sm = ZWarp<LZ>::smem;
+        smem_opt_in(k_zwarp<LZ, Z_RHS>, sm);
+        launch_pdl(c->stream, dim3(L / (ZWarp<LZ>::CW * ZWarp<LZ>::NW), L, nb * 4), dim3(32 * ZWarp<LZ>::NW),
+                   sm, k_zwarp<LZ, Z_RHS>, Bf, kspec(c), zgeom(c), nb,
+                   (const int*)nullptr, ztwiddles(c), sl);
+      } else if constexpr (LZ <= L && !plane_always<L, LZ, C>()) {
         if constexpr (pow2_len(LZ) && LZ <= 256 && L <= 256 && std::is_same<C, float2>::value) {
           // the spectra's ring slots (the march and aim_rhs keep every history slab in the ring)
           const size_t slab = op_slab_bytes(c, c->batch_max);
@@ -1443,8 +1772,8 @@ struct GridOps {
           k_zrhs_spec<LZ, ZW, C><<<dim3(L / ZW, L, nb * 4), kZThreads, sm, c->stream>>>(sl, kspec(c), zgeom(c), Bf,
                                                                                       ztwiddles(c));
         } else {
-          // 8 columns per tile: one step-B item per thread, the delay sum held in registers
-          constexpr int ZW = L < 8 ? L : 8;
+          // one step-B item per thread, the delay sum held in registers
+          constexpr int ZW = zsplit_r1<LZ>() <= 16 ? 16 : 8;
           const size_t sm = smem_z(LZ, ZW);
           smem_opt_in(k_zrhs_2s<LZ, ZW, C>, sm);
           k_zrhs_2s<LZ, ZW, C><<<dim3(nb * 4, L / ZW, L), kZThreads, sm, c->stream>>>(sl, kspec(c), zgeom(c), Bf,

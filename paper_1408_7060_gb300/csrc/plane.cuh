@@ -38,7 +38,7 @@ constexpr int kPlaneSmemMax = 227 * 1024;  // shared memory a block can opt in t
 
 // radix split of a length (R1 for the step next to the padding, whose zero half is pruned)
 __host__ __device__ constexpr int pl_r1(int L) {
-  return L == 16 ? 4 : L == 32 ? 8 : L == 64 ? 8 : (L == 128 || L == 192 || L == 256) ? 16 : 0;
+  return L == 16 ? 4 : L == 32 ? 8 : L == 64 ? 8 : L == 144 ? 12 : (L == 128 || L == 192 || L == 256) ? 16 : 0;
 }
 __host__ __device__ constexpr int pl_r2(int L) { return pl_r1(L) ? L / pl_r1(L) : 0; }
 // the first pitch >= p that is r mod 16
@@ -62,8 +62,9 @@ struct PlaneCfg {
   static constexpr int YB = Y2 + 1;
   static constexpr int PY = ok ? pl_round(Y1 * YB, CW == 2 ? 2 : 4) : 0;
   static constexpr int PZ = ok ? pl_round(Z1 * (Z2 + 1), 4) : 0;  // exchange buffer pitch
+  static constexpr int TY = Y1 * (Y2 + 1), TZ = Z1 * (Z2 + 1);    // twiddle tables
   static constexpr int SCR = CW * PZ;                             // exchange elements per warp
-  static constexpr size_t smem = ok ? ((size_t)(L == LZ ? L : L + LZ) + (size_t)(LZ / 2) * PY + (size_t)NW * SCR) * sizeof(C) : 0;
+  static constexpr size_t smem = ok ? ((size_t)(L == LZ ? TY : TY + TZ) + (size_t)(LZ / 2) * PY + (size_t)NW * SCR) * sizeof(C) : 0;
   static constexpr bool fits = ok && smem <= (size_t)kPlaneSmemMax;
   // blocks per SM the register allocation aims at (shared memory allows as many)
   static constexpr int by_smem = ok ? (int)((size_t)(228 * 1024) / (smem + 1024)) : 1;
@@ -167,7 +168,7 @@ struct PlaneFFT : PlaneCfg<L, LZ, C> {
         HalfDFT<Y1, false, C>::in(v);
         C* dst = slab + (z0 + r) * PY + n2;
 #pragma unroll
-        for (int k1 = 0; k1 < Y1; ++k1) dst[k1 * YB] = k1 ? v[k1] * tw[n2 * k1] : v[k1];
+        for (int k1 = 0; k1 < Y1; ++k1) dst[k1 * YB] = k1 ? v[k1] * tw[k1 * (Y2 + 1) + n2] : v[k1];
       }
     }
     __syncwarp();
@@ -199,7 +200,7 @@ struct PlaneFFT : PlaneCfg<L, LZ, C> {
         for (int k2 = 0; k2 < Y2; ++k2) v[k2] = t[k2];
         DFTL<Y2, L, true, C>::run(v, tw);
 #pragma unroll
-        for (int n2 = 0; n2 < Y2; ++n2) t[n2] = n2 ? v[n2] * conjc(tw[n2 * k1]) : v[n2];
+        for (int n2 = 0; n2 < Y2; ++n2) t[n2] = n2 ? v[n2] * conjc(tw[k1 * (Y2 + 1) + n2]) : v[n2];
       }
     }
     __syncwarp();
@@ -235,10 +236,10 @@ struct PlaneFFT : PlaneCfg<L, LZ, C> {
         C v[Z1];
 #pragma unroll
         for (int n1 = 0; n1 < Z1 / 2; ++n1) v[n1] = src[n1 * Z2 * PY];
-        HalfDFT<Z1, false, C>::in(v);
+        dft_half_in<Z1, LZ, false, C>(v, tw);
         C* dst = scr + col * PZ + n2;
 #pragma unroll
-        for (int k1 = 0; k1 < Z1; ++k1) dst[k1 * (Z2 + 1)] = k1 ? v[k1] * tw[n2 * k1] : v[k1];
+        for (int k1 = 0; k1 < Z1; ++k1) dst[k1 * (Z2 + 1)] = k1 ? v[k1] * tw[k1 * (Z2 + 1) + n2] : v[k1];
       }
     }
   }
@@ -252,7 +253,7 @@ struct PlaneFFT : PlaneCfg<L, LZ, C> {
         C v[Z1];
 #pragma unroll
         for (int k1 = 0; k1 < Z1; ++k1) v[k1] = src[k1 * (Z2 + 1)];
-        HalfDFT<Z1, true, C>::out(v);
+        dft_half_out<Z1, LZ, true, C>(v, nullptr);
         C* dst = slab + n2 * PY + pos(g * CW + col);
 #pragma unroll
         for (int n1 = 0; n1 < Z1 / 2; ++n1) dst[n1 * Z2 * PY] = v[n1];
@@ -267,7 +268,7 @@ struct PlaneFFT : PlaneCfg<L, LZ, C> {
   static __device__ __forceinline__ void b_inverse(C* t, const C* tw, int k1, C (&v)[Z2]) {
     DFTL<Z2, LZ, true, C>::run(v, tw);
 #pragma unroll
-    for (int n2 = 0; n2 < Z2; ++n2) t[n2] = n2 ? v[n2] * conjc(tw[n2 * k1]) : v[n2];
+    for (int n2 = 0; n2 < Z2; ++n2) t[n2] = n2 ? v[n2] * conjc(tw[k1 * (Z2 + 1) + n2]) : v[n2];
   }
 
   // group g of the tabulated kernel spectrum and the unit index of u in it
@@ -311,13 +312,12 @@ __global__ void __launch_bounds__(32 * PlaneCfg<L, LZ, C>::NW, (PlaneCfg<L, LZ, 
   constexpr PlaneOrder o = plane_order<L, LZ, C>();
   constexpr int NT = 32 * F::NW, N = L / 2;
   C* twz = reinterpret_cast<C*>(aim_smem);
-  C* twy = L == LZ ? twz : twz + LZ;
-  C* slab = twy + L;
+  C* twy = L == LZ ? twz : twz + F::TZ;
+  C* slab = twy + F::TY;
   C* scr = slab + (LZ / 2) * F::PY + (threadIdx.x >> 5) * F::SCR;
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-  for (int i = threadIdx.x; i < LZ; i += NT) twz[i] = a.twz[i];
-  if (L != LZ)
-    for (int i = threadIdx.x; i < L; i += NT) twy[i] = a.twy[i];
+  load_twiddles2<F::Z1, F::Z2>(twz, a.twz);
+  if (L != LZ) load_twiddles2<F::Y1, F::Y2>(twy, a.twy);
   if (MODE == PLANE_CONV || MODE == PLANE_FWD)  // the zero padding below the box
     for (int i = a.nz * F::PY + threadIdx.x; i < (LZ / 2) * F::PY; i += NT) slab[i] = C{};
   pdl_wait();

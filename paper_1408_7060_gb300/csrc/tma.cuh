@@ -62,6 +62,13 @@ __device__ __forceinline__ void tma_load_4d(void* dst, const CUtensorMap* map, u
       : "memory");
 }
 
+// 16-byte asynchronous copies into shared memory (per thread groups)
+__device__ __forceinline__ void cp_async16(unsigned dst, const void* src) {
+  asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(dst), "l"(src) : "memory");
+}
+__device__ __forceinline__ void cp_async_commit() { asm volatile("cp.async.commit_group;" ::: "memory"); }
+__device__ __forceinline__ void cp_async_wait() { asm volatile("cp.async.wait_group 0;" ::: "memory"); }
+
 // Host: cuTensorMapEncodeTiled through the runtime's driver entry point (no link to the
 // driver library).  Returns false when the entry point or the encoding is unavailable.
 inline bool encode_tiled_map(CUtensorMap* map, CUtensorMapDataType type, unsigned rank, void* base,

@@ -22,7 +22,12 @@ F_C, BAND = 300e6, 0.3
 SIZES = [("sphere1", 1.0, 8, 16), ("sphere1", 0.2, 16, 16), ("sphere2", 1.0, 16, 32), ("plate", 9, 32, 16),
          ("sphere2", 0.3, 32, 32), ("sphere2", 1.0, 32, 64), ("plate", 14, 64, 16), ("sphere2", 0.15, 64, 32),
          ("sphere2", 0.4, 64, 64), ("sphere2", 1.0, 64, 128), ("plate", 21, 96, 16), ("sphere2", 0.5, 96, 128),
-         ("sphere2", 1.0, 96, 192), ("plate", 30, 128, 16), ("sphere2", 0.4, 128, 128)]
+         ("sphere2", 1.0, 96, 192), ("plate", 30, 128, 16), ("sphere2", 0.4, 128, 128), ("sphere2", 0.72, 96, 144),
+         ("sphere2", 0.53, 128, 144)]
+# grids whose planes do not fit: separate y and z passes (and one whose z-spectral ring would
+# take more than a quarter of the memory)
+SEPARATE = [("sphere2", 0.7, 128, 192, "c64", 3, 3), ("sphere2", 1.0, 128, 256, "c64", 1, 1),
+            ("sphere2", 1.0, 96, 192, "c64", 2, 160), ("sphere2", 0.72, 96, 144, "c128", 1, 1)]
 
 
 def geometry(mesh, size, grid):
@@ -72,14 +77,23 @@ class Plain:
 @pytest.mark.parametrize("mesh,size,grid,lz", SIZES)
 @pytest.mark.parametrize("precision,nb", [("c64", 1), ("c64", 3), ("c128", 2)])
 def test_products_and_sums(mesh, size, grid, lz, precision, nb):
-    from paper_1408_7060_gb300 import AimContext
-
     if grid > 64 and precision == "c128" and lz > 16:
         pytest.skip("the plain evaluation of the larger sizes runs once, in complex64")
+    check(mesh, size, grid, lz, precision, nb, nb)
+
+
+@pytest.mark.parametrize("mesh,size,grid,lz,precision,nb,batch_max", SEPARATE)
+def test_separate_passes(mesh, size, grid, lz, precision, nb, batch_max):
+    check(mesh, size, grid, lz, precision, nb, batch_max)
+
+
+def check(mesh, size, grid, lz, precision, nb, batch_max):
+    from paper_1408_7060_gb300 import AimContext
+
     V, F, h, origin = geometry(mesh, size, grid)
     rng = np.random.default_rng(3)
     with AimContext(V=V, F=F, grid_n=grid, origin=origin, h=h, near_radius=3 * h, dt=0.25 / (BAND * F_C), f_c=F_C,
-                    precision=precision, batch_max=nb) as c:
+                    precision=precision, batch_max=batch_max) as c:
         assert c.info["z_len"] == lz
         plain, ng = Plain(c), c.n_delays
         x = rng.standard_normal((ng, nb, c.ns)) + 1j * rng.standard_normal((ng, nb, c.ns))
