@@ -147,9 +147,10 @@ __global__ void __launch_bounds__(256) k_rows_p2(const C* __restrict__ in, C* __
     C v[R2];
 #pragma unroll
     for (int n2 = 0; n2 < R2; ++n2) v[n2] = t[r * P + k1 * (R2 + 1) + n2];
-    DFTL<R2, L, INV, C>::run(v, tw);
+    if constexpr (INV) dft_half_out<R2, L, INV, C>(v, tw);  // n_out <= L / 2
+    else DFTL<R2, L, INV, C>::run(v, tw);
 #pragma unroll
-    for (int k2 = 0; k2 < R2; ++k2) {
+    for (int k2 = 0; k2 < (INV ? R2 / 2 : R2); ++k2) {
       const int k = k1 + R1 * k2;
       if (k >= out_lo && k < n_out) dst[k] = v[k2];
     }
@@ -245,9 +246,10 @@ __global__ void __launch_bounds__(256) k_cols_p2(const C* __restrict__ in, C* __
     C v[R2];
 #pragma unroll
     for (int n2 = 0; n2 < R2; ++n2) v[n2] = t[(k1 * R2 + n2) * W + l];
-    DFTL<R2, L, INV, C>::run(v, tw);
+    if constexpr (INV) dft_half_out<R2, L, INV, C>(v, tw);  // n_out <= L / 2
+    else DFTL<R2, L, INV, C>::run(v, tw);
 #pragma unroll
-    for (int k2 = 0; k2 < R2; ++k2) {
+    for (int k2 = 0; k2 < (INV ? R2 / 2 : R2); ++k2) {
       const int k = k1 + R1 * k2;
       if (k >= out_lo && k < n_out && l < nw) dst[(long long)k * es_out + l] = v[k2];
     }
