@@ -7,8 +7,9 @@
 //   Bf [b][c][nz][y<L][x<L]   after the forward y-FFT (the slab)
 //   P  [b][c][nz][y<N][x<N]   potentials after the inverse passes
 // The forward z-FFT (length LZ >= 2 nz), the pointwise kernel product and the inverse
-// z-FFT are one kernel per column (k_zconv / k_zrhs), so no 3-D spectrum reaches
-// memory.  Zero padding is pruned in every pass: forward passes read only the non-zero
+// z-FFT are one kernel per column (k_zconv_p2, k_zwarp), so no 3-D spectrum reaches
+// memory.  Where a kx plane fits shared memory (plane.cuh) A is kx-major, [b][c][x<L][nz][y<N],
+// and the y passes join that kernel: Bf is not used.  Zero padding is pruned in every pass: forward passes read only the non-zero
 // inputs, inverse passes write only the needed outputs.
 #pragma once
 #include <algorithm>
@@ -47,7 +48,9 @@ __host__ __device__ constexpr int x_pitch(int L, int yb) {
 // touches are visited (arow: their range per box row, anode: y N + x, aptr: their CSR
 // entries); the operator input is interleaved, xs[k][b], so the BB lanes of a node share
 // its coefficients and gather adjacent values.  With one right-hand side 4 lanes share a
-// node's entries instead (each is an index, coefficient, gather chain).  KXM stores the kx-major grid of the plane
+// node's entries instead (each is an index, coefficient, gather chain).  Both sum a node's
+// entries in the same order (entry e into partial sum e mod 4, then (0 + 2) + (1 + 3)), so a
+// right-hand side's result does not depend on the batch it is in.  KXM stores the kx-major grid of the plane
 // kernel, A[b][c][kx][z][y - ylo] (rows beyond the box written as zeros up to N), runs of
 // YB values; otherwise A[b][c][z][y][kx].
 template <int L, int YB, int BB, bool KXM, class C>
@@ -77,11 +80,18 @@ __global__ void __launch_bounds__(256) k_anterp(const int* __restrict__ arow, co
       const bool on = i < items && (BB == 1 || (b < nb && !(active && !active[b])));
       const int nd = anode[k], yy = nd / N - ylo - y0, x = nd % N;
       const C* vb = xs + b;
-      C a0{}, a1{}, a2{}, a3{};
+      constexpr int NA = 4 / EL;  // partial sums of a lane
+      C a[NA][4] = {};
+      auto add = [&](C* t, const typename Real<C>::F4& w, const C& xv) {
+        t[0] += (R)w.x * xv;
+        t[1] += (R)w.y * xv;
+        t[2] += (R)w.z * xv;
+        t[3] += (R)w.w * xv;
+      };
       int e = on ? aptr[k] + (EL > 1 ? i % EL : 0) : 0;
       const int e1 = on ? aptr[k + 1] : 0;
       // four entries at a time: their index and coefficient loads, then their gathers of
-      // x, are independent and in flight together (the sums keep the entry order)
+      // x, are independent and in flight together
       for (; e + 3 * EL < e1; e += 4 * EL) {
         int j[4];
         typename Real<C>::F4 w[4];
@@ -94,25 +104,19 @@ __global__ void __launch_bounds__(256) k_anterp(const int* __restrict__ arow, co
 #pragma unroll
         for (int u = 0; u < 4; ++u) xv[u] = vb[(size_t)j[u] * nb];
 #pragma unroll
-        for (int u = 0; u < 4; ++u) {
-          a0 += (R)w[u].x * xv[u];
-          a1 += (R)w[u].y * xv[u];
-          a2 += (R)w[u].z * xv[u];
-          a3 += (R)w[u].w * xv[u];
-        }
+        for (int u = 0; u < 4; ++u) add(a[u % NA], w[u], xv[u]);
       }
-      for (; e < e1; e += EL) {
-        const typename Real<C>::F4 w = ncoef[e];
-        const C xv = vb[(size_t)nidx[e] * nb];
-        a0 += (R)w.x * xv;
-        a1 += (R)w.y * xv;
-        a2 += (R)w.z * xv;
-        a3 += (R)w.w * xv;
+      if constexpr (EL == 4) {
+        for (; e < e1; e += EL) add(a[0], ncoef[e], vb[(size_t)nidx[e] * nb]);
+      } else {  // at most 3 are left
+#pragma unroll
+        for (int u = 0; u < 3; ++u)
+          if (e + u < e1) add(a[u], ncoef[e + u], vb[(size_t)nidx[e + u] * nb]);
       }
       if constexpr (EL == 4) {  // lane q of the four keeps component q
         const bool hi = i & 2, od = i & 1;
-        C u0 = hi ? a2 : a0, u1 = hi ? a3 : a1;
-        const C s0 = hi ? a0 : a2, s1 = hi ? a1 : a3;
+        C u0 = hi ? a[0][2] : a[0][0], u1 = hi ? a[0][3] : a[0][1];
+        const C s0 = hi ? a[0][0] : a[0][2], s1 = hi ? a[0][1] : a[0][3];
         u0.x += __shfl_xor_sync(0xffffffffu, s0.x, 2);
         u0.y += __shfl_xor_sync(0xffffffffu, s0.y, 2);
         u1.x += __shfl_xor_sync(0xffffffffu, s1.x, 2);
@@ -122,14 +126,11 @@ __global__ void __launch_bounds__(256) k_anterp(const int* __restrict__ arow, co
         t.x += __shfl_xor_sync(0xffffffffu, s.x, 1);
         t.y += __shfl_xor_sync(0xffffffffu, s.y, 1);
         if (on) in[((i & 3) * YB + yy) * N + x] = t;
-        continue;
+      } else if (on) {
+        C* t = in + (bs * 4 * YB + yy) * N + x;
+#pragma unroll
+        for (int c = 0; c < 4; ++c) t[c * YB * N] = (a[0][c] + a[2][c]) + (a[1][c] + a[3][c]);
       }
-      if (!on) continue;
-      C* t = in + (bs * 4 * YB + yy) * N + x;
-      t[0] = a0;
-      t[YB * N] = a1;
-      t[2 * YB * N] = a2;
-      t[3 * YB * N] = a3;
     }
   }
   __syncthreads();
@@ -1454,12 +1455,13 @@ struct GridOps {
   template <bool KXM>
   static void anterp_as(aim_ctx* c, int nb, const int* active) {
     const int most = std::min(8, L / 2), nyb = nbox(c, 1);
-    // a batch in pairs (two right-hand sides per block share the coefficient loads) where the
-    // pairs fill the chip four times with 4 rows per block (whatever the plan's rows: the order
-    // of the sums depends on this); else 4 lanes per node (3 waves, 1160 unknowns: 8.6 us
-    // against 12.7 in pairs; 64 waves, 7680 unknowns: 533 against 469)
+    // a complex64 batch in pairs (two right-hand sides per block share the coefficient loads)
+    // where the pairs fill the chip four times with 4 rows per block; else 4 lanes per node
+    // (3 waves, 1160 unknowns: 8.6 us against 12.7 in pairs; 64 waves, 7680 unknowns: 533 us against
+    // 469 in pairs with one partial sum per lane).  complex128 keeps the 4 lanes: the pairs' partial sums take too many registers
+    constexpr bool kPairs = std::is_same<C, float2>::value;
     const long long pairs = (long long)((nb + 1) / 2) * c->NZ * ((nyb + 3) / 4);
-    const int bb = nb > 1 && pairs >= 4 * 152 ? 2 : 1;
+    const int bb = kPairs && nb > 1 && pairs >= 4 * 152 ? 2 : 1;
     int yp = ypb(c);
     while (yp > 1 && smem_anterp(yp, bb, KXM) > (size_t)kPlaneSmemMax) yp /= 2;
     with_rows(yp, most, [&](auto yt) {
@@ -1476,8 +1478,10 @@ struct GridOps {
                      (const int*)c->d_nidx, ncoef(c), reinterpret_cast<const C*>(c->d_xs), active, nb,
                      reinterpret_cast<C*>(c->d_A), twiddles(c), c->box_lo[1], nyb, c->NZ);
         };
-        if (bb == 2) go(std::integral_constant<int, 2>{});
-        else go(std::integral_constant<int, 1>{});
+        if constexpr (kPairs) {
+          if (bb == 2) return go(std::integral_constant<int, 2>{});
+        }
+        go(std::integral_constant<int, 1>{});
       }
     });
   }
