@@ -8,7 +8,7 @@ meets the tolerance.
 
 Default workload (the largest configuration that fits one GPU): 4 x 4 array of PEC
 spheres, icosphere subdivision 5 each (491 520 RWG), 1 GHz +-5 %, 384^3 grid (768 x 768
-x 192 transforms: the z transform follows the 72-plane depth of the active box), 16
+x 144 transforms: the z transform follows the 72-plane depth of the active box), 16
 seeded plane waves, tol 1e-5, near-zone SAI preconditioner.  Inputs are synthetic
 (seeded meshes and pulses).  The waves march in chunks of as many as fit in device
 memory next to their history rings (all 16 in one at this workload): every chunk marches
@@ -65,7 +65,7 @@ def kernel_digest(kind):
     """Digest of a kernel's source text and the FFT core it uses: measured DRAM traffic
     is only reported while the kernel is unchanged since the capture."""
     src = open(os.path.join(CSRC, "operator_impl.cuh")).read()
-    names = {"zconv": r"k_zconv(_p2)?", "interp_near": r"k_interp_near", "anterp_xfft": r"k_anterp_rows",
+    names = {"zconv": r"k_zconv(_p2)?", "interp_near": r"k_interp_near", "anterp_xfft": r"k_anterp",
              "zrhs": r"k_zrhs(_spec)?(_tma)?"}
     if kind not in names:
         return None

@@ -225,8 +225,9 @@ int aim_get_info(const aim_ctx* ctx, aim_info* info);
 /* Kernels of the library, for aim_get_profile. */
 enum {
   AIM_K_ANTERP_XFFT = 0, /* anterpolation gather + forward x-FFT                          */
-  AIM_K_YFFT_FWD,        /* forward y-FFT (pruned input)                                   */
-  AIM_K_ZCONV,           /* forward z-FFT, kernel product, inverse z-FFT (immediate term)  */
+  AIM_K_YFFT_FWD,        /* forward y-FFT (pruned input; grids the plane kernel does not hold) */
+  AIM_K_ZCONV,           /* forward z-FFT, kernel product, inverse z-FFT (immediate term); where a
+                            kx plane fits shared memory with both y-FFTs, as one kernel     */
   AIM_K_ZRHS,            /* delay sum over the N_g z-spectra of the history, inverse z-FFT */
                          /* (forward z-FFTs per delay for lengths with a factor 3)        */
   AIM_K_YFFT_INV,        /* inverse y-FFT (pruned output)                                  */
