@@ -1458,7 +1458,7 @@ struct GridOps {
     // a complex64 batch in pairs (two right-hand sides per block share the coefficient loads)
     // where the pairs fill the chip four times with 4 rows per block; else 4 lanes per node
     // (3 waves, 1160 unknowns: 8.6 us against 12.7 in pairs; 64 waves, 7680 unknowns: 533 us against
-    // 469 in pairs with one partial sum per lane).  complex128 keeps the 4 lanes: the pairs' partial sums take too many registers
+    // 469 in pairs with one partial sum per node, about 520 with the four that keep the order).  complex128 keeps the 4 lanes: the pairs' partial sums take too many registers
     constexpr bool kPairs = std::is_same<C, float2>::value;
     const long long pairs = (long long)((nb + 1) / 2) * c->NZ * ((nyb + 3) / 4);
     const int bb = kPairs && nb > 1 && pairs >= 4 * 152 ? 2 : 1;
