@@ -59,15 +59,47 @@ __global__ void __launch_bounds__(kT) k_scale_freq(RcsPhases s, long long n, dou
 // the right-hand side (k_rcs_dirs); the points are the centroid and, for two fractions s,
 // centroid + s (vertex - centroid), so their phases differ from the centroid's by small
 // angles, which need the Taylor series of sine and cosine instead of a range reduction.
-// The kernels are bound by FP64 arithmetic: about 270 operations per face, direction and
+// The 7 points share the rounding of the centroid's phase, which does not average out over
+// them as 7 separately rounded phases would: the centroid is held as an unevaluated sum of two
+// doubles and its phase k r . C likewise (k_rcs_geom, k_rcs_dirs), the second part applied as
+// a rotation to first order.  (Largest error over 40 directions of a 1920-RWG sphere at
+// 300 MHz, of the largest value: 3.6-4.0e-16 with every point evaluated by itself, 7.9-8.9e-16
+// with the rounded phase, 2.8-3.8e-16 with the two parts.)
+// The kernels are bound by FP64 arithmetic: about 280 operations per face, direction and
 // frequency plus 20 per right-hand side (each
 // point evaluated by itself for every right-hand side took about 120 per point: 12.5 ms for
 // 5120 faces, 288 directions, 3 frequencies and 2 waves, 2.3 ms now).
 constexpr int kRcsB = 4;  // right-hand sides per pass
 
+// a + b = result + err (the intrinsics keep a product before it from being contracted into it)
+__device__ __forceinline__ double two_sum(double a, double b, double& err) {
+  const double s = __dadd_rn(a, b), t = __dsub_rn(s, a);
+  err = __dadd_rn(__dsub_rn(a, __dsub_rn(s, t)), __dsub_rn(b, t));
+  return s;
+}
+
+// geo[12][nt]: the centroid C as a sum of two doubles per component, and two of the three
+// vertices relative to it (they add up to zero)
+__global__ void __launch_bounds__(kT) k_rcs_geom(int nt, const int* __restrict__ F, const double* __restrict__ V,
+                                                 double* __restrict__ geo) {
+  const int t = blockIdx.x * kT + threadIdx.x;
+  if (t >= nt) return;
+  for (int d = 0; d < 3; ++d) {
+    const double v0 = V[3 * F[3 * t] + d], v1 = V[3 * F[3 * t + 1] + d], v2 = V[3 * F[3 * t + 2] + d];
+    double e1, e2;
+    const double s = two_sum(two_sum(v0, v1, e1), v2, e2), c = s / 3.0;
+    const double lo = (fma(-3.0, c, s) + (e1 + e2)) / 3.0;
+    geo[(size_t)d * nt + t] = c;
+    geo[(size_t)(3 + d) * nt + t] = lo;
+    geo[(size_t)(6 + d) * nt + t] = (v0 - c) - lo;
+    geo[(size_t)(9 + d) * nt + t] = (v1 - c) - lo;
+  }
+}
+
 // fc[fb][4][nt]: a, b_x, b_y, b_z of every face for right-hand sides b0 .. b0 + nb' - 1 of
 // frequencies f0 .. (fb = (f - f0) kRcsB + (b - b0))
-__global__ void __launch_bounds__(kT) k_rcs_faces(int nt, const int* __restrict__ F, const int* __restrict__ tbk, const double* __restrict__ tbs,
+__global__ void __launch_bounds__(kT) k_rcs_faces(int nt, const double* __restrict__ geo,
+                                                  const int* __restrict__ tbk, const double* __restrict__ tbs,
                                                   const int* __restrict__ tbf, const double* __restrict__ len,
                                                   const double* __restrict__ area, const double* __restrict__ V, int ns,
                                                   int nb, int b0, const double2* __restrict__ spec,
@@ -77,8 +109,6 @@ __global__ void __launch_bounds__(kT) k_rcs_faces(int nt, const int* __restrict_
   double2 m[4] = {};
   if (b0 + bs < nb) {
     const double2* I = spec + ((size_t)f * nb + b0 + bs) * ns;
-    double C[3];
-    for (int d = 0; d < 3; ++d) C[d] = (V[3 * F[3 * t] + d] + V[3 * F[3 * t + 1] + d] + V[3 * F[3 * t + 2] + d]) / 3.0;
     for (int e = 0; e < 3; ++e) {
       const int k = tbk[3 * t + e];
       if (k < 0) continue;
@@ -88,8 +118,9 @@ __global__ void __launch_bounds__(kT) k_rcs_faces(int nt, const int* __restrict_
       m[0].x += x.x;
       m[0].y += x.y;
       for (int d = 0; d < 3; ++d) {
-        m[1 + d].x += x.x * (vf[d] - C[d]);
-        m[1 + d].y += x.y * (vf[d] - C[d]);
+        const double r = (vf[d] - geo[(size_t)d * nt + t]) - geo[(size_t)(3 + d) * nt + t];
+        m[1 + d].x += x.x * r;
+        m[1 + d].y += x.y * r;
       }
     }
   }
@@ -118,7 +149,7 @@ __device__ __forceinline__ void small_sincos(double x, double& s, double& c) {
 
 // part[fb][d][split] = sum over the faces of a split of u . int J e^{jkr.r'} dS'; grid
 // (nd, splits, frequencies).  dirs: [nd][6] (rhat, pol); fk: [n_freq][2] (k, prefactor).
-__global__ void __launch_bounds__(kT) k_rcs_dirs(int nt, const int* __restrict__ F, const double* __restrict__ V,
+__global__ void __launch_bounds__(kT) k_rcs_dirs(int nt, const double* __restrict__ geo,
                                                  const double* __restrict__ area, const double2* __restrict__ fc,
                                                  const double* __restrict__ fk, const double* __restrict__ dirs,
                                                  int nbc, double2* __restrict__ part) {
@@ -133,18 +164,25 @@ __global__ void __launch_bounds__(kT) k_rcs_dirs(int nt, const int* __restrict__
   const double w[2] = {(155.0 - s15) / 1200.0, (155.0 + s15) / 1200.0}, w0 = 9.0 / 40.0;
   double2 acc[kRcsB] = {};
   for (int t = blockIdx.y * kT + threadIdx.x; t < nt; t += ns * kT) {
+    double v[12];
+#pragma unroll
+    for (int i = 0; i < 12; ++i) v[i] = geo[(size_t)i * nt + t];
+    // the vertices relative to the centroid, along the direction and the polarisation
     double ph[3], g[3];
-    for (int i = 0; i < 3; ++i) {
-      const double* v = V + 3 * F[3 * t + i];
-      ph[i] = rd[0] * v[0] + rd[1] * v[1] + rd[2] * v[2];
-      g[i] = u[0] * v[0] + u[1] * v[1] + u[2] * v[2];
+    for (int i = 0; i < 2; ++i) {
+      ph[i] = rd[0] * v[6 + 3 * i] + rd[1] * v[7 + 3 * i] + rd[2] * v[8 + 3 * i];
+      g[i] = u[0] * v[6 + 3 * i] + u[1] * v[7 + 3 * i] + u[2] * v[8 + 3 * i];
     }
-    // (divisions: a rounded 1/3 or k r would shift every phase the same way)
-    const double dc = (ph[0] + ph[1] + ph[2]) / 3.0, gc = (g[0] + g[1] + g[2]) / 3.0, pc = k * dc;
-    for (int i = 0; i < 3; ++i) {
-      ph[i] = k * (ph[i] - dc);
-      g[i] -= gc;
-    }
+    ph[2] = -(ph[0] + ph[1]);
+    g[2] = -(g[0] + g[1]);
+    for (int i = 0; i < 3; ++i) ph[i] *= k;
+    // the centroid's phase, pc + pl
+    const double p0 = __dmul_rn(rd[0], v[0]), p1 = __dmul_rn(rd[1], v[1]), p2 = __dmul_rn(rd[2], v[2]);
+    double t1, t2;
+    const double ps = two_sum(two_sum(p0, p1, t1), p2, t2), pc = __dmul_rn(k, ps);
+    const double pe = (fma(rd[0], v[0], -p0) + fma(rd[1], v[1], -p1) + fma(rd[2], v[2], -p2)) + (t1 + t2) +
+                      (rd[0] * v[3] + rd[1] * v[4] + rd[2] * v[5]);
+    const double pl = fma(k, pe, fma(k, ps, -pc));
     const double big = fmax(fabs(ph[0]), fmax(fabs(ph[1]), fabs(ph[2])));
     double2 X = make_double2(0.0, 0.0), Y = make_double2(w0, 0.0);
     for (int o = 0; o < 2; ++o) {
@@ -165,9 +203,9 @@ __global__ void __launch_bounds__(kT) k_rcs_dirs(int nt, const int* __restrict__
     }
     double sn, cs;
     sincos(pc, &sn, &cs);
-    const double A = area[t];
-    sn *= A;
-    cs *= A;
+    const double A = area[t], c0 = cs;
+    cs = A * fma(-pl, sn, cs);
+    sn = A * fma(pl, c0, sn);
     X = make_double2(X.x * cs - X.y * sn, X.x * sn + X.y * cs);
     Y = make_double2(Y.x * cs - Y.y * sn, Y.x * sn + Y.y * cs);
 #pragma unroll
@@ -265,7 +303,7 @@ size_t rcs_workspace(const aim_ctx* c, int n_freq, int nd, int& nfc, int& splits
   nfc = (int)std::max<size_t>(1, std::min<size_t>((size_t)n_freq, (size_t(64) << 20) / (per_f * sizeof(double2))));
   // splits of the faces so that few directions still occupy every SM
   splits = (int)std::max<long long>(1, std::min<long long>((c->nt + kT - 1) / kT, 608 / ((long long)nd * nfc)));
-  return per_f * nfc + (size_t)nfc * kRcsB * nd * splits;
+  return per_f * nfc + (size_t)nfc * kRcsB * nd * splits + (size_t)6 * c->nt;
 }
 
 void rcs_farfield(aim_ctx* c, int n_freq, int nb, const double2* spec, int nd, const double* dirs, const double* fk,
@@ -273,14 +311,18 @@ void rcs_farfield(aim_ctx* c, int n_freq, int nb, const double2* spec, int nd, c
   int nfc, splits;
   rcs_workspace(c, n_freq, nd, nfc, splits);
   double2* part = work + (size_t)kRcsB * 4 * c->nt * nfc;
+  double* geo = reinterpret_cast<double*>(part + (size_t)nfc * kRcsB * nd * splits);
+  const int tb = (c->nt + kT - 1) / kT;
+  k_rcs_geom<<<tb, kT, 0, c->stream>>>(c->nt, c->d_tri, c->d_v, geo);
+  AIM_CHECK_LAUNCH();
   for (int f0 = 0; f0 < n_freq; f0 += nfc)
     for (int b0 = 0; b0 < nb; b0 += kRcsB) {
       const int nf = std::min(nfc, n_freq - f0), nbc = std::min(kRcsB, nb - b0);
-      k_rcs_faces<<<dim3((c->nt + kT - 1) / kT, nbc, nf), kT, 0, c->stream>>>(
-          c->nt, c->d_tri, c->d_tbk, c->d_tbs, c->d_tbf, c->d_len, c->d_area, c->d_v, c->ns, nb, b0,
+      k_rcs_faces<<<dim3(tb, nbc, nf), kT, 0, c->stream>>>(
+          c->nt, geo, c->d_tbk, c->d_tbs, c->d_tbf, c->d_len, c->d_area, c->d_v, c->ns, nb, b0,
           spec + (size_t)f0 * nb * c->ns, work);
       AIM_CHECK_LAUNCH();
-      k_rcs_dirs<<<dim3(nd, splits, nf), kT, 0, c->stream>>>(c->nt, c->d_tri, c->d_v, c->d_area, work, fk + 2 * f0,
+      k_rcs_dirs<<<dim3(nd, splits, nf), kT, 0, c->stream>>>(c->nt, geo, c->d_area, work, fk + 2 * f0,
                                                              dirs, nbc, part);
       AIM_CHECK_LAUNCH();
       k_rcs_finish<<<dim3((nd + kT - 1) / kT, nbc, nf), kT, 0, c->stream>>>(nd, splits, nb, b0, fk + 2 * f0, part,
