@@ -231,6 +231,7 @@ struct aim_ctx {
   double* d_qp = nullptr;      // [nt][7][3] cubature points
   double* d_qw = nullptr;      // [nt][7] weights * area
   double* d_cent = nullptr;    // [nt][3]
+  double* d_geo = nullptr;     // [12][nt] centroid in two parts and relative vertices (rcs.cu)
   double mean_edge = 0;
   double rmax = 0;             // largest vertex distance from the origin (bounds the time reach
                                // r.u / (c dt) of every cubature point)

@@ -176,6 +176,7 @@ void setup_impl(aim_ctx* c, const aim_mesh* mesh, const aim_grid* grid, double n
   c->d_tbk = upload(c, hm.tbk);
   c->d_tbs = upload(c, hm.tbs);
   c->d_tbf = upload(c, hm.tbf);
+  rcs_tables(c);
   c->d_anchor = upload(c, anchor);
   {
     // interpolation visit order: RWGs sorted by the Morton code of their stencil anchors,
@@ -904,8 +905,8 @@ int aim_rcs(aim_ctx* c, int32_t n_freq, const double* freqs, int32_t nb, const a
     const double2* ds = dev_in(c, spec, n, scratch(c, n, 1));
     const bool dev = is_device_ptr(sigma);
     double* out = dev ? sigma : reinterpret_cast<double*>(scratch(c, no / 2 + 1, 2));
-    int nfc, splits;
-    double2* work = scratch(c, rcs_workspace(c, n_freq, nd, nfc, splits), 3);
+    int nfc, units;
+    double2* work = scratch(c, rcs_workspace(c, n_freq, nd, nfc, units), 3);
     rcs_farfield(c, n_freq, nb, ds, nd, dd, dd + 6 * nd, work, out);
     if (!dev) AIM_CUDA(cudaMemcpyAsync(sigma, out, no * sizeof(double), cudaMemcpyDeviceToHost, c->stream));
     AIM_CUDA(cudaStreamSynchronize(c->stream));

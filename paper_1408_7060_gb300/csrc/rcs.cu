@@ -70,6 +70,7 @@ __global__ void __launch_bounds__(kT) k_scale_freq(RcsPhases s, long long n, dou
 // point evaluated by itself for every right-hand side took about 120 per point: 12.5 ms for
 // 5120 faces, 288 directions, 3 frequencies and 2 waves, 2.3 ms now).
 constexpr int kRcsB = 4;  // right-hand sides per pass
+constexpr int kDirW = 2;  // warps per block of k_rcs_dirs
 
 // a + b = result + err (the intrinsics keep a product before it from being contracted into it)
 __device__ __forceinline__ double two_sum(double a, double b, double& err) {
@@ -147,13 +148,17 @@ __device__ __forceinline__ void small_sincos(double x, double& s, double& c) {
   c = 1.0 + y * q;
 }
 
-// part[fb][d][split] = sum over the faces of a split of u . int J e^{jkr.r'} dS'; grid
-// (nd, splits, frequencies).  dirs: [nd][6] (rhat, pol); fk: [n_freq][2] (k, prefactor).
-__global__ void __launch_bounds__(kT) k_rcs_dirs(int nt, const double* __restrict__ geo,
-                                                 const double* __restrict__ area, const double2* __restrict__ fc,
-                                                 const double* __restrict__ fk, const double* __restrict__ dirs,
-                                                 int nbc, double2* __restrict__ part) {
-  const int d = blockIdx.x, f = blockIdx.z, nd = gridDim.x, ns = gridDim.y;
+// part[fb][d][unit] = sum over the faces of a unit of u . int J e^{jkr.r'} dS'; a unit is 32 m
+// consecutive faces, m to a lane, summed by one warp, and the units are a matter of the mesh
+// alone: a value rounds the same whatever else is in the call.  Grid (nd, blocks, frequencies),
+// a block's warps taking units blockIdx.y kDirW + warp, then gridDim.y kDirW further on.
+// dirs: [nd][6] (rhat, pol); fk: [n_freq][2] (k, prefactor).
+__global__ void __launch_bounds__(32 * kDirW) k_rcs_dirs(int nt, const double* __restrict__ geo,
+                                                         const double* __restrict__ area,
+                                                         const double2* __restrict__ fc, const double* __restrict__ fk,
+                                                         const double* __restrict__ dirs, int nbc, int units, int m,
+                                                         double2* __restrict__ part) {
+  const int d = blockIdx.x, f = blockIdx.z, nd = gridDim.x, lane = threadIdx.x & 31;
   const double* rd = dirs + 6 * d;
   const double k = fk[2 * f];
   const double rp = rd[0] * rd[3] + rd[1] * rd[4] + rd[2] * rd[5];
@@ -162,94 +167,84 @@ __global__ void __launch_bounds__(kT) k_rcs_dirs(int nt, const double* __restric
   const double s15 = 3.8729833462074168852;  // sqrt 15
   const double fr[2] = {1.0 - (6.0 - s15) / 7.0, 1.0 - (6.0 + s15) / 7.0};
   const double w[2] = {(155.0 - s15) / 1200.0, (155.0 + s15) / 1200.0}, w0 = 9.0 / 40.0;
-  double2 acc[kRcsB] = {};
-  for (int t = blockIdx.y * kT + threadIdx.x; t < nt; t += ns * kT) {
-    double v[12];
+  for (int q = blockIdx.y * kDirW + (threadIdx.x >> 5); q < units; q += gridDim.y * kDirW) {
+    const int end = min(nt, (q + 1) * 32 * m);
+    double2 acc[kRcsB] = {};
+    for (int t = q * 32 * m + lane; t < end; t += 32) {
+      double v[12];
 #pragma unroll
-    for (int i = 0; i < 12; ++i) v[i] = geo[(size_t)i * nt + t];
-    // the vertices relative to the centroid, along the direction and the polarisation
-    double ph[3], g[3];
-    for (int i = 0; i < 2; ++i) {
-      ph[i] = rd[0] * v[6 + 3 * i] + rd[1] * v[7 + 3 * i] + rd[2] * v[8 + 3 * i];
-      g[i] = u[0] * v[6 + 3 * i] + u[1] * v[7 + 3 * i] + u[2] * v[8 + 3 * i];
-    }
-    ph[2] = -(ph[0] + ph[1]);
-    g[2] = -(g[0] + g[1]);
-    for (int i = 0; i < 3; ++i) ph[i] *= k;
-    // the centroid's phase, pc + pl
-    const double p0 = __dmul_rn(rd[0], v[0]), p1 = __dmul_rn(rd[1], v[1]), p2 = __dmul_rn(rd[2], v[2]);
-    double t1, t2;
-    const double ps = two_sum(two_sum(p0, p1, t1), p2, t2), pc = __dmul_rn(k, ps);
-    const double pe = (fma(rd[0], v[0], -p0) + fma(rd[1], v[1], -p1) + fma(rd[2], v[2], -p2)) + (t1 + t2) +
-                      (rd[0] * v[3] + rd[1] * v[4] + rd[2] * v[5]);
-    const double pl = fma(k, pe, fma(k, ps, -pc));
-    const double big = fmax(fabs(ph[0]), fmax(fabs(ph[1]), fabs(ph[2])));
-    double2 X = make_double2(0.0, 0.0), Y = make_double2(w0, 0.0);
-    for (int o = 0; o < 2; ++o) {
-      double2 x = make_double2(0, 0), y = make_double2(0, 0);
-      for (int i = 0; i < 3; ++i) {
-        double sn, cs;
-        if (big * fabs(fr[1]) <= 0.5 && big * fabs(fr[0]) <= 0.5) small_sincos(fr[o] * ph[i], sn, cs);
-        else sincos(fr[o] * ph[i], &sn, &cs);
-        y.x += cs;
-        y.y += sn;
-        x.x += g[i] * cs;
-        x.y += g[i] * sn;
+      for (int i = 0; i < 12; ++i) v[i] = geo[(size_t)i * nt + t];
+      // the vertices relative to the centroid, along the direction and the polarisation
+      double ph[3], g[3];
+      for (int i = 0; i < 2; ++i) {
+        ph[i] = rd[0] * v[6 + 3 * i] + rd[1] * v[7 + 3 * i] + rd[2] * v[8 + 3 * i];
+        g[i] = u[0] * v[6 + 3 * i] + u[1] * v[7 + 3 * i] + u[2] * v[8 + 3 * i];
       }
-      X.x += w[o] * fr[o] * x.x;
-      X.y += w[o] * fr[o] * x.y;
-      Y.x += w[o] * y.x;
-      Y.y += w[o] * y.y;
-    }
-    double sn, cs;
-    sincos(pc, &sn, &cs);
-    const double A = area[t], c0 = cs;
-    cs = A * fma(-pl, sn, cs);
-    sn = A * fma(pl, c0, sn);
-    X = make_double2(X.x * cs - X.y * sn, X.x * sn + X.y * cs);
-    Y = make_double2(Y.x * cs - Y.y * sn, Y.x * sn + Y.y * cs);
+      ph[2] = -(ph[0] + ph[1]);
+      g[2] = -(g[0] + g[1]);
+      for (int i = 0; i < 3; ++i) ph[i] *= k;
+      // the centroid's phase, pc + pl
+      const double p0 = __dmul_rn(rd[0], v[0]), p1 = __dmul_rn(rd[1], v[1]), p2 = __dmul_rn(rd[2], v[2]);
+      double t1, t2;
+      const double ps = two_sum(two_sum(p0, p1, t1), p2, t2), pc = __dmul_rn(k, ps);
+      const double pe = (fma(rd[0], v[0], -p0) + fma(rd[1], v[1], -p1) + fma(rd[2], v[2], -p2)) + (t1 + t2) +
+                        (rd[0] * v[3] + rd[1] * v[4] + rd[2] * v[5]);
+      const double pl = fma(k, pe, fma(k, ps, -pc));
+      const double big = fmax(fabs(ph[0]), fmax(fabs(ph[1]), fabs(ph[2])));
+      double2 X = make_double2(0.0, 0.0), Y = make_double2(w0, 0.0);
+      for (int o = 0; o < 2; ++o) {
+        double2 x = make_double2(0, 0), y = make_double2(0, 0);
+        for (int i = 0; i < 3; ++i) {
+          double sn, cs;
+          if (big * fabs(fr[1]) <= 0.5 && big * fabs(fr[0]) <= 0.5) small_sincos(fr[o] * ph[i], sn, cs);
+          else sincos(fr[o] * ph[i], &sn, &cs);
+          y.x += cs;
+          y.y += sn;
+          x.x += g[i] * cs;
+          x.y += g[i] * sn;
+        }
+        X.x += w[o] * fr[o] * x.x;
+        X.y += w[o] * fr[o] * x.y;
+        Y.x += w[o] * y.x;
+        Y.y += w[o] * y.y;
+      }
+      double sn, cs;
+      sincos(pc, &sn, &cs);
+      const double A = area[t], c0 = cs;
+      cs = A * fma(-pl, sn, cs);
+      sn = A * fma(pl, c0, sn);
+      X = make_double2(X.x * cs - X.y * sn, X.x * sn + X.y * cs);
+      Y = make_double2(Y.x * cs - Y.y * sn, Y.x * sn + Y.y * cs);
 #pragma unroll
-    for (int b = 0; b < kRcsB; ++b)
-      if (b < nbc) {
-        const double2* m = fc + (size_t)(f * kRcsB + b) * 4 * nt + t;
-        const double2 a = m[0], bx = m[nt], by = m[2 * (size_t)nt], bz = m[3 * (size_t)nt];
-        const double qx = u[0] * bx.x + u[1] * by.x + u[2] * bz.x, qy = u[0] * bx.y + u[1] * by.y + u[2] * bz.y;
-        acc[b].x += a.x * X.x - a.y * X.y - (qx * Y.x - qy * Y.y);
-        acc[b].y += a.x * X.y + a.y * X.x - (qx * Y.y + qy * Y.x);
-      }
-  }
-  __shared__ double red[kT / 32][2 * kRcsB];
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  for (int b = 0; b < nbc; ++b) {
-    const double2 s = warp_sum_c(acc[b]);
-    if (lane == 0) {
-      red[warp][2 * b] = s.x;
-      red[warp][2 * b + 1] = s.y;
+      for (int b = 0; b < kRcsB; ++b)
+        if (b < nbc) {
+          const double2* c = fc + (size_t)(f * kRcsB + b) * 4 * nt + t;
+          const double2 a = c[0], bx = c[nt], by = c[2 * (size_t)nt], bz = c[3 * (size_t)nt];
+          const double qx = u[0] * bx.x + u[1] * by.x + u[2] * bz.x, qy = u[0] * bx.y + u[1] * by.y + u[2] * bz.y;
+          acc[b].x += a.x * X.x - a.y * X.y - (qx * Y.x - qy * Y.y);
+          acc[b].y += a.x * X.y + a.y * X.x - (qx * Y.y + qy * Y.x);
+        }
     }
-  }
-  __syncthreads();
-  if ((int)threadIdx.x < nbc) {
-    double2 s = make_double2(0, 0);
-    for (int q = 0; q < kT / 32; ++q) {
-      s.x += red[q][2 * threadIdx.x];
-      s.y += red[q][2 * threadIdx.x + 1];
+    for (int b = 0; b < nbc; ++b) {
+      const double2 s = warp_sum_c(acc[b]);
+      if (lane == 0) part[((size_t)(f * kRcsB + b) * nd + d) * units + q] = s;
     }
-    part[((size_t)(f * kRcsB + threadIdx.x) * nd + d) * ns + blockIdx.y] = s;
   }
 }
 
-// sig[f][b0 + bs][d] = prefactor |sum of the splits|^2
-__global__ void __launch_bounds__(kT) k_rcs_finish(int nd, int splits, int nb, int b0, const double* __restrict__ fk,
+// sig[f][b0 + bs][d] = prefactor |sum of the units|^2, a warp per value
+__global__ void __launch_bounds__(kT) k_rcs_finish(int nd, int units, int nb, int b0, const double* __restrict__ fk,
                                                    const double2* __restrict__ part, double* __restrict__ sig) {
-  const int d = blockIdx.x * kT + threadIdx.x, bs = blockIdx.y, f = blockIdx.z;
+  const int d = blockIdx.x * (kT / 32) + (threadIdx.x >> 5), bs = blockIdx.y, f = blockIdx.z, lane = threadIdx.x & 31;
   if (d >= nd) return;
+  const double2* p = part + ((size_t)(f * kRcsB + bs) * nd + d) * units;
   double2 s = make_double2(0, 0);
-  for (int q = 0; q < splits; ++q) {
-    const double2 v = part[((size_t)(f * kRcsB + bs) * nd + d) * splits + q];
-    s.x += v.x;
-    s.y += v.y;
+  for (int q = lane; q < units; q += 32) {
+    s.x += p[q].x;
+    s.y += p[q].y;
   }
-  sig[((size_t)f * nb + b0 + bs) * nd + d] = fk[2 * f + 1] * (s.x * s.x + s.y * s.y);
+  s = warp_sum_c(s);
+  if (lane == 0) sig[((size_t)f * nb + b0 + bs) * nd + d] = fk[2 * f + 1] * (s.x * s.x + s.y * s.y);
 }
 
 int blocks_for(long long n) { return (int)std::min<long long>((n + kT - 1) / kT, 152LL * 16); }
@@ -297,24 +292,35 @@ void rcs_scale(aim_ctx* c, int nb, const RcsPhases& s, double2* acc) {
   AIM_CHECK_LAUNCH();
 }
 
-size_t rcs_workspace(const aim_ctx* c, int n_freq, int nd, int& nfc, int& splits) {
+// Faces per lane of a unit, of the mesh alone: 2, one on meshes of less than 16 blocks, more
+// beyond 2048.  (One face per lane everywhere: the sums over lanes cost 4 % of the work; four:
+// one direction of the 7680-RWG sphere takes 84 us instead of 53.)
+static int rcs_m(const aim_ctx* c) {
+  const int block = 32 * kDirW;
+  return std::max(c->nt >= 16 * block ? 2 : 1, (c->nt + 2048 * block - 1) / (2048 * block));
+}
+
+void rcs_tables(aim_ctx* c) {
+  c->d_geo = (double*)aim_alloc(c, (size_t)12 * c->nt * sizeof(double));
+  k_rcs_geom<<<(c->nt + kT - 1) / kT, kT, 0, c->stream>>>(c->nt, c->d_tri, c->d_v, c->d_geo);
+  AIM_CHECK_LAUNCH();
+}
+
+size_t rcs_workspace(const aim_ctx* c, int n_freq, int nd, int& nfc, int& units) {
   // frequencies per pass: at most 64 MB of face currents (at least one frequency)
   const size_t per_f = (size_t)kRcsB * 4 * c->nt;
   nfc = (int)std::max<size_t>(1, std::min<size_t>((size_t)n_freq, (size_t(64) << 20) / (per_f * sizeof(double2))));
-  // splits of the faces so that few directions still occupy every SM
-  splits = (int)std::max<long long>(1, std::min<long long>((c->nt + kT - 1) / kT, 608 / ((long long)nd * nfc)));
-  return per_f * nfc + (size_t)nfc * kRcsB * nd * splits + (size_t)6 * c->nt;
+  units = (c->nt + 32 * rcs_m(c) - 1) / (32 * rcs_m(c));
+  return per_f * nfc + (size_t)nfc * kRcsB * nd * units;
 }
 
 void rcs_farfield(aim_ctx* c, int n_freq, int nb, const double2* spec, int nd, const double* dirs, const double* fk,
                   double2* work, double* sig) {
-  int nfc, splits;
-  rcs_workspace(c, n_freq, nd, nfc, splits);
+  int nfc, units;
+  rcs_workspace(c, n_freq, nd, nfc, units);
   double2* part = work + (size_t)kRcsB * 4 * c->nt * nfc;
-  double* geo = reinterpret_cast<double*>(part + (size_t)nfc * kRcsB * nd * splits);
+  const double* geo = c->d_geo;
   const int tb = (c->nt + kT - 1) / kT;
-  k_rcs_geom<<<tb, kT, 0, c->stream>>>(c->nt, c->d_tri, c->d_v, geo);
-  AIM_CHECK_LAUNCH();
   for (int f0 = 0; f0 < n_freq; f0 += nfc)
     for (int b0 = 0; b0 < nb; b0 += kRcsB) {
       const int nf = std::min(nfc, n_freq - f0), nbc = std::min(kRcsB, nb - b0);
@@ -322,11 +328,14 @@ void rcs_farfield(aim_ctx* c, int n_freq, int nb, const double2* spec, int nd, c
           c->nt, geo, c->d_tbk, c->d_tbs, c->d_tbf, c->d_len, c->d_area, c->d_v, c->ns, nb, b0,
           spec + (size_t)f0 * nb * c->ns, work);
       AIM_CHECK_LAUNCH();
-      k_rcs_dirs<<<dim3(nd, splits, nf), kT, 0, c->stream>>>(c->nt, geo, c->d_area, work, fk + 2 * f0,
-                                                             dirs, nbc, part);
+      // blocks per value: about 64 for every SM in all
+      const int blocks = (int)std::max<long long>(
+          1, std::min<long long>((units + kDirW - 1) / kDirW, 152 * 64 / ((long long)nd * nf)));
+      k_rcs_dirs<<<dim3(nd, blocks, nf), 32 * kDirW, 0, c->stream>>>(c->nt, geo, c->d_area, work, fk + 2 * f0, dirs,
+                                                                     nbc, units, rcs_m(c), part);
       AIM_CHECK_LAUNCH();
-      k_rcs_finish<<<dim3((nd + kT - 1) / kT, nbc, nf), kT, 0, c->stream>>>(nd, splits, nb, b0, fk + 2 * f0, part,
-                                                                            sig + (size_t)f0 * nb * nd);
+      k_rcs_finish<<<dim3((nd + kT / 32 - 1) / (kT / 32), nbc, nf), kT, 0, c->stream>>>(nd, units, nb, b0, fk + 2 * f0,
+                                                                                      part, sig + (size_t)f0 * nb * nd);
       AIM_CHECK_LAUNCH();
     }
 }

@@ -19,8 +19,10 @@ std::complex<double> basis_spectrum(const TBasis& tb, double w);
 void rcs_dft_accum(aim_ctx* c, int nb, int l, int n_freq, const double* omega, const double2* x, double2* acc);
 // acc[f] *= s.w[f]
 void rcs_scale(aim_ctx* c, int nb, const RcsPhases& s, double2* acc);
+// c->d_geo, with set-up
+void rcs_tables(aim_ctx* c);
 // sig[f][b][d] from spec[f][b][ns]; dirs [nd][6] (rhat, pol), fk [n_freq][2] (k, prefactor),
 // device; work: rcs_workspace elements
-size_t rcs_workspace(const aim_ctx* c, int n_freq, int nd, int& freqs_per_pass, int& splits);
+size_t rcs_workspace(const aim_ctx* c, int n_freq, int nd, int& freqs_per_pass, int& units);
 void rcs_farfield(aim_ctx* c, int n_freq, int nb, const double2* spec, int nd, const double* dirs, const double* fk,
                   double2* work, double* sig);

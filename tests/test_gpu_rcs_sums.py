@@ -3,6 +3,8 @@
 * The phase of a face is as exact as its vertices: on a sphere 64 m from the origin (phases
   of 400 radians at 300 MHz) and on finer spheres around the origin, the error is that of a
   few roundings per face, not of a phase rounded once for all 7 points of the face.
+* A value does not depend on the other directions, frequencies and right-hand sides of the
+  call: bitwise the same alone and among them.
 
 Bound of the first: a face's term (a u.(r - C) - u.b and the sums over its 7 points) passes
 through about 16 roundings of relative size 2^-53, independent from face to face, and the
@@ -85,3 +87,17 @@ def test_phase_of_a_face(sub, f, shift):
     err = np.abs(got - ref) / ref.max()
     print(f"sub {sub} shift {shift}: {float(err.max()):.2e}")
     assert err.max() < 16 * 2.0 ** -53
+
+
+@pytest.mark.parametrize("sub", [1, 3, 4])
+def test_a_value_alone_and_among_others(sub):
+    V, F, c = context(sub)
+    nd, nb, freqs = 37, 6, 1e8 * np.array([1.0, 1.3, 2.0, 3.1, 4.4])
+    with c:
+        rh, pol = random_plane_waves(nd, 4)
+        rng = np.random.default_rng(8)
+        spec = rng.standard_normal((len(freqs), nb, c.ns)) + 1j * rng.standard_normal((len(freqs), nb, c.ns))
+        got = c.rcs(freqs, spec, rh, pol)
+        for f, b, d in ((0, 0, 0), (2, 3, 17), (4, 5, 36)):
+            alone = c.rcs(freqs[f:f + 1], np.ascontiguousarray(spec[f:f + 1, b:b + 1]), rh[d:d + 1], pol[d:d + 1])
+            assert alone[0, 0, 0] == got[f, b, d], (f, b, d)
