@@ -905,9 +905,8 @@ int aim_rcs(aim_ctx* c, int32_t n_freq, const double* freqs, int32_t nb, const a
     const double2* ds = dev_in(c, spec, n, scratch(c, n, 1));
     const bool dev = is_device_ptr(sigma);
     double* out = dev ? sigma : reinterpret_cast<double*>(scratch(c, no / 2 + 1, 2));
-    int nfc, units;
-    double2* work = scratch(c, rcs_workspace(c, n_freq, nd, nfc, units), 3);
-    rcs_farfield(c, n_freq, nb, ds, nd, dd, dd + 6 * nd, work, out);
+    const RcsPlan plan = rcs_plan(c, n_freq, nb, nd);
+    rcs_farfield(c, plan, n_freq, nb, ds, nd, dd, dd + 6 * nd, scratch(c, plan.elems, 3), out);
     if (!dev) AIM_CUDA(cudaMemcpyAsync(sigma, out, no * sizeof(double), cudaMemcpyDeviceToHost, c->stream));
     AIM_CUDA(cudaStreamSynchronize(c->stream));
     return AIM_OK;

@@ -97,13 +97,13 @@ __global__ void __launch_bounds__(kT) k_rcs_geom(int nt, const int* __restrict__
   }
 }
 
-// fc[fb][4][nt]: a, b_x, b_y, b_z of every face for right-hand sides b0 .. b0 + nb' - 1 of
-// frequencies f0 .. (fb = (f - f0) kRcsB + (b - b0))
+// fc[fb][4][nt]: a, b_x, b_y, b_z of every face for right-hand sides b0 .. b0 + gridDim.y - 1 of
+// frequencies f0 .. (fb = (f - f0) sb + (b - b0))
 __global__ void __launch_bounds__(kT) k_rcs_faces(int nt, const double* __restrict__ geo,
                                                   const int* __restrict__ tbk, const double* __restrict__ tbs,
                                                   const int* __restrict__ tbf, const double* __restrict__ len,
                                                   const double* __restrict__ area, const double* __restrict__ V, int ns,
-                                                  int nb, int b0, const double2* __restrict__ spec,
+                                                  int nb, int b0, int sb, const double2* __restrict__ spec,
                                                   double2* __restrict__ fc) {
   const int t = blockIdx.x * kT + threadIdx.x, bs = blockIdx.y, f = blockIdx.z;
   if (t >= nt) return;
@@ -125,7 +125,7 @@ __global__ void __launch_bounds__(kT) k_rcs_faces(int nt, const double* __restri
       }
     }
   }
-  for (int i = 0; i < 4; ++i) fc[((size_t)(f * kRcsB + bs) * 4 + i) * nt + t] = m[i];
+  for (int i = 0; i < 4; ++i) fc[((size_t)(f * sb + bs) * 4 + i) * nt + t] = m[i];
 }
 
 // sin and cos of |x| <= 1/2: Taylor series to x^15 and x^14 (remainders below 1e-18)
@@ -156,8 +156,8 @@ __device__ __forceinline__ void small_sincos(double x, double& s, double& c) {
 __global__ void __launch_bounds__(32 * kDirW) k_rcs_dirs(int nt, const double* __restrict__ geo,
                                                          const double* __restrict__ area,
                                                          const double2* __restrict__ fc, const double* __restrict__ fk,
-                                                         const double* __restrict__ dirs, int nbc, int units, int m,
-                                                         double2* __restrict__ part) {
+                                                         const double* __restrict__ dirs, int nbc, int sb, int units,
+                                                         int m, double2* __restrict__ part) {
   const int d = blockIdx.x, f = blockIdx.z, nd = gridDim.x, lane = threadIdx.x & 31;
   const double* rd = dirs + 6 * d;
   const double k = fk[2 * f];
@@ -218,7 +218,7 @@ __global__ void __launch_bounds__(32 * kDirW) k_rcs_dirs(int nt, const double* _
 #pragma unroll
       for (int b = 0; b < kRcsB; ++b)
         if (b < nbc) {
-          const double2* c = fc + (size_t)(f * kRcsB + b) * 4 * nt + t;
+          const double2* c = fc + (size_t)(f * sb + b) * 4 * nt + t;
           const double2 a = c[0], bx = c[nt], by = c[2 * (size_t)nt], bz = c[3 * (size_t)nt];
           const double qx = u[0] * bx.x + u[1] * by.x + u[2] * bz.x, qy = u[0] * bx.y + u[1] * by.y + u[2] * bz.y;
           acc[b].x += a.x * X.x - a.y * X.y - (qx * Y.x - qy * Y.y);
@@ -227,24 +227,25 @@ __global__ void __launch_bounds__(32 * kDirW) k_rcs_dirs(int nt, const double* _
     }
     for (int b = 0; b < nbc; ++b) {
       const double2 s = warp_sum_c(acc[b]);
-      if (lane == 0) part[((size_t)(f * kRcsB + b) * nd + d) * units + q] = s;
+      if (lane == 0) part[((size_t)(f * sb + b) * nd + d) * units + q] = s;
     }
   }
 }
 
-// sig[f][b0 + bs][d] = prefactor |sum of the units|^2, a warp per value
-__global__ void __launch_bounds__(kT) k_rcs_finish(int nd, int units, int nb, int b0, const double* __restrict__ fk,
-                                                   const double2* __restrict__ part, double* __restrict__ sig) {
+// sig[f][b0 + bs][d], nd of the nd_all directions, = prefactor |sum of the units|^2, a warp per value
+__global__ void __launch_bounds__(kT) k_rcs_finish(int nd, int nd_all, int units, int nb, int b0, int sb,
+                                                   const double* __restrict__ fk, const double2* __restrict__ part,
+                                                   double* __restrict__ sig) {
   const int d = blockIdx.x * (kT / 32) + (threadIdx.x >> 5), bs = blockIdx.y, f = blockIdx.z, lane = threadIdx.x & 31;
   if (d >= nd) return;
-  const double2* p = part + ((size_t)(f * kRcsB + bs) * nd + d) * units;
+  const double2* p = part + ((size_t)(f * sb + bs) * nd + d) * units;
   double2 s = make_double2(0, 0);
   for (int q = lane; q < units; q += 32) {
     s.x += p[q].x;
     s.y += p[q].y;
   }
   s = warp_sum_c(s);
-  if (lane == 0) sig[((size_t)f * nb + b0 + bs) * nd + d] = fk[2 * f + 1] * (s.x * s.x + s.y * s.y);
+  if (lane == 0) sig[((size_t)f * nb + b0 + bs) * nd_all + d] = fk[2 * f + 1] * (s.x * s.x + s.y * s.y);
 }
 
 int blocks_for(long long n) { return (int)std::min<long long>((n + kT - 1) / kT, 152LL * 16); }
@@ -306,36 +307,45 @@ void rcs_tables(aim_ctx* c) {
   AIM_CHECK_LAUNCH();
 }
 
-size_t rcs_workspace(const aim_ctx* c, int n_freq, int nd, int& nfc, int& units) {
-  // frequencies per pass: at most 64 MB of face currents (at least one frequency)
-  const size_t per_f = (size_t)kRcsB * 4 * c->nt;
-  nfc = (int)std::max<size_t>(1, std::min<size_t>((size_t)n_freq, (size_t(64) << 20) / (per_f * sizeof(double2))));
-  units = (c->nt + 32 * rcs_m(c) - 1) / (32 * rcs_m(c));
-  return per_f * nfc + (size_t)nfc * kRcsB * nd * units;
+// Frequencies and directions of a pass: at most 64 MB of face currents and 64 MB of partial sums
+// (at least one of each), for as many right-hand sides as a pass takes.
+RcsPlan rcs_plan(const aim_ctx* c, int n_freq, int nb, int nd) {
+  constexpr size_t kCap = (size_t(64) << 20) / sizeof(double2);
+  RcsPlan p;
+  p.nb = std::min(nb, kRcsB);
+  p.units = (c->nt + 32 * rcs_m(c) - 1) / (32 * rcs_m(c));
+  const size_t per_f = (size_t)p.nb * 4 * c->nt;
+  p.nf = (int)std::max<size_t>(1, std::min<size_t>((size_t)n_freq, kCap / per_f));
+  p.nd = (int)std::max<size_t>(1, std::min<size_t>((size_t)nd, kCap / ((size_t)p.nf * p.nb * p.units)));
+  p.faces = per_f * p.nf;
+  p.elems = p.faces + (size_t)p.nf * p.nb * p.nd * p.units;
+  return p;
 }
 
-void rcs_farfield(aim_ctx* c, int n_freq, int nb, const double2* spec, int nd, const double* dirs, const double* fk,
-                  double2* work, double* sig) {
-  int nfc, units;
-  rcs_workspace(c, n_freq, nd, nfc, units);
-  double2* part = work + (size_t)kRcsB * 4 * c->nt * nfc;
+void rcs_farfield(aim_ctx* c, const RcsPlan& p, int n_freq, int nb, const double2* spec, int nd, const double* dirs,
+                  const double* fk, double2* work, double* sig) {
+  double2* part = work + p.faces;
   const double* geo = c->d_geo;
   const int tb = (c->nt + kT - 1) / kT;
-  for (int f0 = 0; f0 < n_freq; f0 += nfc)
-    for (int b0 = 0; b0 < nb; b0 += kRcsB) {
-      const int nf = std::min(nfc, n_freq - f0), nbc = std::min(kRcsB, nb - b0);
+  for (int f0 = 0; f0 < n_freq; f0 += p.nf)
+    for (int b0 = 0; b0 < nb; b0 += p.nb) {
+      const int nf = std::min(p.nf, n_freq - f0), nbc = std::min(p.nb, nb - b0);
       k_rcs_faces<<<dim3(tb, nbc, nf), kT, 0, c->stream>>>(
-          c->nt, geo, c->d_tbk, c->d_tbs, c->d_tbf, c->d_len, c->d_area, c->d_v, c->ns, nb, b0,
+          c->nt, geo, c->d_tbk, c->d_tbs, c->d_tbf, c->d_len, c->d_area, c->d_v, c->ns, nb, b0, p.nb,
           spec + (size_t)f0 * nb * c->ns, work);
       AIM_CHECK_LAUNCH();
-      // blocks per value: about 64 for every SM in all
-      const int blocks = (int)std::max<long long>(
-          1, std::min<long long>((units + kDirW - 1) / kDirW, 152 * 64 / ((long long)nd * nf)));
-      k_rcs_dirs<<<dim3(nd, blocks, nf), 32 * kDirW, 0, c->stream>>>(c->nt, geo, c->d_area, work, fk + 2 * f0, dirs,
-                                                                     nbc, units, rcs_m(c), part);
-      AIM_CHECK_LAUNCH();
-      k_rcs_finish<<<dim3((nd + kT / 32 - 1) / (kT / 32), nbc, nf), kT, 0, c->stream>>>(nd, units, nb, b0, fk + 2 * f0,
-                                                                                      part, sig + (size_t)f0 * nb * nd);
-      AIM_CHECK_LAUNCH();
+      for (int d0 = 0; d0 < nd; d0 += p.nd) {
+        const int n = std::min(p.nd, nd - d0);
+        // blocks per value: about 64 for every SM in all
+        const int blocks = (int)std::max<long long>(
+            1, std::min<long long>((p.units + kDirW - 1) / kDirW, 152 * 64 / ((long long)n * nf)));
+        k_rcs_dirs<<<dim3(n, blocks, nf), 32 * kDirW, 0, c->stream>>>(c->nt, geo, c->d_area, work, fk + 2 * f0,
+                                                                      dirs + 6 * (size_t)d0, nbc, p.nb, p.units,
+                                                                      rcs_m(c), part);
+        AIM_CHECK_LAUNCH();
+        k_rcs_finish<<<dim3((n + kT / 32 - 1) / (kT / 32), nbc, nf), kT, 0, c->stream>>>(
+            n, nd, p.units, nb, b0, p.nb, fk + 2 * f0, part, sig + (size_t)f0 * nb * nd + d0);
+        AIM_CHECK_LAUNCH();
+      }
     }
 }

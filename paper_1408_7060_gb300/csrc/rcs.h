@@ -21,8 +21,13 @@ void rcs_dft_accum(aim_ctx* c, int nb, int l, int n_freq, const double* omega, c
 void rcs_scale(aim_ctx* c, int nb, const RcsPhases& s, double2* acc);
 // c->d_geo, with set-up
 void rcs_tables(aim_ctx* c);
+// frequencies, right-hand sides and directions of a pass and the elements of its work space
+struct RcsPlan {
+  int nf, nb, nd, units;
+  size_t faces, elems;
+};
+RcsPlan rcs_plan(const aim_ctx* c, int n_freq, int nb, int nd);
 // sig[f][b][d] from spec[f][b][ns]; dirs [nd][6] (rhat, pol), fk [n_freq][2] (k, prefactor),
-// device; work: rcs_workspace elements
-size_t rcs_workspace(const aim_ctx* c, int n_freq, int nd, int& freqs_per_pass, int& units);
-void rcs_farfield(aim_ctx* c, int n_freq, int nb, const double2* spec, int nd, const double* dirs, const double* fk,
-                  double2* work, double* sig);
+// device; work: the plan's elements
+void rcs_farfield(aim_ctx* c, const RcsPlan& p, int n_freq, int nb, const double2* spec, int nd, const double* dirs,
+                  const double* fk, double2* work, double* sig);

@@ -5,6 +5,8 @@
   few roundings per face, not of a phase rounded once for all 7 points of the face.
 * A value does not depend on the other directions, frequencies and right-hand sides of the
   call: bitwise the same alone and among them.
+* The work space stays within twice 64 MB and holds no room for right-hand sides that are not
+  there, and a call of several passes over frequencies and directions gives the same values.
 
 Bound of the first: a face's term (a u.(r - C) - u.b and the sums over its 7 points) passes
 through about 16 roundings of relative size 2^-53, independent from face to face, and the
@@ -101,3 +103,23 @@ def test_a_value_alone_and_among_others(sub):
         for f, b, d in ((0, 0, 0), (2, 3, 17), (4, 5, 36)):
             alone = c.rcs(freqs[f:f + 1], np.ascontiguousarray(spec[f:f + 1, b:b + 1]), rh[d:d + 1], pol[d:d + 1])
             assert alone[0, 0, 0] == got[f, b, d], (f, b, d)
+
+
+def test_work_space_is_bounded():
+    import torch
+
+    from paper_1408_7060_gb300 import abi
+
+    V, F, c = context(1)
+    nd, nf = 9000, 500
+    with c:
+        rh, pol = random_plane_waves(nd, 4)
+        freqs = np.linspace(1e8, 4e8, nf)
+        spec = torch.randn(nf, 1, c.ns, dtype=torch.complex128, device="cuda")
+        out = torch.empty(nf, 1, nd, dtype=torch.float64, device="cuda")
+        before = abi.aim_get_info(c.handle)["device_bytes"]
+        c.rcs(freqs, spec, rh, pol, out=out)
+        assert abi.aim_get_info(c.handle)["device_bytes"] - before < 2 * (64 << 20) + (2 << 20)
+        for f, d in ((0, 0), (nf - 1, nd - 1), (nf // 2, nd // 2)):
+            alone = c.rcs(freqs[f:f + 1], spec[f:f + 1].contiguous(), rh[d:d + 1], pol[d:d + 1])
+            assert float(alone[0, 0, 0]) == float(out[f, 0, d])
