@@ -477,14 +477,14 @@ MeshArgs mesh_args(aim_ctx* c) {
 }  // namespace
 
 // time reach of the cubature points in units of dt: every point r has |r.u| / (c dt) <= this
-// for any unit u (the largest vertex distance from the origin bounds the points)
-static double reach(aim_ctx* c) { return c->rmax / (c->c_med * c->dt); }
+// for any u no longer than len (the largest vertex distance from the origin bounds the points)
+static double reach(aim_ctx* c, double len = 1.0) { return c->rmax * len / (c->c_med * c->dt); }
 
 // shifts an RWG's taps can span: s + w in (-1, Q] with w varying by at most the largest
-// distance between two points of an RWG; 0 where that exceeds kMaxTaps (RWGs of several
-// c dt: the sums go point by point, k_farfield and k_farfield_adj)
-static int tap_count(const aim_ctx* c) {
-  const double n = std::floor(c->tb.Q + 2.0 + c->rwg_span / (c->c_med * c->dt));
+// distance between two points of an RWG times the direction's length; 0 where that exceeds
+// kMaxTaps (RWGs of several c dt: the sums go point by point, k_farfield and k_farfield_adj)
+static int tap_count(const aim_ctx* c, double len) {
+  const double n = std::floor(c->tb.Q + 2.0 + c->rwg_span * len / (c->c_med * c->dt));
   return n <= kMaxTaps ? (int)n : 0;
 }
 
@@ -515,18 +515,19 @@ void adj_excitation_samples_adjoint(aim_ctx* c, const double* khat, const double
 }
 
 // F over n = n0..n0+n_out-1; with accumulate only the n the steps l0..l0+n_steps-1 reach
-void adj_farfield(aim_ctx* c, int nd, const double* d_dirs, int l0, int n_steps, const double2* I, int n0, int n_out,
+void adj_farfield(aim_ctx* c, const FarDirs& dirs, int l0, int n_steps, const double2* I, int n0, int n_out,
                   bool accumulate, double2* F) {
-  DirArgs d{nd, d_dirs, d_dirs + 3 * nd, d_dirs + 6 * nd};
+  const int nd = dirs.nd;
+  DirArgs d{nd, dirs.d, dirs.d + 3 * nd, dirs.d + 6 * nd};
   int na = n0, nb_ = n0 + n_out - 1;
   if (accumulate) {  // A_{n-l} is non-zero only for n - l + w in (-1, Q], |w| <= reach
-    const double u = reach(c);
-    na = std::max(na, (int)std::floor(l0 - u - 1) - 1);
-    nb_ = std::min(nb_, (int)std::ceil(l0 + n_steps - 1 + u + c->tb.Q) + 1);
+    const double u = reach(c, dirs.len);
+    na = (int)std::max<double>(na, std::floor(l0 - u - 1) - 1);
+    nb_ = (int)std::min<double>(nb_, std::ceil(l0 + n_steps - 1 + u + c->tb.Q) + 1);
     if (nb_ < na) return;
   }
   const MeshArgs m = mesh_args(c);
-  const int taps = tap_count(c), n_cnt = nb_ - na + 1;
+  const int taps = tap_count(c, dirs.len), n_cnt = nb_ - na + 1;
   if (taps == 0) {
     k_farfield<<<n_cnt * nd, kT, 0, c->stream>>>(m, d, l0, n_steps, I, n0, na, accumulate ? 1 : 0, F);
     AIM_CHECK_LAUNCH();
@@ -549,10 +550,11 @@ void adj_farfield(aim_ctx* c, int nd, const double* d_dirs, int l0, int n_steps,
   AIM_CHECK_LAUNCH();
 }
 
-void adj_farfield_adjoint(aim_ctx* c, int nd, const double* d_dirs, int l0, int n_steps, int n0, int n_out,
+void adj_farfield_adjoint(aim_ctx* c, const FarDirs& dirs, int l0, int n_steps, int n0, int n_out,
                           const double2* F, bool conj_out, double2* G) {
-  DirArgs d{nd, d_dirs, d_dirs + 3 * nd, d_dirs + 6 * nd};
-  if (const int taps = tap_count(c)) {
+  const int nd = dirs.nd;
+  DirArgs d{nd, dirs.d, dirs.d + 3 * nd, dirs.d + 6 * nd};
+  if (const int taps = tap_count(c, dirs.len)) {
     k_far_adj<<<dim3((c->ns + kAdjK - 1) / kAdjK, (n_steps + kAdjL - 1) / kAdjL), kT,
                 kPairs * taps * 2 * sizeof(double2), c->stream>>>(mesh_args(c), d, l0, n_steps, taps, n0, n_out, F,
                                                                   conj_out ? 1 : 0, G);

@@ -336,6 +336,15 @@ struct aim_ctx {
   std::vector<void*> allocs;
 };
 
+// far-field directions of one call: d [3][nd][3] on the device (directions, two transverse
+// vectors) and the length of the longest direction, at least 1 (infinite where one is not
+// finite), which scales the delays r.r' / (c dt)
+struct FarDirs {
+  int nd;
+  const double* d;
+  double len;
+};
+
 // helpers implemented in api.cu
 void* aim_alloc(aim_ctx* c, size_t bytes);
 

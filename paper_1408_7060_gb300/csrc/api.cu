@@ -406,9 +406,9 @@ void adj_excitation_samples(aim_ctx* c, const double* khat, const double* phat, 
 void adj_excitation_samples_adjoint(aim_ctx* c, const double* khat, const double* phat, int i0, int n_samp,
                                     int l0, int n_steps, const double2* lam, bool conj_lam, bool accumulate,
                                     double2* grad);
-void adj_farfield(aim_ctx* c, int nd, const double* d_dirs, int l0, int n_steps, const double2* I, int n0, int n_out,
+void adj_farfield(aim_ctx* c, const FarDirs& dirs, int l0, int n_steps, const double2* I, int n0, int n_out,
                   bool accumulate, double2* F);
-void adj_farfield_adjoint(aim_ctx* c, int nd, const double* d_dirs, int l0, int n_steps, int n0, int n_out,
+void adj_farfield_adjoint(aim_ctx* c, const FarDirs& dirs, int l0, int n_steps, int n0, int n_out,
                           const double2* F, bool conj_out, double2* G);
 void adj_ensure_near_transpose(aim_ctx* c);
 
@@ -712,8 +712,14 @@ void finish_out(aim_ctx* c, aim_c128* out, const double2* d, size_t n, bool dev)
   if (!dev) AIM_CUDA(cudaMemcpyAsync(out, d, n * sizeof(double2), cudaMemcpyDeviceToHost, c->stream));
   AIM_CUDA(cudaStreamSynchronize(c->stream));
 }
-const double* upload_dirs(aim_ctx* c, int nd, const double* rhat, const double* e1, const double* e2) {
+FarDirs upload_dirs(aim_ctx* c, int nd, const double* rhat, const double* e1, const double* e2) {
   std::vector<double> h((size_t)9 * nd);
+  double len = 1.0;
+  for (int i = 0; i < nd; ++i) {
+    const double* r = rhat + 3 * (size_t)i;
+    const double n = std::sqrt(r[0] * r[0] + r[1] * r[1] + r[2] * r[2]);
+    if (!(n <= len)) len = std::isfinite(n) ? n : HUGE_VAL;
+  }
   for (int i = 0; i < 3 * nd; ++i) {
     h[i] = rhat[i];
     h[3 * nd + i] = e1[i];
@@ -721,7 +727,7 @@ const double* upload_dirs(aim_ctx* c, int nd, const double* rhat, const double* 
   }
   double* d = reinterpret_cast<double*>(scratch(c, (size_t)(9 * nd + 1) / 2 + 1, 4));
   AIM_CUDA(cudaMemcpyAsync(d, h.data(), h.size() * sizeof(double), cudaMemcpyHostToDevice, c->stream));
-  return d;
+  return FarDirs{nd, d, len};
 }
 }  // namespace
 
@@ -764,11 +770,11 @@ int aim_farfield(aim_ctx* c, int32_t nd, const double* rhat, const double* e1, c
     if (nd < 1 || !rhat || !e1 || !e2 || !I || !F || n_steps < 1 || n_out < 1)
       throw AimError{AIM_ERR_ARG, "aim_farfield: bad arguments"};
     const size_t n = (size_t)n_steps * c->ns, nf = (size_t)n_out * nd * 2;
-    const double* dd = upload_dirs(c, nd, rhat, e1, e2);
+    const FarDirs dd = upload_dirs(c, nd, rhat, e1, e2);
     const double2* dI = dev_in(c, I, n, scratch(c, n, 1));
     const bool dev = is_device_ptr(F);
     double2* out = dev ? reinterpret_cast<double2*>(F) : scratch(c, nf, 2);
-    adj_farfield(c, nd, dd, 1, n_steps, dI, n0, n_out, false, out);
+    adj_farfield(c, dd, 1, n_steps, dI, n0, n_out, false, out);
     finish_out(c, F, out, nf, dev);
     return AIM_OK;
   });
@@ -781,11 +787,11 @@ int aim_farfield_adjoint(aim_ctx* c, int32_t nd, const double* rhat, const doubl
     if (nd < 1 || !rhat || !e1 || !e2 || !F || !G || n_steps < 1 || n_out < 1)
       throw AimError{AIM_ERR_ARG, "aim_farfield_adjoint: bad arguments"};
     const size_t n = (size_t)n_steps * c->ns, nf = (size_t)n_out * nd * 2;
-    const double* dd = upload_dirs(c, nd, rhat, e1, e2);
+    const FarDirs dd = upload_dirs(c, nd, rhat, e1, e2);
     const double2* dF = dev_in(c, F, nf, scratch(c, nf, 2));
     const bool dev = is_device_ptr(G);
     double2* out = dev ? reinterpret_cast<double2*>(G) : scratch(c, n, 3);
-    adj_farfield_adjoint(c, nd, dd, 1, n_steps, n0, n_out, dF, false, out);
+    adj_farfield_adjoint(c, dd, 1, n_steps, n0, n_out, dF, false, out);
     finish_out(c, G, out, n, dev);
     return AIM_OK;
   });
@@ -820,7 +826,7 @@ int aim_march_farfield(aim_ctx* c, const double* khat, const double* phat, int32
         n_out < 1 || !F)
       throw AimError{AIM_ERR_ARG, "aim_march_farfield: bad arguments"};
     const size_t nf = (size_t)n_out * nd * 2;
-    const double* dd = upload_dirs(c, nd, rhat, e1, e2);
+    const FarDirs dd = upload_dirs(c, nd, rhat, e1, e2);
     const double2* da = dev_in(c, a, n_samp, scratch(c, n_samp, 0));
     const bool dev = is_device_ptr(F);
     double2* Fd = dev ? reinterpret_cast<double2*>(F) : scratch(c, nf, 2);
@@ -831,7 +837,7 @@ int aim_march_farfield(aim_ctx* c, const double* khat, const double* phat, int32
     StepIO io;
     io.nb = 1;
     io.make_src = [&](int j, double2* b) { adj_excitation_samples(c, khat, phat, i0, n_samp, da, j, 1, b); };
-    io.commit = [&](int j, const double2* x) { adj_farfield(c, nd, dd, j, 1, x, n0, n_out, true, Fd); };
+    io.commit = [&](int j, const double2* x) { adj_farfield(c, dd, j, 1, x, n0, n_out, true, Fd); };
     const int rc = march_steps(c, io, n_steps, tol, stats);
     finish_out(c, F, Fd, nf, dev);
     return rc;
@@ -923,7 +929,7 @@ int aim_march_adjoint_farfield(aim_ctx* c, const double* khat, const double* pha
         n_out < 1 || !F)
       throw AimError{AIM_ERR_ARG, "aim_march_adjoint_farfield: bad arguments"};
     const size_t nf = (size_t)n_out * nd * 2;
-    const double* dd = upload_dirs(c, nd, rhat, e1, e2);
+    const FarDirs dd = upload_dirs(c, nd, rhat, e1, e2);
     const double2* dF = dev_in(c, F, nf, scratch(c, nf, 2));
     const bool dev = is_device_ptr(grad);
     double2* gd = dev ? reinterpret_cast<double2*>(grad) : scratch(c, n_samp, 0);
@@ -937,7 +943,7 @@ int aim_march_adjoint_farfield(aim_ctx* c, const double* khat, const double* pha
     // step j of the transposed march is time step l = n_steps + 1 - j: source conj(G_l),
     // and its solution u gives lam_l = conj(u)
     io.make_src = [&](int j, double2* b) {
-      adj_farfield_adjoint(c, nd, dd, n_steps + 1 - j, 1, n0, n_out, dF, true, b);
+      adj_farfield_adjoint(c, dd, n_steps + 1 - j, 1, n0, n_out, dF, true, b);
     };
     io.commit = [&](int j, const double2* u) {
       adj_excitation_samples_adjoint(c, khat, phat, i0, n_samp, n_steps + 1 - j, 1, u, true, true, gd);

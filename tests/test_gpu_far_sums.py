@@ -1,0 +1,56 @@
+"""The far-field sums and their adjoint on inputs at the edge of what the tap tables hold.
+
+* Directions longer than a unit vector (r.r' / c counts as the delay whatever the length)
+  span more steps than an RWG does along a unit vector: against the plain evaluation of
+  test_gpu_fields, with its tolerance.
+"""
+import math
+
+import numpy as np
+import pytest
+
+from paper_1408_7060_gb300.inputs import random_plane_waves
+from test_gpu_fields import C0, MU0, context, d_basis, surface
+
+pytestmark = pytest.mark.gpu
+
+
+def plain(c, V, F, order, dt, f_c, dirs, I, n0, G_in):
+    """Far field of I [steps][ns] at n0 .. and the adjoint of G_in [n_out][nd][2]."""
+    rh, e1, e2 = dirs
+    r, wS = surface(c, V, F)
+    wc = 2 * math.pi * f_c
+    out, adj = np.zeros_like(G_in), np.zeros_like(I)
+    for d in range(len(rh)):
+        rr = r @ rh[d]
+        ph = -MU0 / (4 * math.pi) * np.exp(1j * wc / C0 * rr)
+        taps = {}
+        for i in range(len(G_in)):
+            for l in range(len(I)):
+                s = n0 + i - (l + 1)
+                if s not in taps:
+                    t = d_basis(s + rr / (C0 * dt), order, dt, wc) * ph
+                    taps[s] = np.stack([(t * (wS @ e1[d])).sum(1), (t * (wS @ e2[d])).sum(1)], 1)
+                out[i, d] += I[l] @ taps[s]
+                adj[l] += taps[s].conj() @ G_in[i, d]
+    return out, adj
+
+
+@pytest.mark.parametrize("order,cdt,length", [(2, 0.8, 1.7), (1, 0.8, 3.0), (3, 0.8, 10.0), (2, 0.8, 0.3)])
+def test_directions_of_any_length(order, cdt, length):
+    from paper_1408_7060_gb300 import abi
+
+    f_c, dt, n0, steps, n_out, nd = 150e6, cdt / C0, -12, 9, 40, 5
+    V, F, c = context(1, order, dt, f_c)
+    with c:
+        rh, e1 = random_plane_waves(nd, 2)
+        e2 = np.cross(rh, e1)
+        rh = rh * np.array([1.0, length, 1.0, length, 0.5])[:, None]
+        rng = np.random.default_rng(5)
+        I = rng.standard_normal((steps, c.ns)) + 1j * rng.standard_normal((steps, c.ns))
+        G_in = rng.standard_normal((n_out, nd, 2)) + 1j * rng.standard_normal((n_out, nd, 2))
+        ref, radj = plain(c, V, F, order, dt, f_c, (rh, e1, e2), I, n0, G_in)
+        got = abi.aim_farfield(c.handle, rh, e1, e2, I, n0, n_out)
+        adj = abi.aim_farfield_adjoint(c.handle, rh, e1, e2, steps, n0, G_in)
+    assert np.abs(got - ref).max() <= 1e-12 * np.abs(ref).max()
+    assert np.abs(adj - radj).max() <= 1e-12 * np.abs(radj).max()
