@@ -348,8 +348,9 @@ __device__ __forceinline__ void far_taps(const MeshArgs& m, const TapCoef& tc, c
   if (side == 0) *first = s0;
 }
 
-// part[split][n - na][d][q] over the RWG tiles of a split; grid (direction tiles, splits,
-// time tiles).  I_l = I[l - l0], l = l0 .. l0 + n_steps - 1.
+// part[split][n - na][d][q] over the RWG tiles of a split (every gridDim.y-th tile: the splits
+// depend on the mesh alone, so that a value rounds the same whatever else is in the call);
+// grid (direction tiles, splits, time tiles).  I_l = I[l - l0], l = l0 .. l0 + n_steps - 1.
 __global__ void __launch_bounds__(kT) k_far_sum(MeshArgs m, DirArgs d, int l0, int n_steps, int taps,
                                                 const double2* __restrict__ I, int na, int n_cnt,
                                                 double2* __restrict__ part) {
@@ -388,18 +389,20 @@ __global__ void __launch_bounds__(kT) k_far_sum(MeshArgs m, DirArgs d, int l0, i
   }
 }
 
-// F (+)= cf * the sum of the splits, n values
-__global__ void __launch_bounds__(kT) k_far_finish(long long n, int splits, double cf, int accumulate,
+// F (+)= cf * the sum of the splits, n values of rows of `row`, rows of F `ldf` apart
+__global__ void __launch_bounds__(kT) k_far_finish(long long n, int splits, double cf, int accumulate, int row, int ldf,
                                                    const double2* __restrict__ part, double2* __restrict__ F) {
   const long long i = blockIdx.x * (long long)kT + threadIdx.x;
   if (i >= n) return;
   double2 s = make_double2(0, 0);
+#pragma unroll 8
   for (int q = 0; q < splits; ++q) {
     s.x += part[q * n + i].x;
     s.y += part[q * n + i].y;
   }
-  const double2 o = accumulate ? F[i] : make_double2(0, 0);
-  F[i] = make_double2(o.x + cf * s.x, o.y + cf * s.y);
+  double2* f = F + (i / row) * ldf + i % row;
+  const double2 o = accumulate ? *f : make_double2(0, 0);
+  *f = make_double2(o.x + cf * s.x, o.y + cf * s.y);
 }
 
 // the adjoint: G_l[k] = cf sum_{n,d,q} conj(A_{n-l}) F[n][d][q]; grid (RWG tiles, step tiles)
@@ -514,6 +517,24 @@ void adj_excitation_samples_adjoint(aim_ctx* c, const double* khat, const double
   AIM_CHECK_LAUNCH();
 }
 
+// Passes of the far field over nd directions and n_cnt times: the splits of the RWG tiles, of
+// the mesh alone (two for every SM where there are as many tiles), and the directions and times
+// of a pass, whose partial sums stay within 64 MB.
+struct FarPass {
+  int splits, nd, n;
+  size_t elems;
+};
+static FarPass far_pass(const aim_ctx* c, int nd, int n_cnt) {
+  constexpr long long kCap = (64LL << 20) / sizeof(double2);
+  FarPass p;
+  p.splits = std::min(304, (c->ns + kFarK - 1) / kFarK);
+  const long long per_d = (long long)p.splits * kFarN * 2;  // one direction, one tile of times
+  p.nd = per_d * nd <= kCap ? nd : (int)(kCap / per_d / kFarD) * kFarD;
+  p.n = (int)std::min<long long>(n_cnt, kCap / (per_d * p.nd) * kFarN);
+  p.elems = (size_t)p.splits * p.nd * 2 * p.n;
+  return p;
+}
+
 // F over n = n0..n0+n_out-1; with accumulate only the n the steps l0..l0+n_steps-1 reach
 void adj_farfield(aim_ctx* c, const FarDirs& dirs, int l0, int n_steps, const double2* I, int n0, int n_out,
                   bool accumulate, double2* F) {
@@ -533,21 +554,25 @@ void adj_farfield(aim_ctx* c, const FarDirs& dirs, int l0, int n_steps, const do
     AIM_CHECK_LAUNCH();
     return;
   }
-  // splits of the RWG tiles that give every SM two blocks, partial sums within 64 MB
-  const long long tiles = (long long)((nd + kFarD - 1) / kFarD) * ((n_cnt + kFarN - 1) / kFarN);
-  const long long n = (long long)n_cnt * nd * 2;
-  const int splits = (int)std::max<long long>(
-      1, std::min<long long>({(c->ns + kFarK - 1) / kFarK, (304 + tiles - 1) / tiles, (4LL << 20) / n}));
-  if (c->far_cap < (size_t)(splits * n)) {
-    c->far_part = (double2*)aim_alloc(c, splits * n * sizeof(double2));
-    c->far_cap = splits * n;
+  const FarPass p = far_pass(c, nd, n_cnt);
+  if (c->far_cap < p.elems) {
+    c->far_part = (double2*)aim_alloc(c, p.elems * sizeof(double2));
+    c->far_cap = p.elems;
   }
-  k_far_sum<<<dim3((nd + kFarD - 1) / kFarD, splits, (n_cnt + kFarN - 1) / kFarN), kT,
-              kPairs * taps * 2 * sizeof(double2), c->stream>>>(m, d, l0, n_steps, taps, I, na, n_cnt, c->far_part);
-  AIM_CHECK_LAUNCH();
-  k_far_finish<<<(int)((n + kT - 1) / kT), kT, 0, c->stream>>>(n, splits, -m.mu / (4.0 * aimc::kPi), accumulate ? 1 : 0,
-                                                               c->far_part, F + (size_t)(na - n0) * nd * 2);
-  AIM_CHECK_LAUNCH();
+  for (int d0 = 0; d0 < nd; d0 += p.nd)
+    for (int i0 = 0; i0 < n_cnt; i0 += p.n) {
+      const int pd = std::min(p.nd, nd - d0), pn = std::min(p.n, n_cnt - i0);
+      const DirArgs dp{pd, d.r + 3 * (size_t)d0, d.e1 + 3 * (size_t)d0, d.e2 + 3 * (size_t)d0};
+      k_far_sum<<<dim3((pd + kFarD - 1) / kFarD, p.splits, (pn + kFarN - 1) / kFarN), kT,
+                  kPairs * taps * 2 * sizeof(double2), c->stream>>>(m, dp, l0, n_steps, taps, I, na + i0, pn,
+                                                                    c->far_part);
+      AIM_CHECK_LAUNCH();
+      const long long n = (long long)pn * pd * 2;
+      k_far_finish<<<(int)((n + kT - 1) / kT), kT, 0, c->stream>>>(
+          n, p.splits, -m.mu / (4.0 * aimc::kPi), accumulate ? 1 : 0, 2 * pd, 2 * nd, c->far_part,
+          F + ((size_t)(na + i0 - n0) * nd + d0) * 2);
+      AIM_CHECK_LAUNCH();
+    }
 }
 
 void adj_farfield_adjoint(aim_ctx* c, const FarDirs& dirs, int l0, int n_steps, int n0, int n_out,

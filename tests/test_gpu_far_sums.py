@@ -3,6 +3,8 @@
 * Directions longer than a unit vector (r.r' / c counts as the delay whatever the length)
   span more steps than an RWG does along a unit vector: against the plain evaluation of
   test_gpu_fields, with its tolerance.
+* A value does not depend on the other directions and times of the call (bitwise), also where
+  the call takes several passes over either.
 """
 import math
 
@@ -54,3 +56,21 @@ def test_directions_of_any_length(order, cdt, length):
         adj = abi.aim_farfield_adjoint(c.handle, rh, e1, e2, steps, n0, G_in)
     assert np.abs(got - ref).max() <= 1e-12 * np.abs(ref).max()
     assert np.abs(adj - radj).max() <= 1e-12 * np.abs(radj).max()
+
+
+@pytest.mark.parametrize("sub,nd,n_out", [(2, 40, 150), (3, 9, 300), (1, 2600, 130), (3, 600, 70)])
+def test_a_value_alone_and_among_others(sub, nd, n_out):
+    from paper_1408_7060_gb300 import abi
+
+    f_c, dt, n0, steps = 150e6, 0.5 / C0, -6, 40
+    V, F, c = context(sub, 2, dt, f_c)
+    with c:
+        rh, e1 = random_plane_waves(nd, 2)
+        e2 = np.cross(rh, e1)
+        rng = np.random.default_rng(5)
+        I = rng.standard_normal((steps, c.ns)) + 1j * rng.standard_normal((steps, c.ns))
+        got = abi.aim_farfield(c.handle, rh, e1, e2, I, n0, n_out)
+        for d, i, k in ((0, 0, 20), (nd - 1, 3, 40), (nd // 2, 11, 1)):
+            one = slice(d, d + 1)
+            alone = abi.aim_farfield(c.handle, rh[one], e1[one], e2[one], I, n0 + i, k)
+            assert np.array_equal(alone[:, 0], got[i:i + k, d]), (d, i, k)
