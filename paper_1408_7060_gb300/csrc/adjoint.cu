@@ -535,6 +535,14 @@ static FarPass far_pass(const aim_ctx* c, int nd, int n_cnt) {
   return p;
 }
 
+// the partial sums that single steps of a march need, at their widest window
+void adj_farfield_reserve(aim_ctx* c, const FarDirs& dirs, int n_out) {
+  if (tap_count(c, dirs.len) == 0) return;
+  const double window = 2.0 * reach(c, dirs.len) + c->tb.Q + 6.0;  // of adj_farfield, one step
+  const FarPass p = far_pass(c, dirs.nd, (int)std::min<double>(n_out, window));
+  aim_grow(c, c->far_part, c->far_cap, p.elems);
+}
+
 // F over n = n0..n0+n_out-1; with accumulate only the n the steps l0..l0+n_steps-1 reach
 void adj_farfield(aim_ctx* c, const FarDirs& dirs, int l0, int n_steps, const double2* I, int n0, int n_out,
                   bool accumulate, double2* F) {
@@ -555,10 +563,7 @@ void adj_farfield(aim_ctx* c, const FarDirs& dirs, int l0, int n_steps, const do
     return;
   }
   const FarPass p = far_pass(c, nd, n_cnt);
-  if (c->far_cap < p.elems) {
-    c->far_part = (double2*)aim_alloc(c, p.elems * sizeof(double2));
-    c->far_cap = p.elems;
-  }
+  aim_grow(c, c->far_part, c->far_cap, p.elems);
   for (int d0 = 0; d0 < nd; d0 += p.nd)
     for (int i0 = 0; i0 < n_cnt; i0 += p.n) {
       const int pd = std::min(p.nd, nd - d0), pn = std::min(p.n, n_cnt - i0);

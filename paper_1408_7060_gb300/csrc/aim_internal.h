@@ -347,6 +347,9 @@ struct FarDirs {
 
 // helpers implemented in api.cu
 void* aim_alloc(aim_ctx* c, size_t bytes);
+void aim_free(aim_ctx* c, void* p, size_t bytes);  // of aim_alloc, before the context goes (synchronises)
+// a buffer of at least n elements: a larger one takes the place of a smaller one
+void aim_grow(aim_ctx* c, double2*& p, size_t& cap, size_t n);
 
 // records events around one kernel launch when profiling is on; counts launches always
 struct KScope {

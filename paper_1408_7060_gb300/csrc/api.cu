@@ -345,6 +345,22 @@ void* aim_alloc(aim_ctx* c, size_t bytes) {
   return p;
 }
 
+void aim_free(aim_ctx* c, void* p, size_t bytes) {
+  if (!p) return;
+  c->allocs.erase(std::find(c->allocs.begin(), c->allocs.end(), p));
+  c->device_bytes -= bytes ? bytes : 16;
+  cudaFree(p);
+}
+
+void aim_grow(aim_ctx* c, double2*& p, size_t& cap, size_t n) {
+  if (n <= cap) return;
+  aim_free(c, p, cap * sizeof(double2));
+  p = nullptr;
+  cap = 0;
+  p = (double2*)aim_alloc(c, n * sizeof(double2));
+  cap = n;
+}
+
 KScope::KScope(aim_ctx* c_, int id_) : c(c_), id(id_) {
   c->prof.launches++;
   c->prof.n[id]++;
@@ -408,6 +424,7 @@ void adj_excitation_samples_adjoint(aim_ctx* c, const double* khat, const double
                                     double2* grad);
 void adj_farfield(aim_ctx* c, const FarDirs& dirs, int l0, int n_steps, const double2* I, int n0, int n_out,
                   bool accumulate, double2* F);
+void adj_farfield_reserve(aim_ctx* c, const FarDirs& dirs, int n_out);
 void adj_farfield_adjoint(aim_ctx* c, const FarDirs& dirs, int l0, int n_steps, int n0, int n_out,
                           const double2* F, bool conj_out, double2* G);
 void adj_ensure_near_transpose(aim_ctx* c);
@@ -702,10 +719,7 @@ const double2* dev_in(aim_ctx* c, const aim_c128* p, size_t n, double2* staging)
   return staging;
 }
 double2* scratch(aim_ctx* c, size_t n, int slot) {
-  if (c->adj_cap[slot] < n) {
-    c->adj_buf[slot] = (double2*)aim_alloc(c, n * sizeof(double2));
-    c->adj_cap[slot] = n;
-  }
+  aim_grow(c, c->adj_buf[slot], c->adj_cap[slot], n);
   return c->adj_buf[slot];
 }
 void finish_out(aim_ctx* c, aim_c128* out, const double2* d, size_t n, bool dev) {
@@ -830,6 +844,7 @@ int aim_march_farfield(aim_ctx* c, const double* khat, const double* phat, int32
     const double2* da = dev_in(c, a, n_samp, scratch(c, n_samp, 0));
     const bool dev = is_device_ptr(F);
     double2* Fd = dev ? reinterpret_cast<double2*>(F) : scratch(c, nf, 2);
+    adj_farfield_reserve(c, dd, n_out);  // nothing is allocated inside the march
     AIM_CUDA(cudaMemsetAsync(Fd, 0, nf * sizeof(double2), c->stream));
     AIM_CUDA(cudaMemsetAsync(c->d_x, 0, (size_t)c->ns * sizeof(double2), c->stream));
     c->l_done = 0;

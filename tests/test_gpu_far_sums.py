@@ -5,6 +5,8 @@
   test_gpu_fields, with its tolerance.
 * A value does not depend on the other directions and times of the call (bitwise), also where
   the call takes several passes over either.
+* The work space of a larger call takes the place of a smaller call's, and a march with the
+  far field allocates nothing after its first step.
 """
 import math
 
@@ -74,3 +76,39 @@ def test_a_value_alone_and_among_others(sub, nd, n_out):
             one = slice(d, d + 1)
             alone = abi.aim_farfield(c.handle, rh[one], e1[one], e2[one], I, n0 + i, k)
             assert np.array_equal(alone[:, 0], got[i:i + k, d]), (d, i, k)
+
+
+def device_bytes(c):
+    from paper_1408_7060_gb300 import abi
+
+    return abi.aim_get_info(c.handle)["device_bytes"]
+
+
+def test_work_space_is_not_left_behind():
+    from paper_1408_7060_gb300 import abi
+
+    held = []
+    for sizes in ((20, 30, 45, 70, 100), (100,)):
+        V, F, c = context(2, 2, 0.5 / C0, 150e6)
+        with c:
+            rh, e1 = random_plane_waves(12, 2)
+            e2 = np.cross(rh, e1)
+            for n in sizes:
+                abi.aim_farfield(c.handle, rh, e1, e2, np.ones((n, c.ns), complex), -3, n + 6)
+            held.append(device_bytes(c))
+    assert held[0] == held[1]
+
+
+def test_a_march_allocates_before_its_first_step():
+    from paper_1408_7060_gb300 import abi
+
+    k, p = random_plane_waves(1, 1)
+    a = np.ones(6, complex)
+    held = []
+    for steps in (1, 12):
+        V, F, c = context(2, 2, 0.5 / C0, 150e6)
+        with c:
+            rh, e1 = random_plane_waves(12, 2)
+            abi.aim_march_farfield(c.handle, k[0], p[0], 0, a, steps, 1e-3, rh, e1, np.cross(rh, e1), 0, 40)
+            held.append(device_bytes(c))
+    assert held[0] == held[1]
