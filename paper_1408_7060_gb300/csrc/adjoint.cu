@@ -290,9 +290,16 @@ __device__ __forceinline__ void load_coef(const MeshArgs& m, TapCoef& tc) {
 }
 
 // the taps of the pair (k, direction d); lanes 2i and 2i + 1 take its two faces.  The first
-// shift goes to *first, taps first .. first + nt - 1 to A[i][q] (zeros for an invalid pair).
+// shift goes to first->s, taps first .. first + nt - 1 to A[i][q] (zeros for an invalid pair),
+// and bit i of first->hit says whether a point lies in the support of tap i: the others are
+// left out of the time sums, where a zero times an infinity would spoil times that the pair
+// does not reach.
+struct FirstTap {
+  int s;
+  unsigned hit;
+};
 __device__ __forceinline__ void far_taps(const MeshArgs& m, const TapCoef& tc, const DirArgs& d, int k, int di,
-                                         bool valid, int nt, double2* A, int* first) {
+                                         bool valid, int nt, double2* A, FirstTap* first) {
   const int side = threadIdx.x & 1, Q = m.tb.Q;
   double2 a1[kMaxTaps] = {}, a2[kMaxTaps] = {};
   double w[7], p1[7], p2[7];
@@ -313,6 +320,7 @@ __device__ __forceinline__ void far_taps(const MeshArgs& m, const TapCoef& tc, c
   }
   wmax = fmax(wmax, __shfl_xor_sync(0xffffffffu, wmax, 1)) / m.cdt;
   const int s0 = valid ? (int)floor(-1.0 - wmax) + 1 : 0;
+  unsigned hit = 0;
   if (valid) {
     const double idt = 1.0 / m.dt;
 #pragma unroll
@@ -326,6 +334,7 @@ __device__ __forceinline__ void far_taps(const MeshArgs& m, const TapCoef& tc, c
         const double v = (s0 + i) + wv, jr = ceil(v);
         if (i < nt && jr >= 0.0 && jr <= (double)Q) {
           const int j = (int)jr;
+          hit |= 1u << i;
           double T = 0, D = 0;
           for (int p = Q; p >= 0; --p) T = T * v + tc.c[j][p];
           for (int p = Q; p >= 1; --p) D = D * v + tc.d[j][p];
@@ -345,7 +354,8 @@ __device__ __forceinline__ void far_taps(const MeshArgs& m, const TapCoef& tc, c
       A[2 * i + side] = make_double2(mine.x + __shfl_xor_sync(0xffffffffu, other.x, 1),
                                      mine.y + __shfl_xor_sync(0xffffffffu, other.y, 1));
     }
-  if (side == 0) *first = s0;
+  hit |= __shfl_xor_sync(0xffffffffu, hit, 1);
+  if (side == 0) *first = FirstTap{s0, hit};
 }
 
 // part[split][n - na][d][q] over the RWG tiles of a split (every gridDim.y-th tile: the splits
@@ -356,7 +366,7 @@ __global__ void __launch_bounds__(kT) k_far_sum(MeshArgs m, DirArgs d, int l0, i
                                                 double2* __restrict__ part) {
   extern __shared__ double2 tap_smem[];  // [pair][taps][2]
   __shared__ TapCoef tc;
-  __shared__ int first[kPairs];
+  __shared__ FirstTap first[kPairs];
   load_coef(m, tc);
   __syncthreads();
   const int pair = threadIdx.x >> 1, d0 = blockIdx.x * kFarD;
@@ -370,9 +380,10 @@ __global__ void __launch_bounds__(kT) k_far_sum(MeshArgs m, DirArgs d, int l0, i
     __syncthreads();
     for (int kk = 0; kk < kFarK && k0 + kk < m.ns; ++kk) {
       const double2* A = tap_smem + (size_t)(dd * kFarK + kk) * taps * 2;
-      const int l = n - first[dd * kFarK + kk] - l0;  // of the first shift
+      const FirstTap ft = first[dd * kFarK + kk];
+      const int l = n - ft.s - l0;  // of the first shift
       for (int i = 0; i < taps; ++i)
-        if (l - i >= 0 && l - i < n_steps) {
+        if ((ft.hit >> i & 1) && l - i >= 0 && l - i < n_steps) {
           const double2 x = I[(size_t)(l - i) * m.ns + k0 + kk], u = cm(A[2 * i], x), v = cm(A[2 * i + 1], x);
           f1.x += u.x;
           f1.y += u.y;
@@ -410,7 +421,7 @@ __global__ void __launch_bounds__(kT) k_far_adj(MeshArgs m, DirArgs d, int l0, i
                                                 const double2* __restrict__ F, int conj_out, double2* __restrict__ G) {
   extern __shared__ double2 tap_smem[];
   __shared__ TapCoef tc;
-  __shared__ int first[kPairs];
+  __shared__ FirstTap first[kPairs];
   load_coef(m, tc);
   __syncthreads();
   const int pair = threadIdx.x >> 1, k0 = blockIdx.x * kAdjK, lb = blockIdx.y * kAdjL;
@@ -424,11 +435,12 @@ __global__ void __launch_bounds__(kT) k_far_adj(MeshArgs m, DirArgs d, int l0, i
     __syncthreads();
     for (int dd = 0; dd < kAdjD && d0 + dd < d.nd; ++dd) {
       const double2* A = tap_smem + (size_t)(dd * kAdjK + kk) * taps * 2;
+      const FirstTap ft = first[dd * kAdjK + kk];
 #pragma unroll
       for (int h = 0; h < kAdjL / 32; ++h) {
-        const int n = l0 + lb + ll + 32 * h + first[dd * kAdjK + kk] - n0;  // of the first shift
+        const int n = l0 + lb + ll + 32 * h + ft.s - n0;  // of the first shift
         for (int i = 0; i < taps; ++i)
-          if (n + i >= 0 && n + i < n_out) {
+          if ((ft.hit >> i & 1) && n + i >= 0 && n + i < n_out) {
             const double2* f = F + ((size_t)(n + i) * d.nd + d0 + dd) * 2;
             const double2 u = cmc(A[2 * i], f[0]), v = cmc(A[2 * i + 1], f[1]);
             acc[h].x += u.x + v.x;

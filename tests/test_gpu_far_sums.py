@@ -7,6 +7,8 @@
   the call takes several passes over either.
 * The work space of a larger call takes the place of a smaller call's, and a march with the
   far field allocates nothing after its first step.
+* An infinite or undefined current (or adjoint input) reaches the times that its support
+  touches and no others, which are those of a call without it, bitwise.
 """
 import math
 
@@ -112,3 +114,35 @@ def test_a_march_allocates_before_its_first_step():
             abi.aim_march_farfield(c.handle, k[0], p[0], 0, a, steps, 1e-3, rh, e1, np.cross(rh, e1), 0, 40)
             held.append(device_bytes(c))
     assert held[0] == held[1]
+
+
+@pytest.mark.parametrize("bad", [np.inf, np.nan])
+@pytest.mark.parametrize("order,cdt", [(1, 0.9), (2, 0.6), (4, 1.2)])
+def test_non_finite_values_stay_within_their_support(order, cdt, bad):
+    from paper_1408_7060_gb300 import abi
+
+    f_c, dt, n0, steps, n_out, nd = 150e6, cdt / C0, -8, 20, 40, 9
+    V, F, c = context(2, order, dt, f_c)
+    with c:
+        r, _ = surface(c, V, F)
+        rh, e1 = random_plane_waves(nd, 2)
+        e2 = np.cross(rh, e1)
+        rng = np.random.default_rng(5)
+        I = rng.standard_normal((steps, c.ns)) + 1j * rng.standard_normal((steps, c.ns))
+        G = rng.standard_normal((n_out, nd, 2)) + 1j * rng.standard_normal((n_out, nd, 2))
+        far = abi.aim_farfield(c.handle, rh, e1, e2, I, n0, n_out)
+        adj = abi.aim_farfield_adjoint(c.handle, rh, e1, e2, steps, n0, G)
+        k, j = 77, 9                                           # the RWG and the step (from 0)
+        I[j, k] = bad
+        got = abi.aim_farfield(c.handle, rh, e1, e2, I, n0, n_out)
+        i, d = 21, 4
+        G[i, d, 1] = bad
+        gadj = abi.aim_farfield_adjoint(c.handle, rh, e1, e2, steps, n0, G)
+    w = r @ rh.T / (C0 * dt)                                   # [ns][14][nd]
+    inside = lambda u: (u > -1) & (u <= order)
+    n = n0 + np.arange(n_out)
+    reach = inside((n - (j + 1))[:, None, None] + w[k][None]).any(1)          # [n_out][nd]
+    assert np.array_equal(got[~reach], far[~reach]) and not np.isfinite(got[reach]).all(-1).any()
+    l = 1 + np.arange(steps)
+    reach = inside((n0 + i - l)[:, None, None] + w[None, :, :, d]).any(-1)    # [steps][ns]
+    assert np.array_equal(gadj[~reach], adj[~reach]) and not np.isfinite(gadj[reach]).any()
