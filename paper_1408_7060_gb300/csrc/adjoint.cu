@@ -416,15 +416,17 @@ __global__ void __launch_bounds__(kT) k_far_finish(long long n, int splits, doub
   *f = make_double2(o.x + cf * s.x, o.y + cf * s.y);
 }
 
-// the adjoint: G_l[k] = cf sum_{n,d,q} conj(A_{n-l}) F[n][d][q]; grid (RWG tiles, step tiles)
+// the adjoint: G_l[k] = cf sum_{n,d,q} conj(A_{n-l}) F[n][d][q]; grid step tiles x RWG tiles,
+// the k_tiles RWG tiles fastest (in one dimension: there may be more step tiles than the others hold)
 __global__ void __launch_bounds__(kT) k_far_adj(MeshArgs m, DirArgs d, int l0, int n_steps, int taps, int n0, int n_out,
-                                                const double2* __restrict__ F, int conj_out, double2* __restrict__ G) {
+                                                int k_tiles, const double2* __restrict__ F, int conj_out,
+                                                double2* __restrict__ G) {
   extern __shared__ double2 tap_smem[];
   __shared__ TapCoef tc;
   __shared__ FirstTap first[kPairs];
   load_coef(m, tc);
   __syncthreads();
-  const int pair = threadIdx.x >> 1, k0 = blockIdx.x * kAdjK, lb = blockIdx.y * kAdjL;
+  const int pair = threadIdx.x >> 1, k0 = blockIdx.x % k_tiles * kAdjK, lb = blockIdx.x / k_tiles * kAdjL;
   const int kk = threadIdx.x >> 5, ll = threadIdx.x & 31;
   double2 acc[kAdjL / 32] = {};
   for (int d0 = 0; d0 < d.nd; d0 += kAdjD) {
@@ -597,9 +599,10 @@ void adj_farfield_adjoint(aim_ctx* c, const FarDirs& dirs, int l0, int n_steps, 
   const int nd = dirs.nd;
   DirArgs d{nd, dirs.d, dirs.d + 3 * nd, dirs.d + 6 * nd};
   if (const int taps = tap_count(c, dirs.len)) {
-    k_far_adj<<<dim3((c->ns + kAdjK - 1) / kAdjK, (n_steps + kAdjL - 1) / kAdjL), kT,
-                kPairs * taps * 2 * sizeof(double2), c->stream>>>(mesh_args(c), d, l0, n_steps, taps, n0, n_out, F,
-                                                                  conj_out ? 1 : 0, G);
+    const int k_tiles = (c->ns + kAdjK - 1) / kAdjK;
+    const long long blocks = (long long)k_tiles * ((n_steps + (long long)kAdjL - 1) / kAdjL);
+    k_far_adj<<<(unsigned)blocks, kT, kPairs * taps * 2 * sizeof(double2), c->stream>>>(
+        mesh_args(c), d, l0, n_steps, taps, n0, n_out, k_tiles, F, conj_out ? 1 : 0, G);
     AIM_CHECK_LAUNCH();
     return;
   }

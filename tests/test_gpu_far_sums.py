@@ -9,6 +9,8 @@
   far field allocates nothing after its first step.
 * An infinite or undefined current (or adjoint input) reaches the times that its support
   touches and no others, which are those of a call without it, bitwise.
+* More steps than a grid dimension holds tiles for: the last steps equal those of a short call
+  with the times moved along, and the far field of the first ones that of a short call.
 """
 import math
 
@@ -146,3 +148,25 @@ def test_non_finite_values_stay_within_their_support(order, cdt, bad):
     l = 1 + np.arange(steps)
     reach = inside((n0 + i - l)[:, None, None] + w[None, :, :, d]).any(-1)    # [steps][ns]
     assert np.array_equal(gadj[~reach], adj[~reach]) and not np.isfinite(gadj[reach]).any()
+
+
+def test_more_steps_than_a_grid_dimension():
+    import torch
+
+    from paper_1408_7060_gb300 import AimContext, abi
+    from paper_1408_7060_gb300.inputs import place_grid, plate_mesh
+
+    V, F = plate_mesh(0.3, 2)
+    h, origin = place_grid(V, 16)
+    steps, tail, nd, n_out = 65535 * 64 + 200, 50, 3, 9
+    with AimContext(V=V, F=F, grid_n=16, origin=origin, h=h, near_radius=-1.0, dt=0.5 / C0, f_c=150e6,
+                    precision="c128") as c:
+        rh, e1 = random_plane_waves(nd, 2)
+        e2 = np.cross(rh, e1)
+        G = torch.randn(n_out, nd, 2, dtype=torch.complex128, device="cuda")
+        long = abi.aim_farfield_adjoint(c.handle, rh, e1, e2, steps, steps - 5, G)
+        short = abi.aim_farfield_adjoint(c.handle, rh, e1, e2, tail, tail - 5, G)
+        assert torch.equal(long[-tail:], short) and float(short.abs().max()) > 0
+        far = abi.aim_farfield(c.handle, rh, e1, e2, long, steps - 40, steps + 30)
+        assert torch.equal(far[:60], abi.aim_farfield(c.handle, rh, e1, e2, long[-90:].contiguous(), 50, 60))
+        assert float(far[60:].abs().max()) == 0.0
