@@ -21,7 +21,7 @@
 
 namespace {
 
-void ensure_ring(aim_ctx* c);
+void alloc_ring(aim_ctx* c);
 
 thread_local std::string g_last_setup_error;
 
@@ -73,6 +73,80 @@ static int z_length(int nz, int L) {
   for (int lz : {16, 32, 64, 128, 144, 192, 256, 768})
     if (lz >= 2 * nz && lz <= L) return lz;
   return L;
+}
+
+// everything that depends on the chosen path: the plane kernel's tables, the ring, the work
+// buffers, the launch plan, and a first run of every kernel
+void setup_work(aim_ctx* c, const aim_opts* opts) {
+  const int B = c->batch_max, ns = c->ns, ng = c->n_delays;
+  const size_t es = grid_elem(c);
+  alloc_ring(c);
+  plane_spectra(c);
+  c->d_A = aim_alloc(c, grid_a_elems(c, B) * es);
+  c->d_Bf = aim_alloc(c, grid_bf_elems(c, B) * es);
+  c->d_P = aim_alloc(c, grid_p_elems(c, B) * es);
+  c->d_xs = aim_alloc(c, (size_t)B * ns * es);
+  c->d_xd = (double2*)aim_alloc(c, (size_t)B * ns * sizeof(double2));
+  c->d_vf = (float2*)aim_alloc(c, (size_t)B * ns * sizeof(float2));
+  const size_t vec = (size_t)B * ns * sizeof(double2);
+  c->d_iring = (double2*)aim_alloc(c, (size_t)ng * vec);
+  c->d_x = (double2*)aim_alloc(c, vec);
+  c->d_y = (double2*)aim_alloc(c, vec);
+  c->d_b = (double2*)aim_alloc(c, vec);
+  c->d_r = (double2*)aim_alloc(c, vec);
+  c->d_w = (double2*)aim_alloc(c, vec);
+  c->d_err = (int*)aim_alloc(c, sizeof(int));
+  AIM_CUDA(cudaMemsetAsync(c->d_err, 0, sizeof(int), c->stream));
+  if (c->d_sai) c->d_u = (double2*)aim_alloc(c, vec);
+  c->d_V = (double2*)aim_alloc(c, (size_t)(c->restart + 1) * vec);
+  c->d_hist = (double2*)aim_alloc(c, (size_t)ng * vec);
+  c->d_exc = (double*)aim_alloc(c, (size_t)B * 6 * sizeof(double));
+  if (c->refine > 0) {
+    // FP64 grid buffers for the refinement residual, for as many right-hand sides at a
+    // time as fit in 8 GiB (at least one)
+    const size_t per = (grid_a_elems(c, 1) + grid_bf_elems(c, 1) + grid_p_elems(c, 1)) * sizeof(double2);
+    c->ref_nb = (int)std::max<size_t>(1, std::min<size_t>((size_t)B, (size_t(8) << 30) / per));
+    const int rb = c->ref_nb;
+    c->d_A64 = aim_alloc(c, grid_a_elems(c, rb) * sizeof(double2));
+    c->d_Bf64 = aim_alloc(c, grid_bf_elems(c, rb) * sizeof(double2));
+    c->d_P64 = aim_alloc(c, grid_p_elems(c, rb) * sizeof(double2));
+    c->d_xs64 = aim_alloc(c, (size_t)rb * ns * sizeof(double2));
+    c->d_rn = (double*)aim_alloc(c, 2 * (size_t)B * sizeof(double));
+    if (!c->h_rn) AIM_CUDA(cudaMallocHost(&c->h_rn, 2 * (size_t)B * sizeof(double)));
+  }
+  gmres_alloc(c);
+  if (op_plane(c)) {  // several delays of aim_rhs at a time; without the memory, one at a time
+    const size_t per = grid_a_elems(c, 1) * es;
+    const int cap = (int)std::min<size_t>((size_t)ng * B, kBatchBytes / per);
+    if (cap >= 2 * B || (B == 1 && cap >= 2)) {
+      try {
+        c->d_Ab = aim_alloc(c, cap * per);
+        c->d_xsb = aim_alloc(c, (size_t)cap * ns * es);
+        c->batch_cap = cap;
+      } catch (const AimError&) {
+        aim_free(c, c->d_Ab, cap * per);
+        c->d_Ab = nullptr;
+      }
+    }
+  }
+  if (opts->autotune < 0 || opts->autotune > 2) throw AimError{AIM_ERR_ARG, "aim_setup: autotune must be 0, 1 or 2"};
+  op_autotune(c, opts->autotune);
+  // run every operator kernel once outside any stream capture: sets the shared-memory
+  // attributes of each instantiation and surfaces launch errors at setup
+  AIM_CUDA(cudaMemsetAsync(c->d_x, 0, vec, c->stream));
+  op_apply(c, 0, 1, c->d_x, nullptr, nullptr, 1.0, nullptr, c->d_y);
+  if (c->refine > 0) op_apply_f64(c, 0, 1, c->d_x, nullptr, 1.0, c->d_y);
+  op_forward_slab(c, 1, c->d_x, c->d_ring);
+  {
+    SlabList sl{};
+    sl.p[0] = c->d_ring;
+    sl.m[0] = 1;
+    sl.n = 1;
+    NearList nl{};
+    op_apply_rhs(c, 1, sl, c->d_ring, nl, nullptr, 1.0, c->d_y);
+  }
+  AIM_CUDA(cudaStreamSynchronize(c->stream));
+  c->prof = ProfState();
 }
 
 void setup_impl(aim_ctx* c, const aim_mesh* mesh, const aim_grid* grid, double near_radius, double dt,
@@ -211,88 +285,32 @@ void setup_impl(aim_ctx* c, const aim_mesh* mesh, const aim_grid* grid, double n
     while ((1 << c->blk_P) < c->n_delays) ++c->blk_P;  // 2^P >= N_g (<= 32)
   }
 
-  // work buffers
-  const int B = c->batch_max, ns = c->ns, ng = c->n_delays;
-  const size_t es = grid_elem(c);
-  c->d_A = aim_alloc(c, grid_a_elems(c, B) * es);
-  c->d_Bf = aim_alloc(c, grid_bf_elems(c, B) * es);
-  c->d_P = aim_alloc(c, grid_p_elems(c, B) * es);
-  if (op_plane(c)) {
-    const size_t per = grid_a_elems(c, 1) * es;
-    const int cap = (int)std::min<size_t>((size_t)ng * B, kBatchBytes / per);
-    if (cap >= 2 * B || (B == 1 && cap >= 2)) {
-      c->d_Ab = aim_alloc(c, cap * per);
-      c->d_xsb = aim_alloc(c, (size_t)cap * ns * es);
-      c->batch_cap = cap;
-    }
+  plane_choose(c);
+  const size_t mark = c->allocs.size(), bytes = c->device_bytes;
+  try {
+    setup_work(c, opts);
+  } catch (const AimError& e) {
+    // Out of memory with z-spectra of a factor-3 z length: the ring of x/y-transformed slabs is
+    // the smaller one, so the set-up is made again with the separate passes.
+    if (e.code != AIM_ERR_OOM || !op_plane(c) || (c->LZ & (c->LZ - 1)) == 0) throw;
+    AIM_CUDA(cudaStreamSynchronize(c->stream));
+    for (size_t i = mark; i < c->allocs.size(); ++i) cudaFree(c->allocs[i]);
+    c->allocs.resize(mark);
+    c->device_bytes = bytes;
+    c->d_Ab = c->d_xsb = nullptr;
+    c->batch_cap = 0;
+    gmres_free_host(c);
+    (c->precision == AIM_C64 ? c->plane : c->plane64) = false;
+    setup_work(c, opts);
   }
-  c->d_xs = aim_alloc(c, (size_t)B * ns * es);
-  c->d_xd = (double2*)aim_alloc(c, (size_t)B * ns * sizeof(double2));
-  c->d_vf = (float2*)aim_alloc(c, (size_t)B * ns * sizeof(float2));
-  const size_t vec = (size_t)B * ns * sizeof(double2);
-  c->d_iring = (double2*)aim_alloc(c, (size_t)ng * vec);
-  c->d_x = (double2*)aim_alloc(c, vec);
-  c->d_y = (double2*)aim_alloc(c, vec);
-  c->d_b = (double2*)aim_alloc(c, vec);
-  c->d_r = (double2*)aim_alloc(c, vec);
-  c->d_w = (double2*)aim_alloc(c, vec);
-  c->d_err = (int*)aim_alloc(c, sizeof(int));
-  AIM_CUDA(cudaMemsetAsync(c->d_err, 0, sizeof(int), c->stream));
-  if (c->d_sai) c->d_u = (double2*)aim_alloc(c, vec);
-  c->d_V = (double2*)aim_alloc(c, (size_t)(c->restart + 1) * vec);
-  c->d_hist = (double2*)aim_alloc(c, (size_t)ng * vec);
-  c->d_exc = (double*)aim_alloc(c, (size_t)B * 6 * sizeof(double));
-  if (c->refine > 0) {
-    // FP64 grid buffers for the refinement residual, for as many right-hand sides at a
-    // time as fit in 8 GiB (at least one)
-    const size_t per = (grid_a_elems(c, 1) + grid_bf_elems(c, 1) + grid_p_elems(c, 1)) * sizeof(double2);
-    c->ref_nb = (int)std::max<size_t>(1, std::min<size_t>((size_t)B, (size_t(8) << 30) / per));
-    const int rb = c->ref_nb;
-    c->d_A64 = aim_alloc(c, grid_a_elems(c, rb) * sizeof(double2));
-    c->d_Bf64 = aim_alloc(c, grid_bf_elems(c, rb) * sizeof(double2));
-    c->d_P64 = aim_alloc(c, grid_p_elems(c, rb) * sizeof(double2));
-    c->d_xs64 = aim_alloc(c, (size_t)rb * ns * sizeof(double2));
-    c->d_rn = (double*)aim_alloc(c, 2 * (size_t)B * sizeof(double));
-    AIM_CUDA(cudaMallocHost(&c->h_rn, 2 * (size_t)B * sizeof(double)));
-  }
-  gmres_alloc(c);
-  if (opts->autotune < 0 || opts->autotune > 2) throw AimError{AIM_ERR_ARG, "aim_setup: autotune must be 0, 1 or 2"};
-  op_autotune(c, opts->autotune);
-  // run every operator kernel once outside any stream capture: sets the shared-memory
-  // attributes of each instantiation and surfaces launch errors at setup
-  AIM_CUDA(cudaMemsetAsync(c->d_x, 0, vec, c->stream));
-  op_apply(c, 0, 1, c->d_x, nullptr, nullptr, 1.0, nullptr, c->d_y);
-  if (c->refine > 0) op_apply_f64(c, 0, 1, c->d_x, nullptr, 1.0, c->d_y);
-  ensure_ring(c);
-  op_forward_slab(c, 1, c->d_x, c->d_ring);
-  {
-    SlabList sl{};
-    sl.p[0] = c->d_ring;
-    sl.m[0] = 1;
-    sl.n = 1;
-    NearList nl{};
-    op_apply_rhs(c, 1, sl, c->d_ring, nl, nullptr, 1.0, c->d_y);
-  }
-  AIM_CUDA(cudaStreamSynchronize(c->stream));
-  c->prof = ProfState();
 }
 
-// the spectral history ring (N_g forward slabs per right-hand side) is the largest
-// buffer; it is allocated on the first call that needs it
-void ensure_ring(aim_ctx* c) {
-  if (c->d_ring) return;
+// the spectral history ring (N_g forward slabs per right-hand side), the largest buffer
+void alloc_ring(aim_ctx* c) {
   // blocked sums: 2^P >= N_g source slots and 2^(P+1) pending slots
   const int nslots = c->rhs_blocked ? 1 << c->blk_P : c->n_delays;
-  size_t slab = op_slab_bytes(c, c->batch_max);
-  try {
-    c->d_ring = aim_alloc(c, (size_t)nslots * slab);
-  } catch (const AimError&) {
-    // a factor-3 z length: the ring of x/y-transformed slabs is the smaller one
-    if (!op_plane(c) || (c->LZ & (c->LZ - 1)) == 0) throw;
-    (c->precision == AIM_C64 ? c->plane : c->plane64) = false;
-    slab = op_slab_bytes(c, c->batch_max);
-    c->d_ring = aim_alloc(c, (size_t)nslots * slab);
-  }
+  const size_t slab = op_slab_bytes(c, c->batch_max);
+  c->d_ring = aim_alloc(c, (size_t)nslots * slab);
   if (c->rhs_blocked) {
     c->d_pend = aim_alloc(c, ((size_t)2 << c->blk_P) * slab);
     AIM_CUDA(cudaMemsetAsync(c->d_pend, 0, ((size_t)2 << c->blk_P) * slab, c->stream));
@@ -577,7 +595,6 @@ int aim_rhs(aim_ctx* c, int32_t l, int32_t nb, const aim_c128* hist, aim_c128* r
     const int ng = c->n_delays;
     const size_t n = (size_t)nb * c->ns;
     const double2* hs = stage_in(c, hist, (size_t)ng * n, c->d_hist);
-    ensure_ring(c);
     const size_t slab = op_slab_bytes(c, c->batch_max);
     SlabList sl{};
     NearList nl{};
@@ -1075,7 +1092,6 @@ static int march_steps(aim_ctx* c, const StepIO& io, int n_steps, double tol, ai
   const size_t n = (size_t)nb * ns;
   const size_t slab = op_slab_bytes(c, B);
   const bool dev_out = currents && is_device_ptr(currents);
-  ensure_ring(c);
   cudaEvent_t ev[3];
   for (auto& e : ev) AIM_CUDA(cudaEventCreate(&e));
   std::vector<int> its(nb);

@@ -29,7 +29,9 @@ void body_tune(aim_ctx*);
 template <class C>
 void body_plan_fill(aim_ctx*);
 template <class C>
-bool plane_tables(aim_ctx*, int, const C*, C**);
+bool plane_holds(const aim_ctx*);
+template <class C>
+C* plane_tables(aim_ctx*, int, const C*);
 
 void op_apply(aim_ctx* c, int m, int nb, const double2* v, const double2* dinv, const double2* base, double sign,
               const int* active, double2* y, VecSel vin, VecSel yout) {
@@ -210,23 +212,26 @@ bool op_plane(const aim_ctx* c) { return c->precision == AIM_C64 ? c->plane : c-
 
 // A plane kept in shared memory saves the padded slab's four trips through memory, so every
 // size that fits uses it.  Its history ring holds z-spectra; for a z length with a factor 3
-// that is LZ / NZ times the bytes of the x/y-transformed ring, so there it also has to leave
-// three quarters of the free memory to everything else.
-void plane_setup(aim_ctx* c) {
-  const int nm = c->n_delays + 1;
+// that is LZ / NZ times the bytes of the x/y-transformed ring, so there the ring also has to
+// stay within 64 GiB (the rest of the memory, and as much again for a second context, stay
+// free): at 96^3 with 7 delays, up to 43 waves.  Delayed sum of 96^3, 7 delays, 4 waves: 5.1 ms
+// with the plane, 8.4 ms without.  The rule asks nothing of the memory that happens to be free,
+// so that equal set-ups run equal kernels; a set-up that does not find the memory for the plane
+// path is made again without it (setup_work).
+constexpr size_t kPlaneRingMax = size_t(64) << 30;
+
+void plane_choose(aim_ctx* c) {
   const bool c64 = c->precision == AIM_C64;
-  if ((c->LZ & (c->LZ - 1)) != 0) {
-    size_t free = 0, total = 0;
-    AIM_CUDA(cudaMemGetInfo(&free, &total));
-    const size_t ring = (size_t)c->n_delays * c->batch_max * 4 * c->L * c->L * c->LZ * (c64 ? 8 : 16);
-    if (ring > free / 4) return;
-  }
-  if (c64) {
-    c->plane = plane_tables<float2>(c, nm, c->d_kspecf, &c->d_planef);
-    if (c->refine > 0) c->plane64 = plane_tables<double2>(c, 1, c->d_kspec, &c->d_plane);
-  } else {
-    c->plane64 = plane_tables<double2>(c, nm, c->d_kspec, &c->d_plane);
-  }
+  const size_t ring = (size_t)c->n_delays * c->batch_max * 4 * c->L * c->L * c->LZ * (c64 ? 8 : 16);
+  const bool own = (c->LZ & (c->LZ - 1)) == 0 || ring <= kPlaneRingMax;
+  c->plane = c64 && own && plane_holds<float2>(c);
+  c->plane64 = c64 ? c->refine > 0 && plane_holds<double2>(c) : own && plane_holds<double2>(c);
+}
+
+void plane_spectra(aim_ctx* c) {
+  const int nm = c->n_delays + 1;
+  if (c->plane) c->d_planef = plane_tables<float2>(c, nm, c->d_kspecf);
+  if (c->plane64) c->d_plane = plane_tables<double2>(c, c->precision == AIM_C64 ? 1 : nm, c->d_kspec);
 }
 
 size_t grid_a_elems(const aim_ctx* c, int nb) { return (size_t)nb * 4 * c->NZ * c->N * c->L; }

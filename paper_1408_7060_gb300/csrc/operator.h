@@ -74,8 +74,9 @@ void op_excitation(aim_ctx* c, int nb, const double* d_kp, double sigma, double 
 int op_kernel_count(const aim_ctx* c);
 // the context's own operator runs the plane kernel on kx-major grids
 bool op_plane(const aim_ctx* c);
-// decide that, and tabulate the plane kernel's spectra (after the octants)
-void plane_setup(aim_ctx* c);
+// decide that, from the sizes alone, and tabulate the plane kernel's spectra (after the octants)
+void plane_choose(aim_ctx* c);
+void plane_spectra(aim_ctx* c);
 // one launch of the plane kernel (mode: PLANE_* of plane.cuh) on d_A, for `slots` spectra of
 // nb right-hand sides each, slot_elems apart from S on
 template <class C>

@@ -71,24 +71,34 @@ void plane_rhs(aim_ctx* c, int nb, const SlabList& sl, C* S) {
   plane_launch<C>(c, nb, PLANE_INV, 0, nullptr, S, 1, 0);
 }
 
-// Whether grids of this size run the plane kernel, and its spectra of nm delays from the
-// octants.  Returns false where a plane does not fit shared memory.
+// Whether a plane of this context's size fits shared memory, and the order of its spectra.
 template <class C>
-bool plane_tables(aim_ctx* c, int nm, const C* oct, C** out) {
+static bool plane_order_of(const aim_ctx* c, PlaneOrder* o) {
   if (c->L > 256) return false;
   bool fits = false;
-  PlaneOrder o{};
   plane_with_l(c->L, [&](auto lt) {
     constexpr int L = decltype(lt)::value;
     plane_with_z<L>(c->LZ, [&](auto zt) {
       constexpr int LZ = decltype(zt)::value;
       if constexpr (plane_fits<L, LZ, C>()) {
         fits = true;
-        o = plane_order<L, LZ, C>();
+        *o = plane_order<L, LZ, C>();
       }
     });
   });
-  if (!fits) return false;
+  return fits;
+}
+template <class C>
+bool plane_holds(const aim_ctx* c) {
+  PlaneOrder o{};
+  return plane_order_of<C>(c, &o);
+}
+
+// The plane kernel's spectra of nm delays from the octants.
+template <class C>
+C* plane_tables(aim_ctx* c, int nm, const C* oct) {
+  PlaneOrder o{};
+  if (!plane_order_of<C>(c, &o)) throw AimError{AIM_ERR_ARG, "plane kernel: the plane does not fit shared memory"};
   const size_t per = plane_spec_elems(o);
   C* g = (C*)aim_alloc(c, (size_t)nm * per * sizeof(C));
   const size_t no = 2 * (size_t)(c->N + 1) * (c->N + 1) * (c->LZ / 2 + 1);
@@ -97,6 +107,5 @@ bool plane_tables(aim_ctx* c, int nm, const C* oct, C** out) {
         o, oct + m * no, g + m * per);
     AIM_CHECK_LAUNCH();
   }
-  *out = g;
-  return true;
+  return g;
 }

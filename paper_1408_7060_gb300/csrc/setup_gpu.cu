@@ -18,7 +18,6 @@
 #include "aim_internal.h"
 #include "fft_kernels.cuh"
 #include "setup_host.h"
-#include "operator.h"
 #include "setup_gpu.h"
 #include "tbasis.cuh"
 
@@ -719,7 +718,6 @@ void setup_device_tables(aim_ctx* c, HostMesh& hm, const std::vector<int>& ancho
     cudaFree(GA);
     cudaFree(GP);
   }
-  plane_setup(c);
   // ---- near zone
   {
     std::vector<int> rowptr, col;
