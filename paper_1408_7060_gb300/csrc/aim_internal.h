@@ -294,7 +294,7 @@ struct aim_ctx {
 
   // ---- work buffers (sized for batch_max) ----
   void* d_A = nullptr;         // [B][4][NZ][N][L]  after the x pass; kx-major contexts: [B][4][L][NZ][N]
-  void* d_Bf = nullptr;        // [B][4][NZ][L][L]  after the y pass (the slab); unused when kx-major
+  void* d_Bf = nullptr;        // [B][4][NZ][L][L]  after the y pass (the slab); none when kx-major
   void* d_P = nullptr;         // [B][4][NZ][N][N]  potentials on the grid
   void* d_ring = nullptr;      // [N_g][B][4][Z][L][L] history slabs: z-spectra (Z = LZ, power-of-two
                                // LZ, and plane-kernel contexts, in its order) or x/y-transformed grids (Z = NZ)

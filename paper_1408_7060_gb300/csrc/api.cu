@@ -83,7 +83,7 @@ void setup_work(aim_ctx* c, const aim_opts* opts) {
   alloc_ring(c);
   plane_spectra(c);
   c->d_A = aim_alloc(c, grid_a_elems(c, B) * es);
-  c->d_Bf = aim_alloc(c, grid_bf_elems(c, B) * es);
+  c->d_Bf = op_plane(c) ? nullptr : aim_alloc(c, grid_bf_elems(c, B) * es);  // the separate passes' slab
   c->d_P = aim_alloc(c, grid_p_elems(c, B) * es);
   c->d_xs = aim_alloc(c, (size_t)B * ns * es);
   c->d_xd = (double2*)aim_alloc(c, (size_t)B * ns * sizeof(double2));
@@ -108,7 +108,7 @@ void setup_work(aim_ctx* c, const aim_opts* opts) {
     c->ref_nb = (int)std::max<size_t>(1, std::min<size_t>((size_t)B, (size_t(8) << 30) / per));
     const int rb = c->ref_nb;
     c->d_A64 = aim_alloc(c, grid_a_elems(c, rb) * sizeof(double2));
-    c->d_Bf64 = aim_alloc(c, grid_bf_elems(c, rb) * sizeof(double2));
+    c->d_Bf64 = c->plane64 ? nullptr : aim_alloc(c, grid_bf_elems(c, rb) * sizeof(double2));
     c->d_P64 = aim_alloc(c, grid_p_elems(c, rb) * sizeof(double2));
     c->d_xs64 = aim_alloc(c, (size_t)rb * ns * sizeof(double2));
     c->d_rn = (double*)aim_alloc(c, 2 * (size_t)B * sizeof(double));

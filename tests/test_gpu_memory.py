@@ -7,6 +7,8 @@ allocation while a context of a factor-3 z length (96^3, a ring of several GB) i
 * Where the plane path's ring does not fit but that of the separate passes does, the set-up
   goes through with the separate passes: buffers, launch plan and warm-up of that path, none
   of the other's memory kept, products and marches within the complex64 rounding of the grid.
+
+A context of the plane kernel holds no slab of the separate passes, in either precision.
 """
 import contextlib
 
@@ -87,3 +89,33 @@ def test_path_follows_from_the_sizes(tmp_path, monkeypatch):
             assert separate and c.info["device_bytes"] < full - ring // 3
             assert c.info["plan_source"] == abi.AIM_PLAN_MEASURED
     assert all(rel(a, b) < 1e-5 for a, b in zip(got[:2], want[:2])) and rel(got[2], want[2]) < 1e-4
+
+
+def plane_table(n, lz):
+    """Bytes of the FP64 spectra of one delay in the plane kernel's order, at most."""
+    return 2 * (n + 1) * 2 * n * lz * 16
+
+
+def test_no_slab_beside_the_plane_kernel():
+    from paper_1408_7060_gb300 import AimContext
+
+    V, F = icosphere(4, 1.0)
+    h, origin = place_grid(V, 64)
+
+    def held(**kw):
+        with AimContext(V=V, F=F, grid_n=64, origin=origin, h=h, near_radius=3 * h, dt=0.25 / (BAND * F_C), f_c=F_C,
+                        **kw) as c:
+            assert c.info["z_len"] == 128
+            c.matvec(0, np.ones((1, c.ns), complex))
+            assert c.get_profile()[0]["yfft_fwd"][0] == 0
+            nz = c.info["box_hi"][2] - c.info["box_lo"][2] + 1
+            ring = c.n_delays * 4 * 128 ** 3                   # elements per wave: ring, A, P
+            return c.info["device_bytes"], ring, 4 * nz * 64 * (128 + 64), 4 * nz * 128 ** 2
+
+    # what 40 more waves take beyond their ring, A and P is less than their slab
+    (b1, ring, grid, slab), b41 = held(precision="c64"), held(precision="c64", batch_max=41)[0]
+    vectors = 40 * V.shape[0] * 3 * 16 * (51 + 60)             # Krylov basis, histories, work vectors
+    assert b41 - b1 < 40 * 8 * (ring + grid) + vectors + 40 * 8 * slab // 2
+    # and the refinement's buffers likewise (FP64, A and P of one wave)
+    more = held(precision="c64", refine=2)[0] - b1
+    assert more < 16 * grid + 16 * slab // 2 + plane_table(64, 128)
