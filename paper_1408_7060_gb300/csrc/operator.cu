@@ -124,9 +124,15 @@ void op_block_square(aim_ctx* c, int nb, const BlockSquare& sq) {
 
 // ---------------------------------------------------------------- launch plans
 // The plan cache: one JSON object per line,
-//   {"key": "<gpu name>|L=<L>|LZ=<LZ>|prec=<c64|c128>|nb=<batch>", "zw": .., "cw": .., "rp": .., "ypb": ..}
-// in the file named by AIM_GB300_PLAN_CACHE, else $HOME/.cache/aim_gb300_plans.jsonl.
+//   {"key": "<gpu name>|L=<L>|LZ=<LZ>|prec=<c64|c128>|nb=<batch>|path=<plane|separate>|ny=<box rows>|
+//    nz=<box planes>|v=<revision>", "zw": .., "cw": .., "rp": .., "ypb": ..}
+// in the file named by AIM_GB300_PLAN_CACHE, else $HOME/.cache/aim_gb300_plans.jsonl.  The path
+// decides which kernels rp and ypb are rows of, the box how many blocks they make.
 namespace {
+// raised with the kernels that the numbers of a plan belong to: plans of another revision are
+// measured anew
+constexpr int kPlanRevision = 2;
+
 std::string plan_cache_path() {
   if (const char* e = std::getenv("AIM_GB300_PLAN_CACHE")) return e;
   if (const char* h = std::getenv("HOME")) return std::string(h) + "/.cache/aim_gb300_plans.jsonl";
@@ -142,7 +148,9 @@ std::string plan_key(const aim_ctx* c) {
   for (char& ch : name)
     if (ch == '"' || ch == '|') ch = '_';
   return name + "|L=" + std::to_string(c->L) + "|LZ=" + std::to_string(c->LZ) + "|prec=" + (c->precision == AIM_C64 ? "c64" : "c128") +
-         "|nb=" + std::to_string(c->batch_max);
+         "|nb=" + std::to_string(c->batch_max) + "|path=" + (op_plane(c) ? "plane" : "separate") +
+         "|ny=" + std::to_string(c->box_hi[1] - c->box_lo[1] + 1) + "|nz=" + std::to_string(c->NZ) +
+         "|v=" + std::to_string(kPlanRevision);
 }
 
 int json_int(const std::string& line, const char* field) {

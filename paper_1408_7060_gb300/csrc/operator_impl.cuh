@@ -1693,16 +1693,20 @@ struct GridOps {
       }
       field = arg;
     };
-    if (kxm(c)) {  // the plane kernel has one shape; its fields keep the defaults
+    // k_plane, k_zwarp and k_ypipe have one shape: the fields keep the defaults there
+    bool zwarp = false;
+    with_zlen(c->LZ, [&](auto lz) { zwarp = zwarp_len<L, decltype(lz)::value, C>(); });
+    if (kxm(c) || zwarp)
       p.zw = def_zw(c);
-      p.cw = def_cw();
-    } else {
+    else
       pick(p.zw, zwidths(c), [&] { zconv(c, nb, 0, nullptr); });
+    if (kxm(c) || ypipe_len<L, C>())
+      p.cw = def_cw();
+    else
       pick(p.cw, ywidths(), [&] {
         y_fwd(c, nb, reinterpret_cast<C*>(c->d_Bf));
         y_inv(c, nb);
       });
-    }
     pick(p.rp, rps(c), [&] { x_inv(c, nb); });
     pick(p.ypb, ypbs(c), [&] { anterp_x(c, nb, nullptr); });
     cudaEventDestroy(e0);
