@@ -135,7 +135,7 @@ void setup_work(aim_ctx* c, const aim_opts* opts) {
   // attributes of each instantiation and surfaces launch errors at setup
   AIM_CUDA(cudaMemsetAsync(c->d_x, 0, vec, c->stream));
   op_apply(c, 0, 1, c->d_x, nullptr, nullptr, 1.0, nullptr, c->d_y);
-  if (c->refine > 0) op_apply_f64(c, 0, 1, c->d_x, nullptr, 1.0, c->d_y);
+  if (c->refine > 0) op_apply_f64(c, 1, c->d_x, nullptr, 1.0, c->d_y);
   op_forward_slab(c, 1, c->d_x, c->d_ring);
   {
     SlabList sl{};
@@ -1061,7 +1061,7 @@ static int refine_solution(aim_ctx* c, int nb, double tol, std::vector<int>& its
   res.assign(nb, 0.0);
   n_corr = 0;
   for (int k = 0;; ++k) {
-    op_apply_f64(c, 0, nb, c->d_x, c->d_b, -1.0, c->d_r);  // r = b - Z_0 x, FP64 grid stages
+    op_apply_f64(c, nb, c->d_x, c->d_b, -1.0, c->d_r);  // r = b - Z_0 x, FP64 grid stages
     gmres_norms(c, nb, c->d_r, c->d_rn);
     gmres_norms(c, nb, c->d_b, c->d_rn + nb);
     AIM_CUDA(cudaMemcpyAsync(c->h_rn, c->d_rn, 2 * nb * sizeof(double), cudaMemcpyDeviceToHost, st));

@@ -41,9 +41,9 @@ void op_apply(aim_ctx* c, int m, int nb, const double2* v, const double2* dinv, 
     body_apply<double2>(c, m, nb, v, dinv, base, sign, active, y, vin, yout);
 }
 
-void op_apply_f64(aim_ctx* c, int m, int nb, const double2* v, const double2* base, double sign, double2* y) {
+void op_apply_f64(aim_ctx* c, int nb, const double2* v, const double2* base, double sign, double2* y) {
   if (c->precision == AIM_C128) {
-    op_apply(c, m, nb, v, nullptr, base, sign, nullptr, y);
+    op_apply(c, 0, nb, v, nullptr, base, sign, nullptr, y);
     return;
   }
   if (!c->d_A64 || c->ref_nb < 1) throw AimError{AIM_ERR_ARG, "FP64 operator: refinement buffers not set up"};
@@ -67,7 +67,7 @@ void op_apply_f64(aim_ctx* c, int m, int nb, const double2* v, const double2* ba
   const size_t ns = c->ns;
   for (int b0 = 0; b0 < nb; b0 += c->ref_nb) {
     const int n = std::min(c->ref_nb, nb - b0);
-    body_apply<double2>(c, m, n, v + b0 * ns, nullptr, base ? base + b0 * ns : nullptr, sign, nullptr, y + b0 * ns,
+    body_apply<double2>(c, 0, n, v + b0 * ns, nullptr, base ? base + b0 * ns : nullptr, sign, nullptr, y + b0 * ns,
                         VecSel(), VecSel());
   }
 }
