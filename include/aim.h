@@ -127,7 +127,8 @@ typedef struct {
                             passes, rows per block of the x passes): 0 built-in defaults;
                             1 time every candidate on this context's buffers at setup and
                             keep the fastest, reusing a plan cached for the same GPU model,
-                            padded lengths, precision and batch; 2 time and refresh the cache.
+                            padded lengths, precision, batch, box and path of the grid
+                            passes; 2 time and refresh the cache.
                             Cache: the file named by AIM_GB300_PLAN_CACHE, else
                             $HOME/.cache/aim_gb300_plans.jsonl (one JSON object per line).
                             The results do not depend on the plan (same arithmetic per line). */
