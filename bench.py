@@ -62,20 +62,14 @@ def load_peaks():
 
 
 def kernel_digest(kind):
-    """Digest of a kernel's source text and the FFT core it uses: measured DRAM traffic
-    is only reported while the kernel is unchanged since the capture."""
-    src = open(os.path.join(CSRC, "operator_impl.cuh")).read()
-    names = {"zconv": r"k_zconv(_p2)?", "interp_near": r"k_interp_near", "anterp_xfft": r"k_anterp",
-             "zrhs": r"k_zrhs(_spec)?(_tma)?"}
-    if kind not in names:
+    """Digest of the sources a grid kernel is made of (its body, the structures and the FFT core
+    it is built from): measured DRAM traffic is only reported while they are unchanged since the
+    capture."""
+    if kind not in ("zconv", "interp_near", "anterp_xfft", "zrhs", "yfft_fwd", "yfft_inv", "xfft_inv"):
         return None
-    blocks = [m.group(0) for m in re.finditer(r"__global__ void __launch_bounds__\([^)]*\) " + names[kind]
-                                              + r"\(.*?\n}\n", src, re.S)]
-    if not blocks:
-        return None
-    h = hashlib.sha1("".join(blocks).encode())
-    for f in ("fft.cuh", "fft_kernels.cuh"):
-        h.update(open(os.path.join(CSRC, f)).read().encode())
+    h = hashlib.sha1(kind.encode())
+    for f in ("operator_impl.cuh", "plane.cuh", "plane_launch.cuh", "fft.cuh", "fft_kernels.cuh"):
+        h.update(open(os.path.join(CSRC, f), "rb").read())
     return h.hexdigest()[:16]
 
 
@@ -84,26 +78,78 @@ def kernel_digest(kind):
 TRAFFIC = {}
 
 
-def kernel_bytes(kind, N, ns, nnz, ng, nb, box=None, esz=8, lz=None):
+# shapes of the plane kernel (PlaneCfg in plane.cuh): radix split of a length, shared memory of
+# a plane, columns whose kernel spectra are tabulated
+PLANE_R1 = {16: 4, 32: 8, 64: 8, 128: 16, 144: 12, 192: 16, 256: 16}
+
+
+def plane_shape(L, lz, esz):
+    """(shared-memory bytes, tabulated columns ky) of a plane of an L-point y and an lz-point z
+    transform with esz-byte elements, or None where there is no such plane."""
+    if L not in PLANE_R1 or lz not in PLANE_R1 or lz > L:
+        return None
+    y1, z1 = PLANE_R1[L], PLANE_R1[lz]
+    y2, z2 = L // y1, lz // z1
+    warps = 4 if L <= 32 else 16 if L == lz == 192 else 8
+    cw = 8 if z2 == 4 else 2 if z2 == 16 or lz == 192 else 4
+    up = lambda p, r: next(q for q in range(p, p + 16) if q % 16 == r)
+    py, pz = up(y1 * (y2 + 1), 2 if cw == 2 else 4), up(z1 * (z2 + 1), 4)
+    tables = y1 * (y2 + 1) + (z1 * (z2 + 1) if L != lz else 0)
+    smem = (tables + lz // 2 * py + warps * cw * pz) * esz
+    return smem, (y1 // 2 + 1) * y2 if y2 % cw == 0 else L
+
+
+def plane_fits(L, lz, esz):
+    """Whether such a plane fits the shared memory a block can opt in to."""
+    shape = plane_shape(L, lz, esz)
+    return shape is not None and shape[0] <= 227 * 1024
+
+
+PLANE_RING_MAX = 64 << 30   # z-spectra of a factor-3 z length beyond this: separate passes
+
+
+def runs_plane(L, lz, esz, n_delays, nb):
+    """The library's rule for contexts of nb right-hand sides."""
+    pow2 = (lz & (lz - 1)) == 0
+    return plane_fits(L, lz, esz) and (pow2 or n_delays * nb * 4 * L * L * lz * esz <= PLANE_RING_MAX)
+
+
+def kernel_bytes(kind, N, ns, nnz, ng, nb, box=None, esz=8, lz=None, plane=False, n_active=None):
     """Algorithmic HBM bytes of one launch of each kernel (each byte counted once), for the
     grid lines each pass touches: with the active box (nx, ny, nz nodes per axis) the
     anterpolation writes the box rows of A, the forward y pass reads them and writes the
     box-z rows of the slab, the z pass reads and writes those rows, the inverse y pass
-    writes the box rows of A and the inverse x pass the box of P.  lz: the length of the
-    z transform (2N without a shorter one)."""
+    writes the box rows of A and the inverse x pass the box of P.  With plane (the plane
+    kernel's kx-major grid) A holds whole kx planes, rows of N nodes, the z pass reads and writes
+    it with the tabulated spectrum instead of octants, and the history holds z-spectra.
+    lz: the length of the z transform (2N without a shorter one); n_active: nodes some stencil
+    touches (every box node if not given)."""
     L = 2 * N
     lz = lz or L
     bx, by, bz = box if box else (N, N, N)
     slab = 4 * bz * L * L * esz * nb          # [nb][4][z in box][L][L]
-    spec = 4 * lz * L * L * esz * nb          # [nb][4][lz][L][L]: z-spectrum of a slab (power-of-two lz)
+    spec = 4 * lz * L * L * esz * nb          # [nb][4][lz][L][L]: z-spectrum of a slab
     pow2 = (lz & (lz - 1)) == 0
     A = 4 * bz * by * L * esz * nb            # [nb][4][z, y in box][L]
+    Ak = 4 * bz * N * L * esz * nb            # [nb][4][L][z in box][N]
     P = 4 * bz * by * bx * esz * nb           # [nb][4][box]
     oct_ = (N + 1) ** 2 * (lz // 2 + 1) * esz  # one kernel spectrum octant
     lam = ns * 256 * (esz // 2)               # interpolation rows
-    csrT = 64 * ns * (4 + 2 * esz) + (bz * by * N + 1) * 4
+    active = n_active if n_active is not None else bx * by * bz
+    csrT = 64 * ns * (4 + 2 * esz) + 8 * active + 4 * bz * by   # entries, nodes, box rows
     near = nnz * (4 + 16) + (ns + 1) * 4
     vec = ns * 16 * nb
+    if plane:
+        table = 2 * (N + 1) * plane_shape(L, lz, esz)[1] * lz * esz   # both kinds, in the kernel's order
+        return {
+            "prep": vec + ns * 16 + ns * (esz + 16) * nb,
+            "anterp_xfft": csrT + ns * esz * nb + Ak,
+            "zconv": 2 * Ak + table,
+            "zrhs": (ng + 2) * spec + ng * table + Ak,   # the sum is written and read by the inverse
+            "zfwd": Ak + spec,
+            "xfft_inv": A + P,
+            "interp_near": P + lam + ns * 12 + near + 2 * vec,
+        }.get(kind)
     return {
         "prep": vec + ns * 16 + ns * (esz + 16) * nb,
         "anterp_xfft": csrT + ns * esz * nb + A,
@@ -117,25 +163,35 @@ def kernel_bytes(kind, N, ns, nnz, ng, nb, box=None, esz=8, lz=None):
     }.get(kind)
 
 
-# FP32 arithmetic peak of the z pass's roofline (it is bound by FP32 instruction issue,
-# not by DRAM): 152 SMs x 128 FP32 lanes x 2 flops per FMA x 2.07 GHz (maximum SM clock)
+# FP32 arithmetic peak of the z pass's roofline (it is bound by FP32 instruction issue, or on
+# the plane kernel by shared memory, not by DRAM): 152 SMs x 128 FP32 lanes x 2 flops per FMA x
+# 2.07 GHz (maximum SM clock)
 FP32_PEAK_TFLOPS = 152 * 128 * 2 * 2.07e9 / 1e12
-ALU_KERNELS = ("zconv", "zrhs")
 
 
-def kernel_flops(kind, N, nb, ng, lz=None):
+def alu_kernels(lz, plane):
+    """z-pass kernels reported against the FP32 peak: the delay sum only where it transforms
+    every slab (separate passes of a factor-3 z length); elsewhere it streams spectra."""
+    return ("zconv",) if plane or (lz & (lz - 1)) == 0 else ("zconv", "zrhs")
+
+
+def kernel_flops(kind, N, nb, ng, lz=None, plane=False, bz=None):
     """Algorithmic FP32 flops of one launch of the z-pass kernels: per z column the
     conventional 5 n log2 n of a length-n complex FFT (n = lz, the z transform length)
-    forward and inverse, and 6 n for the product with the kernel spectrum (the delay sum:
-    N_g forward transforms and products, one inverse); 4 nb L^2 columns per launch."""
+    forward and inverse, and 6 n for the product with the kernel spectrum (the delay sum: 8 n
+    per delay and one inverse transform, with N_g forward transforms where the history is kept
+    x/y-transformed); 4 nb L^2 columns per launch.  The plane kernel adds the y transforms of
+    its bz rows of every kx."""
     L = 2 * N
     n = lz or L
     fft = 5 * n * math.log2(n)
     cols = 4 * nb * L * L
+    rows = 4 * nb * L * (bz or n // 2) * 5 * L * math.log2(L) if plane else 0
     if kind == "zconv":
-        return cols * (2 * fft + 6 * n)
+        return cols * (2 * fft + 6 * n) + 2 * rows
     if kind == "zrhs":
-        return cols * ((ng + 1) * fft + 8 * ng * n)
+        forward = 0 if plane or (n & (n - 1)) == 0 else ng
+        return cols * ((forward + 1) * fft + 8 * ng * n) + rows
     return None
 
 
@@ -233,25 +289,37 @@ def box_depth(w):
     return nz, lz
 
 
-def chunk_size(w, ng_est, refine, total_bytes, restart=50):
-    """Right-hand sides per context that fit in device memory: per-RHS work buffers and
-    history ring over the box's z-planes (x/y-transformed slabs for z lengths with a
-    factor 3, z-spectra for powers of two) against the tables (kernel octants in both
-    precisions, anterpolation, near zone and preconditioner estimated at 80 entries per
-    row, FP64 refinement buffers of up to 8 GiB) and a 6 GB margin."""
+def context_bytes(w, ng_est, refine, nb, restart=50):
+    """Estimated device memory of a context of nb right-hand sides: work buffers and history ring
+    (z-spectra for power-of-two z lengths and on the plane kernel, else x/y-transformed slabs of
+    the box's z-planes; the padded slab and its FP64 counterpart for the separate passes only),
+    tables (kernel octants in both precisions, the plane kernel's spectra and batch buffers,
+    anterpolation, near zone and preconditioner estimated at 80 entries per row) and FP64
+    refinement buffers of up to 8 GiB."""
     N, L = w.grid_n, 2 * w.grid_n
     nz, lz = box_depth(w)
-    V, F = w.mesh
-    ns = len(F) * 3 // 2
+    ns = len(w.mesh[1]) * 3 // 2
     es = 8
-    Z = lz if (lz & (lz - 1)) == 0 else nz
-    grid = 4 * nz * (N * L + L * L + N * N)
+    plane = runs_plane(L, lz, es, ng_est, nb)
+    Z = lz if plane or (lz & (lz - 1)) == 0 else nz
+    grid = 4 * nz * (N * L + N * N + (0 if plane else L * L))
     per = es * grid + ng_est * es * 4 * Z * L * L + ns * 16 * (restart + 2 * ng_est + 10)
     base = (ng_est + 1) * 2 * (N + 1) ** 2 * (lz // 2 + 1) * 24 + ns * 256 * 12 + 64 * ns * 52 + 4 * N ** 3
     base += ns * 80 * (16 * (ng_est + 1) + 8 + 24)
+    if plane:
+        base += (ng_est + 1) * 2 * (N + 1) * plane_shape(L, lz, es)[1] * lz * es + 2 * (64 << 20)
     if refine:
-        base += min(16 * grid * 16, 8 << 30)
-    return max(1, int((total_bytes - base - 6e9) // per))
+        grid64 = 4 * nz * (N * L + N * N + (0 if plane_fits(L, lz, 16) else L * L))
+        base += min(16 * grid64 * 16, 8 << 30)
+    return base + nb * per
+
+
+def chunk_size(w, ng_est, refine, total_bytes, restart=50):
+    """Right-hand sides per context that fit in device memory with a 6 GB margin (at least one)."""
+    nb = 1
+    while nb < 4096 and context_bytes(w, ng_est, refine, nb + 1, restart) + 6e9 <= total_bytes:
+        nb += 1
+    return nb
 
 
 # --------------------------------------------------------------------------- GPU arm
@@ -383,7 +451,10 @@ def run_aim(args):
     hbm, src = load_peaks()
     box = tuple(hi - lo + 1 for lo, hi in zip(info["box_lo"], info["box_hi"]))
     lz = info["z_len"]
-    kb = lambda kind: kernel_bytes(kind, w.grid_n, ns, info["near_nnz"], info["n_delays"], prof_nb, box, lz=lz)
+    plane = prof["yfft_fwd"][0] == 0      # no separate y pass: the plane kernel ran
+    kb = lambda kind: kernel_bytes(kind, w.grid_n, ns, info["near_nnz"], info["n_delays"], prof_nb, box, lz=lz,
+                                   plane=plane, n_active=info["n_active"])
+    kf = lambda kind: kernel_flops(kind, w.grid_n, prof_nb, info["n_delays"], lz, plane, box[2])
     tot_ms = sum(v[1] for v in prof.values()) or 1e-12
     kernels = {}
     for kind, (n_l, ms_l) in prof.items():
@@ -393,9 +464,9 @@ def run_aim(args):
         kernels[kind] = {"launches": n_l, "ms": round(ms_l, 4), "share": round(ms_l / tot_ms, 4),
                          "gbs": round(b / (ms_l / n_l * 1e-3) / 1e9, 1) if b and ms_l > 0 else None,
                          "frac": round(b / (ms_l / n_l * 1e-3) / 1e9 / hbm, 4) if b and ms_l > 0 else None}
-    for kind in ALU_KERNELS:
+    for kind in alu_kernels(lz, plane):
         if kind in kernels and kernels[kind]["ms"] > 0:
-            fl = kernel_flops(kind, w.grid_n, prof_nb, info["n_delays"], lz)
+            fl = kf(kind)
             tf = fl / (kernels[kind]["ms"] / kernels[kind]["launches"] * 1e-3) / 1e12
             kernels[kind]["tflops"] = round(tf, 2)
             kernels[kind]["alu_frac"] = round(tf / FP32_PEAK_TFLOPS, 4)
@@ -409,6 +480,7 @@ def run_aim(args):
         "dtype": "c64 grid / f64 solve + f64 refinement" if w.refine else "c64 grid / f64 solve",
         "data": "synthetic",
         "config": {"workload": w.name, "ns": ns, "grid": f"{w.grid_n}^3",
+                   "grid_passes": "plane kernel" if plane else "separate y and z passes",
                    "fft": f"{2 * w.grid_n} x {2 * w.grid_n} x {lz} (z: {box[2]} box planes)",
                    "n_delays": info["n_delays"], "near_nnz": info["near_nnz"], "plane_waves": nw,
                    "waves_per_context": chunk, "chunks": len(chunks), "tol": w.tol, "chi": round(w.chi, 3),
@@ -427,7 +499,7 @@ def run_aim(args):
         "refine_corrections_per_step": round(corr / (K * len(chunks)), 2),
         "split_ms_per_step": {"rhs": round(float(np.mean([s[0] for s in split])) * len(chunks), 3),
                               "solve": round(float(np.mean([s[1] for s in split])) * len(chunks), 3)},
-        "roofline": roofline_entry(dom, kb(dom), kernel_flops(dom, w.grid_n, prof_nb, info["n_delays"], lz),
+        "roofline": roofline_entry(dom, kb(dom), kf(dom) if dom in alu_kernels(lz, plane) else None,
                                    per_launch_ms, hbm, src, w.name, prof_nb),
         "kernels": kernels,
         "e2e": {"value": e2e, "unit": UNIT, "h2d_bytes_per_step": nw * 6 * 8, "d2h_bytes_per_step": nw * ns * 16},
@@ -454,12 +526,12 @@ def run_aim(args):
 
 
 def roofline_entry(kind, nbytes, nflops, per_launch_ms, hbm, src, workload, nb):
-    """The dominant kernel against its bound: the z-pass kernels against the FP32 peak
-    (instruction-bound, DRAM a few per cent busy in the ncu profile), the other passes
-    against the measured HBM copy bandwidth."""
+    """The dominant kernel against its bound: those with nflops (alu_kernels) against the FP32
+    peak (bound by instructions or shared memory, DRAM a third busy at most in the ncu
+    profile), the other passes against the measured HBM copy bandwidth."""
     t = per_launch_ms * 1e-3
     traffic = TRAFFIC.get((kind, workload, kernel_digest(kind)))
-    if kind in ALU_KERNELS and nflops:
+    if nflops:
         achieved = nflops / t / 1e12
         return {"bound": "alu", "kernel": kind, "achieved": round(achieved, 2), "peak": round(FP32_PEAK_TFLOPS, 1),
                 "peak_source": "derived: 152 SMs x 128 FP32 lanes x 2 flops x 2.07 GHz", "unit": "TFLOP/s",
