@@ -1797,8 +1797,12 @@ struct GridOps {
   // blocked right-hand side: pending z-spectra -> slab of potentials in Bf (cleared)
   static void zinv_pending(aim_ctx* c, int nb, C* S) {
     if (kxm(c)) {
+      // (cleared by a memset: with zeros stored between its loads the plane kernel took 204 us for
+      // one vector on the 64^3 grid, the inverse and the memset take 39)
       KScope ks(c, AIM_K_ZINV_PENDING);
-      return plane_launch<C>(c, nb, PLANE_PENDING, 0, nullptr, S, 1, 0);
+      plane_launch<C>(c, nb, PLANE_INV, 0, nullptr, S, 1, 0);
+      AIM_CUDA(cudaMemsetAsync(S, 0, op_slab_bytes(c, nb), c->stream));
+      return;
     }
     with_zlen(c->LZ, [&](auto lz) {
       constexpr int LZ = decltype(lz)::value;

@@ -130,10 +130,9 @@ __device__ __forceinline__ void st2(double2* p, double2 a, double2 b) {
 }
 
 // ---------------------------------------------------------------- the plane kernel
-enum { PLANE_CONV = 0,    // A <- inverse(G_m . forward(A))
-       PLANE_FWD = 1,     // S <- forward(A)
-       PLANE_INV = 2,     // A <- inverse(S)
-       PLANE_PENDING = 3  // A <- inverse(S), S <- 0
+enum { PLANE_CONV = 0,  // A <- inverse(G_m . forward(A))
+       PLANE_FWD = 1,   // S <- forward(A)
+       PLANE_INV = 2    // A <- inverse(S)
 };
 
 template <int L, int LZ, class C>
@@ -293,7 +292,7 @@ struct PlaneFFT : PlaneCfg<L, LZ, C> {
 template <class C>
 struct PlaneArgs {
   C* A;              // [nb * 4][L][nz][N]
-  C* S;              // FWD: spectra out; INV, PENDING: spectra in
+  C* S;              // FWD: spectra out; INV: spectra in
   const C* G;        // CONV: the tabulated spectrum of the delay
   int sbc;           // (right-hand side, component) pairs per spectrum; further ones go on
   size_t sstride;    // sstride elements after it (several delays in one launch)
@@ -373,7 +372,7 @@ __global__ void __launch_bounds__(32 * PlaneCfg<L, LZ, C>::NW, (PlaneCfg<L, LZ, 
       }
       __syncwarp();
     } else {
-      C* in = a.S + soff + (size_t)g * (F::CW * LZ);
+      const C* in = a.S + soff + (size_t)g * (F::CW * LZ);
 #pragma unroll
       for (int q = 0; q < F::QB; ++q) {
         const int u = lane + 32 * q, k1 = u / F::CW;
@@ -381,9 +380,7 @@ __global__ void __launch_bounds__(32 * PlaneCfg<L, LZ, C>::NW, (PlaneCfg<L, LZ, 
           C v[F::Z2];
 #pragma unroll
           for (int h = 0; h < F::Z2 / 2; ++h) {
-            C* e = in + h * (2 * F::UB) + 2 * u;
-            ld2_stream(e, v[2 * h], v[2 * h + 1]);
-            if (MODE == PLANE_PENDING) st2(e, C{}, C{});
+            ld2_stream(in + h * (2 * F::UB) + 2 * u, v[2 * h], v[2 * h + 1]);
           }
           F::b_inverse(scr + (u % F::CW) * F::PZ + k1 * (F::Z2 + 1), twz, k1, v);
         }

@@ -43,8 +43,7 @@ void plane_launch(aim_ctx* c, int nb, int mode, int m, const int* active, C* S, 
         switch (mode) {
           case PLANE_CONV: go(k_plane<L, LZ, C, PLANE_CONV>); break;
           case PLANE_FWD: go(k_plane<L, LZ, C, PLANE_FWD>); break;
-          case PLANE_INV: go(k_plane<L, LZ, C, PLANE_INV>); break;
-          default: go(k_plane<L, LZ, C, PLANE_PENDING>);
+          default: go(k_plane<L, LZ, C, PLANE_INV>);
         }
       } else {
         throw AimError{AIM_ERR_ARG, "plane kernel: the plane does not fit shared memory"};
