@@ -989,15 +989,17 @@ __global__ void __launch_bounds__(256) k_block_square(BlockSquare sq, const C* _
 }
 
 // The same on spectra in the plane kernel's order, [bc][kx][group][pair][unit][2], with the
-// taps from its tabulated kernel spectra.
+// taps from its tabulated kernel spectra; grid (blocks, nb * 4), so that an element's place in
+// the table takes 32-bit divisions only.
 template <int B, class C>
 __global__ void __launch_bounds__(256) k_block_square_plane(BlockSquare sq, const C* __restrict__ G, PlaneOrder o,
-                                                            int ng, long long n) {
-  const long long per_bc = (long long)o.L * o.L * o.LZ;
-  const size_t kind_off = (size_t)(o.L / 2 + 1) * plane_g_elems(o), gm = plane_spec_elems(o);
+                                                            int ng) {
+  const int per_bc = o.L * o.L * o.LZ;
+  const size_t gm = plane_spec_elems(o);
   const int m0 = sq.toff - B + 1;  // tap[t] = G^_{m0 + t}
-  for (long long q = blockIdx.x * 256LL + threadIdx.x; q < n; q += (long long)gridDim.x * 256) {
-    const size_t go = ((q / per_bc) & 3) == 3 ? kind_off + plane_g_index(o, q % per_bc) : plane_g_index(o, q % per_bc);
+  if ((blockIdx.y & 3) == 3) G += (size_t)(o.L / 2 + 1) * plane_g_elems(o);
+  for (int i = blockIdx.x * 256 + threadIdx.x; i < per_bc; i += gridDim.x * 256) {
+    const size_t go = plane_g_index(o, i), q = (size_t)blockIdx.y * per_bc + i;
     C tap[2 * B - 1];
 #pragma unroll
     for (int t = 0; t < 2 * B - 1; ++t) {
@@ -1823,14 +1825,15 @@ struct GridOps {
   static void block_square(aim_ctx* c, int nb, const BlockSquare& sq) {
     const long long n = (long long)nb * 4 * c->LZ * L * L;
     const int grid = (int)std::min<long long>((n + 255) / 256, 152LL * 8);
+    const int per = (grid + nb * 4 - 1) / (nb * 4);  // blocks per right-hand side and component
     KScope ks(c, AIM_K_BLOCK_SQUARE);
     auto go = [&](auto bt) {
       constexpr int B = decltype(bt)::value;
       if (kxm(c))
         with_zlen(c->LZ, [&](auto lz) {
           if constexpr (plane_fits<L, decltype(lz)::value, C>())
-            k_block_square_plane<B, C><<<grid, 256, 0, c->stream>>>(
-                sq, plane_spec(c), plane_order<L, decltype(lz)::value, C>(), c->n_delays, n);
+            k_block_square_plane<B, C><<<dim3(per, nb * 4), 256, 0, c->stream>>>(
+                sq, plane_spec(c), plane_order<L, decltype(lz)::value, C>(), c->n_delays);
         });
       else
         k_block_square<B, C><<<grid, 256, 0, c->stream>>>(sq, kspec(c), zgeom(c), c->LZ, c->n_delays, n);

@@ -398,9 +398,10 @@ __global__ void __launch_bounds__(32 * PlaneCfg<L, LZ, C>::NW, (PlaneCfg<L, LZ, 
 
 // Element i of the spectra of one (right-hand side, component), [kx][group]..., in the
 // tabulated kernel spectrum of a kind.
-__device__ __forceinline__ size_t plane_g_index(const PlaneOrder& o, long long i) {
+// (at most 256^3 elements)
+__device__ __forceinline__ size_t plane_g_index(const PlaneOrder& o, int i) {
   const int N = o.L / 2, per_kx = o.L * o.LZ, gsz = o.cw * o.LZ;
-  const int kx = (int)(i / per_kx), q = (int)(i % per_kx);
+  const int kx = i / per_kx, q = i % per_kx;
   int g = q / gsz, r = q % gsz;
   const size_t base = (size_t)fold(kx, N) * plane_g_elems(o);
   if (o.h && g / o.h > o.y1 / 2) {  // the mirror group, columns reversed
@@ -418,8 +419,7 @@ __device__ __forceinline__ size_t plane_g_index(const PlaneOrder& o, long long i
 template <class C>
 __global__ void __launch_bounds__(256) k_spec_sum(const __grid_constant__ SlabList sl, const C* __restrict__ G,
                                                   PlaneOrder o, C* out) {
-  const long long per = (long long)o.L * o.L * o.LZ;
-  const long long i = 2 * (blockIdx.x * 256LL + threadIdx.x);
+  const int per = o.L * o.L * o.LZ, i = 2 * (blockIdx.x * 256 + threadIdx.x);
   if (i >= per) return;
   const int bc = blockIdx.y;
   const C* gp = G + ((bc & 3) == 3 ? (size_t)(o.L / 2 + 1) * plane_g_elems(o) : 0);

@@ -126,3 +126,19 @@ def test_batch_is_its_vectors_on_the_largest_grid():
         for b in (0, 2):
             one, so, _ = abi.aim_march_source(c.handle, np.ascontiguousarray(src[:, b:b + 1]), 1e-2)
             assert rel(cur[:, b], one[:, 0]) < 1e-10 and np.array_equal(st["iters"][:, b], so["iters"][:, 0])
+
+
+@pytest.mark.parametrize("precision,tol,bound", [("c128", 1e-10, 1e-9), ("c64", 1e-6, 1e-5)])
+def test_blocked_march_of_several_waves_on_the_plane_kernel(precision, tol, bound):
+    """Blocked and direct marches of three waves of a context for four (bounds of test_gpu_blocked)."""
+    from paper_1408_7060_gb300 import AimContext
+    from paper_1408_7060_gb300.inputs import make_workload
+
+    w = make_workload("sphere480", band_frac=0.2, n_t=24)
+    k, p = random_plane_waves(3, 5)
+    got = []
+    for blocked in (0, 1):
+        with AimContext.from_workload(w, precision=precision, batch_max=4, rhs_blocked=blocked) as c:
+            got.append(c.march(k, p, w.sigma, w.t_d, w.n_t, tol)[0])
+            assert launches(c, "yfft_fwd") == 0 and (launches(c, "block_square") > 0) == bool(blocked)
+    assert all(rel(got[1][:, b], got[0][:, b]) < bound for b in range(3))
