@@ -100,9 +100,10 @@ def plane_shape(L, lz, esz):
 
 
 def plane_fits(L, lz, esz):
-    """Whether such a plane fits the shared memory a block can opt in to."""
+    """Whether such a plane fits the shared memory a block can opt in to (complex128: that of
+    two blocks on an SM)."""
     shape = plane_shape(L, lz, esz)
-    return shape is not None and shape[0] <= 227 * 1024
+    return shape is not None and shape[0] <= (227 if esz == 8 else 113) * 1024
 
 
 PLANE_RING_MAX = 64 << 30   # z-spectra of a factor-3 z length beyond this: separate passes

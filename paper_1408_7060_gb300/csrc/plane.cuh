@@ -66,9 +66,14 @@ struct PlaneCfg {
   static constexpr int TY = Y1 * (Y2 + 1), TZ = Z1 * (Z2 + 1);    // twiddle tables
   static constexpr int SCR = CW * PZ;                             // exchange elements per warp
   static constexpr size_t smem = ok ? ((size_t)(L == LZ ? TY : TY + TZ) + (size_t)(LZ / 2) * PY + (size_t)NW * SCR) * sizeof(C) : 0;
-  static constexpr bool fits = ok && smem <= (size_t)kPlaneSmemMax;
   // blocks per SM the register allocation aims at (shared memory allows as many)
   static constexpr int by_smem = ok ? (int)((size_t)(228 * 1024) / (smem + 1024)) : 1;
+  // A plane of complex128 has to leave room for a second one on its SM: alone, its load, FP64
+  // and store phases follow one another, and the separate passes are as fast or faster (one
+  // vector, us per product, plane against separate: 64^3 with 128 points in z 1319 and 1186,
+  // with 64 points 583 and 518, 96^3 with 64 points 1537 and 1293; four vectors 4557 and 4503,
+  // 1919 and 1856, 5220 and 4887; 16 vectors on 64^3 17.5 and 17.7 ms).
+  static constexpr bool fits = ok && smem <= (size_t)kPlaneSmemMax && (sizeof(C) == 8 || by_smem >= 2);
   static constexpr int threads = (Y1 == 16 || Z1 == 16) ? (sizeof(C) == 8 ? 512 : 256) : (sizeof(C) == 8 ? 1024 : 512);
   static constexpr int most = threads / (32 * NW) < 1 ? 1 : threads / (32 * NW);
   static constexpr int blocks = by_smem < 1 ? 1 : by_smem < most ? by_smem : most;

@@ -96,26 +96,29 @@ def plane_table(n, lz):
     return 2 * (n + 1) * 2 * n * lz * 16
 
 
-def test_no_slab_beside_the_plane_kernel():
+@pytest.mark.parametrize("grid,precision", [(64, "c64"), (32, "c128")])
+def test_no_slab_beside_the_plane_kernel(grid, precision):
     from paper_1408_7060_gb300 import AimContext
 
     V, F = icosphere(4, 1.0)
-    h, origin = place_grid(V, 64)
+    h, origin = place_grid(V, grid)
+    es = 8 if precision == "c64" else 16
 
     def held(**kw):
-        with AimContext(V=V, F=F, grid_n=64, origin=origin, h=h, near_radius=3 * h, dt=0.25 / (BAND * F_C), f_c=F_C,
+        kw = {"precision": precision, **kw}
+        with AimContext(V=V, F=F, grid_n=grid, origin=origin, h=h, near_radius=3 * h, dt=0.25 / (BAND * F_C), f_c=F_C,
                         **kw) as c:
-            assert c.info["z_len"] == 128
+            assert c.info["z_len"] == 2 * grid
             c.matvec(0, np.ones((1, c.ns), complex))
             assert c.get_profile()[0]["yfft_fwd"][0] == 0
-            nz = c.info["box_hi"][2] - c.info["box_lo"][2] + 1
-            ring = c.n_delays * 4 * 128 ** 3                   # elements per wave: ring, A, P
-            return c.info["device_bytes"], ring, 4 * nz * 64 * (128 + 64), 4 * nz * 128 ** 2
+            nz, L = c.info["box_hi"][2] - c.info["box_lo"][2] + 1, 2 * grid
+            # elements per wave: ring, A and P, slab
+            return c.info["device_bytes"], c.n_delays * 4 * L ** 3, 4 * nz * grid * (L + grid), 4 * nz * L ** 2, c.ns
 
-    # what 40 more waves take beyond their ring, A and P is less than their slab
-    (b1, ring, grid, slab), b41 = held(precision="c64"), held(precision="c64", batch_max=41)[0]
-    vectors = 40 * V.shape[0] * 3 * 16 * (51 + 60)             # Krylov basis, histories, work vectors
-    assert b41 - b1 < 40 * 8 * (ring + grid) + vectors + 40 * 8 * slab // 2
-    # and the refinement's buffers likewise (FP64, A and P of one wave)
-    more = held(precision="c64", refine=2)[0] - b1
-    assert more < 16 * grid + 16 * slab // 2 + plane_table(64, 128)
+    # what 100 more waves take beyond their ring, A, P and vectors is less than their slab
+    (b1, ring, work, slab, ns), more = held(), held(batch_max=101)[0]
+    vectors = 100 * ns * 16 * (51 + 40)                        # Krylov basis, histories, work vectors
+    assert more - b1 < 100 * (es * (ring + work) + es * slab // 2) + vectors
+    if grid == 32:                                             # and the refinement's FP64 buffers likewise
+        b1, more = held(precision="c64")[0], held(precision="c64", refine=2)[0]
+        assert more - b1 < 16 * work + 16 * slab // 2 + plane_table(grid, 2 * grid)

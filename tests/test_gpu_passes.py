@@ -38,9 +38,11 @@ def crandn(rng, *shape):
 
 # (mesh, size, grid, z length, precision, right-hand sides, separate passes)
 SIZES = [("sphere2", 0.12, 96, 32, "c64", 3, False), ("sphere2", 0.12, 96, 32, "c128", 2, False),
-         ("sphere2", 0.25, 96, 64, "c64", 3, False), ("sphere2", 0.25, 96, 64, "c128", 2, False),
-         ("sphere2", 0.09, 128, 32, "c64", 3, False), ("sphere2", 0.09, 128, 32, "c128", 2, False),
-         ("sphere2", 0.2, 128, 64, "c64", 3, False), ("sphere2", 0.2, 128, 64, "c128", 2, False),
+         ("sphere2", 0.25, 96, 64, "c64", 3, False), ("sphere2", 0.25, 96, 64, "c128", 2, True),
+         ("sphere2", 0.09, 128, 32, "c64", 3, False), ("sphere2", 0.09, 128, 32, "c128", 2, True),
+         ("sphere2", 0.2, 128, 64, "c64", 3, False), ("sphere2", 0.2, 128, 64, "c128", 2, True),
+         ("sphere2", 1.0, 64, 128, "c128", 2, True), ("sphere2", 0.4, 64, 64, "c128", 2, True),
+         ("sphere2", 0.15, 64, 32, "c128", 2, False), ("sphere2", 1.0, 32, 64, "c128", 2, False),
          ("sphere2", 0.5, 96, 128, "c128", 2, True), ("sphere2", 0.4, 128, 128, "c128", 2, True),
          ("sphere2", 0.53, 128, 144, "c128", 1, True), ("sphere2", 0.7, 128, 192, "c64", 3, True),
          ("sphere2", 1.0, 128, 256, "c64", 2, True), ("plate", 14, 384, 16, "c64", 2, True)]
