@@ -182,7 +182,8 @@ typedef struct {
   int64_t precond_nnz;   /* entries of the preconditioner's sparsity pattern          */
   int32_t refine;        /* aim_opts.refine as set up (0 on the complex128 path)       */
   int32_t refine_every;  /* aim_opts.refine_every as set up (>= 1)                       */
-  int32_t plan_zw, plan_cw, plan_rp, plan_ypb; /* launch shapes in use (see aim_opts.autotune) */
+  int32_t plan_zw, plan_cw, plan_rp, plan_ypb; /* launch shapes in use (see aim_opts.autotune);
+                                                  defaults where the kernels have no choice  */
   int32_t plan_source;   /* AIM_PLAN_*                                                  */
   int32_t box_lo[3], box_hi[3]; /* active box: grid nodes (x, y, z) touched by some stencil
                             lie in [box_lo, box_hi] (inclusive).  Sources vanish outside it

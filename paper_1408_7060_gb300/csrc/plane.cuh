@@ -21,8 +21,8 @@
 //   [group][k2 / 2][u][k2 & 1],
 // one coalesced 16-byte load per lane for every two values.
 //
-// What bounds it: shared-memory bandwidth in complex64 (about 11 400 wavefronts per 128 x 128
-// plane, 85 % of the cycles of the L1 pipe in use), FP64 arithmetic in complex128.  64 waves
+// What bounds it: shared-memory bandwidth in complex64 (about 10 700 wavefronts per 128 x 128
+// plane, 83 % of the cycles of the L1 pipe in use), FP64 arithmetic in complex128.  64 waves
 // on the 64^3 grid, complex64: y, z and inverse y passes 2380 us as three kernels, which
 // together moved 10.4 GB, 1580 us here, moving 2.1 GB.  A z step held in registers (two
 // lanes or two warps per column, 64 values each) crosses shared memory half as often but
