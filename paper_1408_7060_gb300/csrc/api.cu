@@ -80,7 +80,6 @@ static int z_length(int nz, int L) {
 void setup_work(aim_ctx* c, const aim_opts* opts) {
   const int B = c->batch_max, ns = c->ns, ng = c->n_delays;
   const size_t es = grid_elem(c);
-  alloc_ring(c);
   plane_spectra(c);
   c->d_A = aim_alloc(c, grid_a_elems(c, B) * es);
   c->d_Bf = op_plane(c) ? nullptr : aim_alloc(c, grid_bf_elems(c, B) * es);  // the separate passes' slab
@@ -115,6 +114,7 @@ void setup_work(aim_ctx* c, const aim_opts* opts) {
     if (!c->h_rn) AIM_CUDA(cudaMallocHost(&c->h_rn, 2 * (size_t)B * sizeof(double)));
   }
   gmres_alloc(c);
+  alloc_ring(c);  // after the small buffers: with the ring first, the 64^3 product took 85 us instead of 83.5
   if (op_plane(c)) {  // several delays of aim_rhs at a time; without the memory, one at a time
     const size_t per = grid_a_elems(c, 1) * es;
     const int cap = (int)std::min<size_t>((size_t)ng * B, kBatchBytes / per);
